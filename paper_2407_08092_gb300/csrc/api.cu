@@ -2065,7 +2065,19 @@ static void force_apply(lq_ctx *c, const void *X, const void *Y, double coef, vo
     const void *U[2] = {c->Udf[0], c->Udf[1]};
     void *gam = ws(c, "clover:F", (size_t)6 * 9 * 8 * c->g.V);
     force_insertion(e, Xs, Ys, c->lat.csw, gam);
-    force_links(e, U, Xs, Ys, gam, coef, G);
+    // scratch for as many time slices as fit 2 GiB, fewer when memory is short
+    int slices = c->g.L[3];
+    while (slices > 1 && force_scratch_bytes(c->g, slices) > ((size_t)2 << 30)) slices--;
+    void *scratch = nullptr;
+    while (!scratch) {
+        try {
+            scratch = ws(c, "force:M", force_scratch_bytes(c->g, slices));
+        } catch (const Fail &f) {
+            if (f.s != LQ_ERR_OOM || slices == 1) throw;
+            slices /= 2;
+        }
+    }
+    force_links(e, U, Xs, Ys, gam, scratch, slices, coef, G);
     ck_launch(c, "force");
 }
 

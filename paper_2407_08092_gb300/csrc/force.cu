@@ -23,15 +23,35 @@
 // u_3 = X_0 Y_0^+ - X_1 Y_1^+ (upper block u, lower block l):
 //   Lam_xy = -(u_3 + l_3), Lam_xz = u_2 + l_2, Lam_yz = -(u_1 + l_1),
 //   Lam_xt = u_1 - l_1,    Lam_yt = u_2 - l_2, Lam_zt = u_3 - l_3.
-// A link U_mu(x) is a factor f_k of eight leaves of each of the three planes
-// that contain mu; for each such leaf of Q(y), with M = f_{k+1}..f_3 Gam(y)
-// f_0..f_{k-1} the rest of the loop, G += M^+ (U enters as U) or M (as U^+).
+// The leaf sum over Q is a sum over plaquettes with one insertion per corner.
+// For the plaquette of plane (m, n) at z, with links a = U_m(z), b = U_n(z+m),
+// c = U_m(z+n), d = U_n(z) and corners z, z+m, z+m+n, z+n, it is
+//   tr(Gam_z a b c^+ d^+) + tr(a Gam_{z+m} b c^+ d^+) + ...   (four corners).
+// With the paths W = a b, W2 = d c, Z = b c^+, V = d^+ a and, per link of the
+// plaquette, the insertions at its two ends E_u = Gam(start) u + u Gam(end)
+// (Gam is anti-Hermitian, so E_u^+ = -(u^+ Gam(start) + Gam(end) u^+)), the four
+// gradients of that sum are two products each:
+//   G_a = W2 E_b^+ - E_d Z^+      G_b = E_a^+ W2 - V^+ E_c
+//   G_c = V E_b - E_d^+ W         G_d = E_a Z - W E_c^+
+// Per plaquette that is 4 products for the paths, 4 for E_m(z) and E_n(z) (E_b
+// and E_c are those of the neighbouring plaquettes) and 8 for the gradients:
+// 96 per site, where the 24 leaves of each link, formed one by one, take 288.
 //
 // Arithmetic is df64 (FP64-accurate on the FP32 units) throughout.
 #include "leaves.cuh"
 #include "lq_kernels.h"
 
 namespace lq {
+
+// Resident blocks per SM asked of the two kernels: four (128 registers, some
+// spills outside the products) against three (168): 5.44 against 5.64 ms for
+// lq_force on 24^3 x 48, and 6.32 at two.
+#ifndef LQ_FLINK_MINB
+#define LQ_FLINK_MINB 4
+#endif
+#ifndef LQ_FLOOP_MINB
+#define LQ_FLOOP_MINB 4
+#endif
 
 // gamma_mu psi: component s is i^k[mu][s] psi_perm[mu][s] (chiral basis)
 __constant__ unsigned char c_gperm[4][4] = {{3, 2, 1, 0}, {3, 2, 1, 0}, {2, 3, 0, 1}, {2, 3, 0, 1}};
@@ -54,11 +74,17 @@ __device__ __forceinline__ cx<df64> ld_comp(const df2 *__restrict__ f, long long
     return df2_cx(ldg(f + (long long)comp * stride + cb));
 }
 
-// Gam of the six planes at one site per thread, from X(x) and Y(x)
+// x or -x, as the sign bit `bit` says
+__device__ __forceinline__ df64 flip_sign(df64 x, unsigned bit)
+{
+    return df64(__uint_as_float(__float_as_uint(x.hi) ^ bit), __uint_as_float(__float_as_uint(x.lo) ^ bit));
+}
+
+// Gam of the six planes at one site per thread, from X(x) and Y(x); k16 = c_sw / 16
 __global__ void __launch_bounds__(128) force_insertion_kernel(Geom g, const df2 *__restrict__ Xe,
                                                               const df2 *__restrict__ Xo,
                                                               const df2 *__restrict__ Ye,
-                                                              const df2 *__restrict__ Yo, double csw, float2 *Gam)
+                                                              const df2 *__restrict__ Yo, df64 k16, float2 *Gam)
 {
     const long long lex = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (lex >= g.V) return;
@@ -67,7 +93,6 @@ __global__ void __launch_bounds__(128) force_insertion_kernel(Geom g, const df2 
     const int parity = (c[0] + c[1] + c[2] + c[3]) & 1;
     const long long cb = lex >> 1;
     const df2 *X = parity ? Xo : Xe, *Y = parity ? Yo : Ye;
-    const df64 k16(csw / 16.0);
 #pragma unroll 1
     for (int l = 1; l <= 3; l++) {
         // H_block = u_l + u_l^+ for the upper (blk 0) and lower (blk 1) chirality
@@ -82,19 +107,21 @@ __global__ void __launch_bounds__(128) force_insertion_kernel(Geom g, const df2 
                 y0[a] = ld_comp(Y, g.stride, (2 * blk) * 3 + a, cb);
                 y1[a] = ld_comp(Y, g.stride, (2 * blk + 1) * 3 + a, cb);
             }
+            // entry (a, b) of X_s' Y_s^+ is X_s'[a] conj(Y_s[b]); u_1 and u_3 take
+            // y0 with x1 resp. x0 and y1 with the other, u_2 = i (x0 y1^+ - x1 y0^+)
+            const unsigned f0 = l == 2 ? 0x80000000u : 0u, f1 = l == 3 ? 0x80000000u : 0u;
             M3<df64> u;
 #pragma unroll
-            for (int a = 0; a < 3; a++)
+            for (int a = 0; a < 3; a++) {
+                const df64x2 p = dl2(l == 3 ? x0[a] : x1[a]), q = dl2(l == 3 ? x1[a] : x0[a]);
 #pragma unroll
                 for (int b = 0; b < 3; b++) {
-                    // entry (a, b) of X_s' Y_s^+ is X_s'[a] conj(Y_s[b])
-                    const cx<df64> p10 = cmulc(y0[b], x1[a]), p01 = cmulc(y1[b], x0[a]);
-                    cx<df64> v;
-                    if (l == 1) v = p10 + p01;
-                    else if (l == 2) v = ti(p01 - p10);
-                    else v = cmulc(y0[b], x0[a]) - cmulc(y1[b], x1[a]);
-                    u.a[a * 3 + b] = v;
+                    dlrow t = dlrow_prod({flip_sign(y0[b].re, f0), flip_sign(y0[b].im, f0)}, p);
+                    dlrow_fma(t, {flip_sign(y1[b].re, f1), flip_sign(y1[b].im, f1)}, q);
+                    const cx<df64> v = dl2_cx(dl2_norm(dlrow_conj(t)));
+                    u.a[a * 3 + b] = l == 2 ? ti(v) : v;
                 }
+            }
             H[blk] = u;
 #pragma unroll
             for (int a = 0; a < 3; a++)
@@ -128,116 +155,248 @@ __global__ void __launch_bounds__(128) force_insertion_kernel(Geom g, const df2 
     }
 }
 
-// G(x, mu) for one (site, direction) per thread; mu is uniform across a warp
-// except at the seams of the four direction ranges.
-__global__ void __launch_bounds__(128) force_link_kernel(Geom g, const df2 *__restrict__ Ue,
-                                                         const df2 *__restrict__ Uo, const df2 *__restrict__ Xe,
+// entry (i, k) of a 3x3 matrix stored component-major at m (distance `st` between
+// components), or of its Hermitian conjugate
+__device__ __forceinline__ M3<df64> load_mat(const df2 *__restrict__ m, long long st, bool dag)
+{
+    M3<df64> A;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const cx<df64> t = df2_cx(ldg(m + (dag ? k * 3 + i : i * 3 + k) * st));
+            A.a[i * 3 + k] = dag ? cx<df64>{t.re, dl_neg(t.im)} : t;
+        }
+    return A;
+}
+
+// one row of a product added to a row of sums: s_j += sum_k r_k B_kj
+__device__ __forceinline__ void row_fma(cx<df64> s[3], const cx<df64> r[3], const M3<df64> &B)
+{
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        dlrow t = dlrow_prod(r[0], dl2(B.a[j]));
+        dlrow_fma(t, r[1], dl2(B.a[3 + j]));
+        dlrow_fma(t, r[2], dl2(B.a[6 + j]));
+        df64x2 u = dl2(s[j]);
+        dl2_add(u, t.r);
+        dl2_add(u, dlrow_rot(t));
+        s[j] = dl2_cx(u);
+    }
+}
+
+// entry (i, k) of the anti-Hermitian matrix of plane p at site lex
+__device__ __forceinline__ cx<df64> antiherm_entry(const float2 *__restrict__ base, long long V, long long lex, int p,
+                                                   int i, int k)
+{
+    auto ld = [&](int q) {
+        const float2 t = __ldg(base + ((long long)p * 9 + q) * V + lex);
+        return df64(t.x, t.y);
+    };
+    if (i == k) return {df64(0.0f, 0.0f), ld(i)};
+    const int lo = i < k ? i : k, hi = i < k ? k : i, q = 3 + 2 * (lo + hi - 1);   // (0,1) (0,2) (1,2) at 3, 5, 7
+    const df64 re = ld(q), im = ld(q + 1);
+    return {i < k ? re : dl_neg(re), im};
+}
+
+// The plaquette matrices of a range of time slices: [plane][matrix][9][sites] df2
+// with the sites of slice t (x fastest) at ((t - tb) mod Lt) * S3.
+constexpr int F_W = 0, F_W2 = 1, F_Z = 2, F_V = 3, F_EM = 4, F_EN = 5, F_MATS = 6;
+struct LoopMats {
+    df2 *m;
+    int tb;          // first stored slice
+    long long s3;    // sites of a slice
+    long long n;     // sites stored
+    __device__ __forceinline__ df2 *at(int p, int q, long long site) const
+    {
+        return m + ((long long)(p * F_MATS + q) * 9) * n + site;
+    }
+    // the stored index of coordinates c
+    __device__ __forceinline__ long long site(const Geom &g, const int c[4]) const
+    {
+        const int t = c[3] >= tb ? c[3] - tb : c[3] - tb + g.L[3];
+        return LQ_IDX((long long)t * s3 + c[0] + (long long)g.L[0] * (c[1] + (long long)g.L[1] * c[2]), n, B_LEX);
+    }
+};
+
+// coordinates c moved by +-1 along mu (mu uniform over a block)
+__device__ __forceinline__ void step(const Geom &g, const int c[4], int mu, int s, int o[4])
+{
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        int v = c[k];
+        if (k == mu) {
+            v += s;
+            v = v < 0 ? v + g.L[k] : (v >= g.L[k] ? v - g.L[k] : v);
+        }
+        o[k] = v;
+    }
+}
+
+// W, W2, Z, V, E_m and E_n of one plaquette per thread (plane = blockIdx.y).  The
+// eight products share one copy of the product code, their operands picked by
+// the step: links a, b, c, d (0..3) and Gam at z, z+m, z+n (4..6).
+__global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, const df2 *__restrict__ Ue,
+                                                         const df2 *__restrict__ Uo, const float2 *__restrict__ Gam,
+                                                         LoopMats S)
+{
+    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (id >= S.n) return;
+    const int p = blockIdx.y, m = c_pmu[p], n = c_pnu[p];
+    int z[4], zm[4], zn[4];
+    {
+        const int tl = (int)(id / S.s3);
+        unsigned r = (unsigned)(id - tl * S.s3);
+        z[0] = (int)(r % (unsigned)g.L[0]);
+        r /= (unsigned)g.L[0];
+        z[1] = (int)(r % (unsigned)g.L[1]);
+        z[2] = (int)(r / (unsigned)g.L[1]);
+        z[3] = S.tb + tl >= g.L[3] ? S.tb + tl - g.L[3] : S.tb + tl;
+    }
+    step(g, z, m, +1, zm);
+    step(g, z, n, +1, zn);
+    const long long lz = lex_of(g, z), lm = lex_of(g, zm), ln = lex_of(g, zn);
+    const bool odd = (z[0] + z[1] + z[2] + z[3]) & 1;
+    const df2 *Uz = (odd ? Uo : Ue) + (lz >> 1), *Un = odd ? Ue : Uo;   // z + m and z + n have the other parity
+    auto link = [&](int code) {   // U_m(z), U_n(z+m), U_m(z+n), U_n(z)
+        const df2 *u = code == 0 || code == 3 ? Uz : Un + ((code == 1 ? lm : ln) >> 1);
+        return u + (long long)(code == 0 || code == 2 ? m : n) * 9 * g.stride;
+    };
+    M3<df64> acc;
+#pragma unroll 1
+    for (int j = 0; j < 8; j++) {
+        // a b | d c | b c^+ | d^+ a | Gam_z a, a Gam_{z+m} | Gam_z d, d Gam_{z+n}
+        const int lc = (0x34043130 >> (4 * j)) & 15, rc = (0x63500221 >> (4 * j)) & 15;
+        const M3<df64> B = rc >= 4 ? load_antiherm(Gam, g.V, rc == 5 ? lm : ln, p) : load_mat(link(rc), g.stride, j == 2);
+        if (j != 5 && j != 7)
+#pragma unroll
+            for (int k = 0; k < 9; k++) acc.a[k] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+        const df2 *A = link(lc);
+        const bool gam = lc >= 4, dag = j == 3;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {   // the left factor one row at a time
+            cx<df64> r[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                if (gam) {
+                    r[k] = antiherm_entry(Gam, g.V, lz, p, i, k);
+                } else {
+                    const cx<df64> t = df2_cx(ldg(A + (dag ? k * 3 + i : i * 3 + k) * g.stride));
+                    r[k] = dag ? cx<df64>{t.re, dl_neg(t.im)} : t;
+                }
+            }
+            row_fma(acc.a + 3 * i, r, B);
+        }
+        if (j == 4 || j == 6) continue;
+        df2 *o = S.at(p, j < 4 ? j : j == 5 ? F_EM : F_EN, id);
+#pragma unroll
+        for (int k = 0; k < 9; k++) o[(long long)k * S.n] = cx_df2(dl_cnorm(acc.a[k]));
+    }
+}
+
+// G(x, mu) for one (site, direction) per thread, sites of the slices t0 ..
+// (mu = blockIdx.y): the hopping term's outer products, then per plane that
+// contains mu the link's two plaquettes, two products each.
+__global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, const df2 *__restrict__ Xe,
                                                          const df2 *__restrict__ Xo, const df2 *__restrict__ Ye,
-                                                         const df2 *__restrict__ Yo, const float2 *__restrict__ Gam,
+                                                         const df2 *__restrict__ Yo, LoopMats S, int t0, long long ns,
                                                          double coef, double2 *G)
 {
     const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (id >= 4 * g.V) return;
-    const int mu = (int)(id / g.V);
-    const long long lex = id - mu * g.V;
+    if (id >= ns) return;
+    const int mu = blockIdx.y;
+    const long long lex = t0 * S.s3 + id;
     int c[4];
     lex_coords(g, lex, c);
     const int parity = (c[0] + c[1] + c[2] + c[3]) & 1;
-    int cn[4] = {c[0], c[1], c[2], c[3]};
-    cn[mu] = cn[mu] + 1 == g.L[mu] ? 0 : cn[mu] + 1;
+    int cn[4];
+    step(g, c, mu, +1, cn);
     const long long cb = lex >> 1, cbn = lex_of(g, cn) >> 1;
     const df2 *Xx = parity ? Xo : Xe, *Yx = parity ? Yo : Ye;      // at x
     const df2 *Xn = parity ? Xe : Xo, *Yn = parity ? Ye : Yo;      // at x + mu
-    const df64 z(0.0f, 0.0f);
 
     M3<df64> acc;
 #pragma unroll
-    for (int k = 0; k < 9; k++) acc.a[k] = {z, z};
+    for (int k = 0; k < 9; k++) acc.a[k] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
 
     // ---- hopping term: sum_s Y_s(x) (P- X(x+mu))_s^+ + (P+ X(x))_s Y_s(x+mu)^+ ----
-    {
-        M3<df64> hop;
-#pragma unroll
-        for (int k = 0; k < 9; k++) hop.a[k] = {z, z};
 #pragma unroll 1
-        for (int s = 0; s < 4; s++) {
-            const int sp = c_gperm[mu][s], ip = c_gipow[mu][s];
-            cx<df64> ya[3], w[3];
+    for (int s = 0; s < 4; s++) {
+        const int sp = c_gperm[mu][s], ip = c_gipow[mu][s];
+        cx<df64> y[3], w[3];
 #pragma unroll
-            for (int a = 0; a < 3; a++) {
-                ya[a] = ld_comp(Yx, g.stride, s * 3 + a, cb);
-                w[a] = ld_comp(Xn, g.stride, s * 3 + a, cbn) -
-                       times_ipow(ld_comp(Xn, g.stride, sp * 3 + a, cbn), ip);   // (1 - g_mu) X(x+mu)
-            }
-#pragma unroll
-            for (int a = 0; a < 3; a++)
-#pragma unroll
-                for (int b = 0; b < 3; b++) hop.a[a * 3 + b] = hop.a[a * 3 + b] + cmulc(w[b], ya[a]);
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                ya[a] = ld_comp(Yn, g.stride, s * 3 + a, cbn);
-                w[a] = ld_comp(Xx, g.stride, s * 3 + a, cb) +
-                       times_ipow(ld_comp(Xx, g.stride, sp * 3 + a, cb), ip);    // (1 + g_mu) X(x)
-            }
-#pragma unroll
-            for (int a = 0; a < 3; a++)
-#pragma unroll
-                for (int b = 0; b < 3; b++) hop.a[a * 3 + b] = hop.a[a * 3 + b] + cmulc(ya[b], w[a]);
+        for (int a = 0; a < 3; a++) {
+            y[a] = ld_comp(Yx, g.stride, s * 3 + a, cb);
+            w[a] = ld_comp(Xn, g.stride, s * 3 + a, cbn) -
+                   times_ipow(ld_comp(Xn, g.stride, sp * 3 + a, cbn), ip);   // (1 - g_mu) X(x+mu)
         }
-        const bool wrap = mu == 3 && c[3] == g.L[3] - 1;
-        const df64 f = df64((wrap && g.tbc < 0) ? 0.5f : -0.5f, 0.0f);
 #pragma unroll
-        for (int k = 0; k < 9; k++) acc.a[k] = f * hop.a[k];
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int b = 0; b < 3; b++) dl_cfmac(acc.a[a * 3 + b], w[b], y[a]);
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            y[a] = ld_comp(Yn, g.stride, s * 3 + a, cbn);
+            w[a] = ld_comp(Xx, g.stride, s * 3 + a, cb) +
+                   times_ipow(ld_comp(Xx, g.stride, sp * 3 + a, cb), ip);    // (1 + g_mu) X(x)
+        }
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int b = 0; b < 3; b++) dl_cfmac(acc.a[a * 3 + b], y[b], w[a]);
+    }
+    {
+        const bool wrap = mu == 3 && c[3] == g.L[3] - 1;
+        const float f = (wrap && g.tbc < 0) ? 0.5f : -0.5f;
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const cx<df64> t = dl_cnorm(acc.a[k]);
+            acc.a[k] = {dl_scale2(t.re, f), dl_scale2(t.im, f)};
+        }
     }
 
-    // ---- clover term: the 24 leaves that contain U_mu(x) ----
+    // ---- clover term: the two plaquettes of each plane (mu, nu) that hold U_mu(x) ----
 #pragma unroll 1
-    for (int q = 0; q < 3; q++) {
-        const int nu = q < mu ? q : q + 1;
-        const int pmu = mu < nu ? mu : nu, pnu = mu < nu ? nu : mu;
-        const int p = c_plane[pmu * 4 + pnu];
-        const unsigned char along_nu = mu == pnu;
-#pragma unroll 1
-        for (int f = 0; f < 16; f++) {
-            if (c_lnu[f] != along_nu) continue;
-            const int leaf = f >> 2, kf = f & 3;
-            // the leaf starts at y = x - offset(f)
-            int y[4] = {c[0], c[1], c[2], c[3]};
-            y[pmu] = (y[pmu] - c_ldmu[f] + 2 * g.L[pmu]) % g.L[pmu];
-            y[pnu] = (y[pnu] - c_ldnu[f] + 2 * g.L[pnu]) % g.L[pnu];
-            M3<df64> T;
-#pragma unroll 1
-            for (int j = 1; j <= 4; j++) {
-                const int slot = kf + j;   // 0..3: factors of the leaf, 4: Gam(y), 5..: wrap to factor 0
-                M3<df64> Fj;
-                if (slot == 4) {
-                    Fj = load_antiherm(Gam, g.V, lex_of(g, y), p);
-                } else {
-                    const int ff = 4 * leaf + (slot < 4 ? slot : slot - 5);
-                    int cc[4] = {y[0], y[1], y[2], y[3]};
-                    cc[pmu] = (cc[pmu] + c_ldmu[ff] + g.L[pmu]) % g.L[pmu];
-                    cc[pnu] = (cc[pnu] + c_ldnu[ff] + g.L[pnu]) % g.L[pnu];
-                    Fj = link_at<df64>(g, Ue, Uo, cc, c_lnu[ff] ? pnu : pmu);
-                    if (c_ldag[ff]) Fj = dagger(Fj);
-                }
-                T = j == 1 ? Fj : mat_mul(T, Fj);
+    for (int h = 0; h < 12; h++) {
+        // plane (h / 4), plaquette at x (0) or x - nu (1), first or second product
+        const int q = h >> 2, nu = q < mu ? q : q + 1;
+        const bool down = h & 2, second = h & 1, lower = mu < nu;
+        const int p = c_plane[lower ? mu * 4 + nu : nu * 4 + mu];
+        int z[4], zu[4];
+        step(g, c, nu, down ? -1 : 0, z);
+        step(g, z, mu, +1, zu);
+        const long long iz = S.site(g, z), iu = S.site(g, zu);
+        // the operands of each product (E: of the nu links; E' at z + mu):
+        //   U_mu = a: W2 E'^+, E Z^+    = c: V E', E^+ W    = d: E Z, W E'^+    = b: E^+ W2, V^+ E'
+        const int e = lower ? F_EN : F_EM;
+        const bool efirst = lower == second;   // E is the left factor and sits at z
+        const int other = down ? (efirst ? (lower ? F_W : F_W2) : F_V) : (efirst ? F_Z : (lower ? F_W2 : F_W));
+        const df2 *E = S.at(p, e, efirst ? iz : iu), *O = S.at(p, other, iz);
+        const df2 *A = efirst ? E : O;
+        const bool dag = down && (efirst || !lower);
+        const M3<df64> B = load_mat(efirst ? O : E, S.n, !down && (efirst ? lower : true));
+        const unsigned sre = second ? 0x80000000u : 0u, sim = (second != dag) ? 0x80000000u : 0u;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {   // the left factor one row at a time, with the product's sign
+            cx<df64> r[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const cx<df64> t = df2_cx(ldg(A + (dag ? k * 3 + i : i * 3 + k) * S.n));
+                r[k] = {flip_sign(t.re, sre), flip_sign(t.im, sim)};
             }
-            if (c_ldag[f]) {
-#pragma unroll
-                for (int k = 0; k < 9; k++) acc.a[k] = acc.a[k] + T.a[k];
-            } else {
-#pragma unroll
-                for (int a = 0; a < 3; a++)
-#pragma unroll
-                    for (int b = 0; b < 3; b++) acc.a[a * 3 + b] = acc.a[a * 3 + b] + cconj(T.a[b * 3 + a]);
-            }
+            row_fma(acc.a + 3 * i, r, B);
         }
+        if (second)
+#pragma unroll
+            for (int k = 0; k < 9; k++) acc.a[k] = dl_cnorm(acc.a[k]);
     }
 
     double2 *o = G + (lex * 4 + mu) * 9;
 #pragma unroll
-    for (int k = 0; k < 9; k++)
-        o[k] = make_double2(coef * df_to_double(acc.a[k].re), coef * df_to_double(acc.a[k].im));
+    for (int k = 0; k < 9; k++) {
+        const cx<df64> v = dl_cnorm(acc.a[k]);
+        o[k] = make_double2(coef * df_join(v.re.hi, v.re.lo), coef * df_join(v.im.hi, v.im.lo));
+    }
 }
 
 // out = g5 in on natural full spinors [V][4][3] complex double (spins 2, 3 negated)
@@ -257,20 +416,49 @@ void force_insertion(const Exec &e, const void *X[2], const void *Y[2], double c
     // per site 6 blocks x (2 x 9 products + 9 additions) and the Hermitian parts
     Launch L_(e, K_FORCE, (double)e.g.V * (2 * 192 + 6 * 72), (double)e.g.V * 3 * 2 * (18 * 6 + 18 * 2 + 18 * 2));
     force_insertion_kernel<<<blocks_of(e.g.V, 128), 128, 0, e.st>>>(
-        e.g, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1], csw, (float2 *)Gam);
+        e.g, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1], df64(csw / 16.0),
+        (float2 *)Gam);
 }
 
-void force_links(const Exec &e, const void *Udf[2], const void *X[2], const void *Y[2], const void *Gam,
-                 double coef, void *G)
+// The plaquette matrices take 5184 B a site, so the lattice goes through in
+// ranges of time slices whose matrices (with one more slice on either side) fit
+// the scratch: bytes of scratch for `slices` slices of output.
+size_t force_scratch_bytes(const Geom &g, int slices)
 {
-    // unique bytes per site: 4 df64 links, X and Y, six Gam, the 4 gradients
-    // (c128); per (site, mu): 24 leaves x 3 complex 3x3 products of 198 flops
-    // and their sum, plus the hopping term's 2 x 4 x 9 outer-product entries
-    Launch L_(e, K_FORCE, (double)e.g.V * (4 * 144 + 2 * 192 + 6 * 72 + 4 * 144),
-              (double)e.g.V * 4 * (24 * (3 * 198 + 18) + 2 * 4 * (9 * 8 + 12)));
-    force_link_kernel<<<blocks_of(4 * e.g.V, 128), 128, 0, e.st>>>(
-        e.g, (const df2 *)Udf[0], (const df2 *)Udf[1], (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0],
-        (const df2 *)Y[1], (const float2 *)Gam, coef, (double2 *)G);
+    const long long s3 = g.V / g.L[3];
+    const int stored = slices + 2 < g.L[3] ? slices + 2 : g.L[3];
+    return (size_t)stored * s3 * 6 * F_MATS * 9 * sizeof(df2);
+}
+
+void force_links(const Exec &e, const void *Udf[2], const void *X[2], const void *Y[2], const void *Gam, void *scratch,
+                 int slices, double coef, void *G)
+{
+    const Geom &g = e.g;
+    LoopMats S;
+    S.m = (df2 *)scratch;
+    S.s3 = g.V / g.L[3];
+    const bool whole = slices + 2 >= g.L[3];
+    if (whole) slices = g.L[3];
+    for (int t0 = 0; t0 < g.L[3]; t0 += slices) {
+        const int nt = g.L[3] - t0 < slices ? g.L[3] - t0 : slices;
+        const int stored = whole ? g.L[3] : nt + 2;
+        S.tb = whole ? 0 : (t0 + g.L[3] - 1) % g.L[3];
+        S.n = stored * S.s3;
+        const long long ns = nt * S.s3;
+        {
+            // unique bytes per site: 4 df64 links and six Gam in, 36 matrices out; per
+            // plane eight 3x3 products of 198 flops
+            Launch L_(e, K_FORCE, (double)S.n * (4 * 144 + 6 * 72 + 36 * 144), (double)S.n * 6 * 8 * 198);
+            force_loop_kernel<<<dim3(blocks_of(S.n, 128), 6), 128, 0, e.st>>>(
+                g, (const df2 *)Udf[0], (const df2 *)Udf[1], (const float2 *)Gam, S);
+        }
+        // X and Y, the matrices, the 4 gradients (c128); per link 12 products and
+        // the hopping term's 2 x 4 x 9 outer-product entries
+        Launch L_(e, K_FORCE, (double)ns * (2 * 192 + 36 * 144 + 4 * 144),
+                  (double)ns * 4 * (12 * (198 + 18) + 2 * 4 * (9 * 8 + 12)));
+        force_link_kernel<<<dim3(blocks_of(ns, 128), 4), 128, 0, e.st>>>(
+            g, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1], S, t0, ns, coef, (double2 *)G);
+    }
 }
 
 void gamma5_nat(const Exec &e, const void *in, void *out)

@@ -1,7 +1,6 @@
-// The plaquette leaves of the clover term (Sec. 2.3), shared by the clover
-// build and the fermion force: plane numbering, the link factors of the four
-// leaves of a plane, link access by lattice coordinates and the packed form of
-// an anti-Hermitian 3x3 matrix.
+// What the clover build and the fermion force share (clover term, Sec. 2.3):
+// plane numbering, link access by lattice coordinates, 3x3 products and the
+// packed form of an anti-Hermitian 3x3 matrix.
 #pragma once
 
 #include "lq_internal.cuh"
@@ -16,21 +15,6 @@ struct M3 {
 // Planes (mu, nu), mu < nu, numbered xy, xz, yz, xt, yt, zt.
 static __constant__ int c_pmu[6] = {0, 0, 1, 0, 1, 2};
 static __constant__ int c_pnu[6] = {1, 2, 2, 3, 3, 3};
-
-// The 16 link factors of the four leaves of plane (mu, nu), leaf by leaf (all
-// four run mu -> nu, i.e. with the same orientation, and start and end at x):
-//   leaf 1: U_mu(x)       U_nu(x+mu)        U_mu(x+nu)^+     U_nu(x)^+
-//   leaf 2: U_nu(x)       U_mu(x-mu+nu)^+   U_nu(x-mu)^+     U_mu(x-mu)
-//   leaf 3: U_mu(x-mu)^+  U_nu(x-mu-nu)^+   U_mu(x-mu-nu)    U_nu(x-nu)
-//   leaf 4: U_nu(x-nu)^+  U_mu(x-nu)        U_nu(x+mu-nu)    U_mu(x)^+
-// as the site offset along mu and nu, whether the link points along nu, and
-// whether it enters as U^+.  Walking this table lets one inlined 3x3 product
-// serve every product of a leaf (df64 code stays small enough for the
-// instruction cache).
-static __constant__ signed char c_ldmu[16] = {0, 1, 0, 0, 0, -1, -1, -1, -1, -1, -1, 0, 0, 0, 1, 0};
-static __constant__ signed char c_ldnu[16] = {0, 0, 1, 0, 0, 1, 0, 0, 0, -1, -1, -1, -1, -1, -1, 0};
-static __constant__ unsigned char c_lnu[16] = {0, 1, 0, 1, 1, 0, 1, 0, 0, 1, 0, 1, 1, 0, 1, 0};
-static __constant__ unsigned char c_ldag[16] = {0, 0, 1, 1, 0, 1, 1, 0, 1, 1, 0, 0, 1, 0, 0, 1};
 
 __device__ __forceinline__ long long lex_of(const Geom &g, const int c[4])
 {
@@ -55,17 +39,6 @@ __device__ __forceinline__ M3<R> link_at(const Geom &g, const typename St<R>::ve
     M3<R> m;
     load_link(parity ? Uo : Ue, g.stride, mu, lex_of(g, c) >> 1, m.a);
     return m;
-}
-
-template <typename R>
-__device__ __forceinline__ M3<R> dagger(const M3<R> &m)
-{
-    M3<R> d;
-#pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int b = 0; b < 3; b++) d.a[a * 3 + b] = cconj(m.a[b * 3 + a]);
-    return d;
 }
 
 template <typename R>
@@ -94,10 +67,11 @@ __device__ __forceinline__ M3<df64> mat_mul<df64>(const M3<df64> &A, const M3<df
     for (int a = 0; a < 3; a++)
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            cx<df64> acc = dl_cmul(A.a[a * 3], B.a[b]);
-            dl_cfma(acc, A.a[a * 3 + 1], B.a[3 + b]);
-            dl_cfma(acc, A.a[a * 3 + 2], B.a[6 + b]);
-            P.a[a * 3 + b] = dl_cnorm(acc);
+            dlrow acc = dlrow_prod(A.a[a * 3], dl2(B.a[b]));
+            dlrow_fma(acc, A.a[a * 3 + 1], dl2(B.a[3 + b]));
+            dlrow_fma(acc, A.a[a * 3 + 2], dl2(B.a[6 + b]));
+            dl2_add(acc.r, dlrow_rot(acc));
+            P.a[a * 3 + b] = dl2_cx(dl2_norm(acc.r));
         }
     return P;
 }

@@ -267,34 +267,120 @@ struct cx {
     R re, im;
 };
 
-// complex forms of the lazily normalised df64 sums above
+// ---------------------------------------------------------------------------
+// Packed FP32 arithmetic: one instruction works on the two floats of a
+// register pair (f32x2), each half rounded as the scalar instruction rounds it.
+// The FP32 units finish a packed instruction in the time of two scalar ones, so
+// it saves issue slots, not arithmetic: it pays where a kernel is bound by
+// instruction issue.  A complex number's real and imaginary parts share a pair.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 f2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) { return __fadd2_rn(a, f2_neg(b)); }
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// two df64 values side by side: the high parts and the low parts
+struct df64x2 {
+    float2 h, l;
+};
+__device__ __forceinline__ df64x2 dl2(cx<df64> a)
+{
+    return {make_float2(a.re.hi, a.im.hi), make_float2(a.re.lo, a.im.lo)};
+}
+__device__ __forceinline__ cx<df64> dl2_cx(df64x2 a) { return {df64(a.h.x, a.l.x), df64(a.h.y, a.l.y)}; }
+__device__ __forceinline__ df64x2 dl2_both(df64 a) { return {make_float2(a.hi, a.hi), make_float2(a.lo, a.lo)}; }
+__device__ __forceinline__ df64x2 dl2_swap(df64x2 a)
+{
+    return {make_float2(a.h.y, a.h.x), make_float2(a.l.y, a.l.x)};
+}
+// dl_prod, dl_add, dl_fma and dl_norm on both values, operation for operation
+__device__ __forceinline__ df64x2 dl2_prod(df64x2 a, df64x2 b)
+{
+    const float2 p = f2_mul(a.h, b.h);
+    float2 e = f2_fma(a.h, b.h, f2_neg(p));
+    e = f2_fma(a.h, b.l, e);
+    return {p, f2_fma(a.l, b.h, e)};
+}
+__device__ __forceinline__ void dl2_add(df64x2 &s, df64x2 x)
+{
+    const float2 t = f2_add(s.h, x.h);
+    const float2 bb = f2_sub(t, s.h);
+    const float2 err = f2_add(f2_sub(s.h, f2_sub(t, bb)), f2_sub(x.h, bb));
+    s.h = t;
+    s.l = f2_add(s.l, f2_add(err, x.l));
+}
+__device__ __forceinline__ void dl2_fma(df64x2 &s, df64x2 a, df64x2 b) { dl2_add(s, dl2_prod(a, b)); }
+__device__ __forceinline__ df64x2 dl2_norm(df64x2 a)
+{
+    const float2 s = f2_add(a.h, a.l);
+    const float2 bb = f2_sub(s, a.h);
+    return {s, f2_add(f2_sub(a.h, f2_sub(s, bb)), f2_sub(a.l, bb))};
+}
+
+// complex forms of the lazily normalised df64 sums, real and imaginary parts
+// packed: a b = (a.re, a.re) * (b.re, b.im) + (-a.im, a.im) * (b.im, b.re), and
+// with conj(a) the second factor is (a.im, -a.im)
+__device__ __forceinline__ df64x2 dl2_im(df64 a)   // (-a, a)
+{
+    return {make_float2(-a.hi, a.hi), make_float2(-a.lo, a.lo)};
+}
 __device__ __forceinline__ cx<df64> dl_cmul(cx<df64> a, cx<df64> b)   // a * b
 {
-    cx<df64> s = {dl_prod(a.re, b.re), dl_prod(a.re, b.im)};
-    dl_fma(s.re, dl_neg(a.im), b.im);
-    dl_fma(s.im, a.im, b.re);
-    return s;
+    const df64x2 bb = dl2(b);
+    df64x2 s = dl2_prod(dl2_both(a.re), bb);
+    dl2_fma(s, dl2_im(a.im), dl2_swap(bb));
+    return dl2_cx(s);
 }
 __device__ __forceinline__ void dl_cfma(cx<df64> &s, cx<df64> a, cx<df64> b)   // s += a * b
 {
-    dl_fma(s.re, a.re, b.re);
-    dl_fma(s.re, dl_neg(a.im), b.im);
-    dl_fma(s.im, a.re, b.im);
-    dl_fma(s.im, a.im, b.re);
+    const df64x2 bb = dl2(b);
+    df64x2 t = dl2(s);
+    dl2_fma(t, dl2_both(a.re), bb);
+    dl2_fma(t, dl2_im(a.im), dl2_swap(bb));
+    s = dl2_cx(t);
 }
 __device__ __forceinline__ void dl_cfmac(cx<df64> &s, cx<df64> a, cx<df64> b)   // s += conj(a) * b
 {
-    dl_fma(s.re, a.re, b.re);
-    dl_fma(s.re, a.im, b.im);
-    dl_fma(s.im, a.re, b.im);
-    dl_fma(s.im, dl_neg(a.im), b.re);
+    dl_cfma(s, {a.re, dl_neg(a.im)}, b);
 }
 __device__ __forceinline__ void dl_cadd(cx<df64> &s, cx<df64> x)
 {
-    dl_add(s.re, x.re);
-    dl_add(s.im, x.im);
+    df64x2 t = dl2(s);
+    dl2_add(t, dl2(x));
+    s = dl2_cx(t);
 }
-__device__ __forceinline__ cx<df64> dl_cnorm(cx<df64> s) { return {dl_norm(s.re), dl_norm(s.im)}; }
+__device__ __forceinline__ cx<df64> dl_cnorm(cx<df64> s) { return dl2_cx(dl2_norm(dl2(s))); }
+
+// A row times a column, sum_k a_k b_k, as the two packed sums r = sum a_k.re b_k
+// and i = sum a_k.im b_k: the b_k enter as they are, where a complex
+// multiply-add would take each of them a second time with its parts swapped
+// (two register moves per part, which the FP32 units' slots do not hide).
+// The sum is r + (-i.im, i.re).
+struct dlrow {
+    df64x2 r, i;
+};
+__device__ __forceinline__ dlrow dlrow_prod(cx<df64> a, df64x2 b)
+{
+    return {dl2_prod(dl2_both(a.re), b), dl2_prod(dl2_both(a.im), b)};
+}
+__device__ __forceinline__ void dlrow_fma(dlrow &s, cx<df64> a, df64x2 b)
+{
+    dl2_fma(s.r, dl2_both(a.re), b);
+    dl2_fma(s.i, dl2_both(a.im), b);
+}
+// r + (i.im, -i.re): the sum with the conjugates of the a_k
+__device__ __forceinline__ df64x2 dlrow_conj(const dlrow &s)
+{
+    df64x2 t = s.r;
+    dl2_add(t, {make_float2(s.i.h.y, -s.i.h.x), make_float2(s.i.l.y, -s.i.l.x)});
+    return t;
+}
+// (-i.im, i.re), the part of the sum that s.i holds
+__device__ __forceinline__ df64x2 dlrow_rot(const dlrow &s)
+{
+    return {make_float2(-s.i.h.y, s.i.h.x), make_float2(-s.i.l.y, s.i.l.x)};
+}
 
 template <typename R>
 __device__ __forceinline__ cx<R> mk(R a, R b) { return cx<R>{a, b}; }
@@ -361,9 +447,13 @@ struct St<float> {
 };
 
 // one df64 complex (or a pair of df64 reals) in 16 bytes: the df64 layouts
-// mirror the FP64 ones vector for vector
+// mirror the FP64 ones vector for vector.  In memory the two high parts come
+// first, so that a 16-byte load leaves the high parts in one register pair and
+// the low parts in the next, as the packed arithmetic takes them.
 struct __align__(16) df2 {
-    float rh, rl, ih, il;
+    float rh, ih, rl, il;
+    __host__ __device__ df2() {}
+    __host__ __device__ df2(float rh_, float rl_, float ih_, float il_) : rh(rh_), ih(ih_), rl(rl_), il(il_) {}
 };
 
 template <>
@@ -403,7 +493,7 @@ __device__ __forceinline__ float4 ldg(const F4S *p)
 __device__ __forceinline__ df2 ldg(const df2 *p)
 {
     const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-    return df2{t.x, t.y, t.z, t.w};
+    return df2(t.x, t.z, t.y, t.w);
 }
 __device__ __forceinline__ cx<df64> df2_cx(df2 t) { return {df64(t.rh, t.rl), df64(t.ih, t.il)}; }
 __device__ __forceinline__ df2 cx_df2(cx<df64> v) { return df2{v.re.hi, v.re.lo, v.im.hi, v.im.lo}; }
