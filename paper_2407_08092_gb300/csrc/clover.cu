@@ -84,6 +84,26 @@ __device__ __forceinline__ void shifted(const Geom &g, const int c[4], int mu, i
     else out[3] = v;
 }
 
+// sum_k conj(B_k) A_k over three entries of two rows (or columns) `step` apart
+__device__ __forceinline__ df64x2 conj_dot(const cx<df64> *B, const cx<df64> *A, int step)
+{
+    dlrow t = dlrow_prod(B[0], dl2(A[0]));
+    dlrow_fma(t, B[step], dl2(A[step]));
+    dlrow_fma(t, B[2 * step], dl2(A[2 * step]));
+    return dlrow_conj(t);
+}
+
+// Im sum_k conj(B_k) A_k, unnormalised: both products of a term in one packed sum
+__device__ __forceinline__ df64 im_conj_dot(const cx<df64> *B, const cx<df64> *A, int step)
+{
+    df64x2 t = dl2_prod(dl2(B[0]), dl2_swap(dl2(A[0])));   // (B.re A.im, B.im A.re)
+    dl2_fma(t, dl2(B[step]), dl2_swap(dl2(A[step])));
+    dl2_fma(t, dl2(B[2 * step]), dl2_swap(dl2(A[2 * step])));
+    cx<df64> s = dl2_cx(t);
+    dl_add(s.re, dl_neg(s.im));
+    return s.re;
+}
+
 // A B^+ (full product), each entry a lazily normalised compensated sum
 __device__ __forceinline__ M3<df64> mat_mul_nd(const M3<df64> &A, const M3<df64> &B)
 {
@@ -91,13 +111,8 @@ __device__ __forceinline__ M3<df64> mat_mul_nd(const M3<df64> &A, const M3<df64>
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
-        for (int b = 0; b < 3; b++) {
-            // sum_k A_ak conj(B_bk) = sum_k conj(B_bk) A_ak
-            cx<df64> acc = dl_cmul(cconj(B.a[b * 3]), A.a[a * 3]);
-            dl_cfmac(acc, B.a[b * 3 + 1], A.a[a * 3 + 1]);
-            dl_cfmac(acc, B.a[b * 3 + 2], A.a[a * 3 + 2]);
-            P.a[a * 3 + b] = dl_cnorm(acc);
-        }
+        for (int b = 0; b < 3; b++)   // sum_k A_ak conj(B_bk)
+            P.a[a * 3 + b] = dl2_cx(dl2_norm(conj_dot(B.a + b * 3, A.a + a * 3, 1)));
     return P;
 }
 
@@ -105,31 +120,18 @@ __device__ __forceinline__ M3<df64> mat_mul_nd(const M3<df64> &A, const M3<df64>
 __device__ __forceinline__ void ah_of_mul_nd(const M3<df64> &A, const M3<df64> &B, df64 v[9])
 {
 #pragma unroll
-    for (int a = 0; a < 3; a++) {   // Im sum_k A_ak conj(B_ak) = sum_k (A.im B.re - A.re B.im)
-        df64 s = dl_prod(A.a[a * 3].im, B.a[a * 3].re);
-        dl_fma(s, dl_neg(A.a[a * 3].re), B.a[a * 3].im);
-#pragma unroll
-        for (int k = 1; k < 3; k++) {
-            dl_fma(s, A.a[a * 3 + k].im, B.a[a * 3 + k].re);
-            dl_fma(s, dl_neg(A.a[a * 3 + k].re), B.a[a * 3 + k].im);
-        }
-        v[a] = dl_scale2(dl_norm(s), 2.0f);
-    }
+    for (int a = 0; a < 3; a++) v[a] = dl_scale2(dl_norm(im_conj_dot(B.a + a * 3, A.a + a * 3, 1)), 2.0f);
     const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
 #pragma unroll
     for (int q = 0; q < 3; q++) {
         const int a = pa[q], b = pb[q];
         // X = sum_k A_ak conj(B_bk), Y = sum_k A_bk conj(B_ak); AH_ab = X - conj(Y)
-        cx<df64> x = dl_cmul(cconj(B.a[b * 3]), A.a[a * 3]), y = dl_cmul(cconj(B.a[a * 3]), A.a[b * 3]);
-#pragma unroll
-        for (int k = 1; k < 3; k++) {
-            dl_cfmac(x, B.a[b * 3 + k], A.a[a * 3 + k]);
-            dl_cfmac(y, B.a[a * 3 + k], A.a[b * 3 + k]);
-        }
-        dl_add(x.re, dl_neg(y.re));
-        dl_add(x.im, y.im);
-        v[3 + 2 * q] = dl_norm(x.re);
-        v[4 + 2 * q] = dl_norm(x.im);
+        df64x2 x = conj_dot(B.a + b * 3, A.a + a * 3, 1);
+        const cx<df64> y = dl2_cx(conj_dot(B.a + a * 3, A.a + b * 3, 1));
+        dl2_add(x, dl2({dl_neg(y.re), y.im}));
+        const cx<df64> n = dl2_cx(dl2_norm(x));
+        v[3 + 2 * q] = n.re;
+        v[4 + 2 * q] = n.im;
     }
 }
 
@@ -138,25 +140,13 @@ __device__ __forceinline__ void ah_conj(const M3<df64> &H, const M3<df64> &W, df
 {
     const M3<df64> Y = mat_mul<df64>(H, W);
 #pragma unroll
-    for (int a = 0; a < 3; a++) {   // Im sum_k conj(W_ka) Y_ka = sum_k (W.re Y.im - W.im Y.re)
-        df64 s = dl_prod(W.a[a].re, Y.a[a].im);
-        dl_fma(s, dl_neg(W.a[a].im), Y.a[a].re);
-#pragma unroll
-        for (int k = 1; k < 3; k++) {
-            dl_fma(s, W.a[k * 3 + a].re, Y.a[k * 3 + a].im);
-            dl_fma(s, dl_neg(W.a[k * 3 + a].im), Y.a[k * 3 + a].re);
-        }
-        v[a] = dl_norm(s);
-    }
+    for (int a = 0; a < 3; a++) v[a] = dl_norm(im_conj_dot(W.a + a, Y.a + a, 3));   // Im sum_k conj(W_ka) Y_ka
     const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
 #pragma unroll
-    for (int q = 0; q < 3; q++) {
-        const int a = pa[q], b = pb[q];
-        cx<df64> z = dl_cmul(cconj(W.a[a]), Y.a[b]);   // sum_k conj(W_ka) Y_kb
-#pragma unroll
-        for (int k = 1; k < 3; k++) dl_cfmac(z, W.a[k * 3 + a], Y.a[k * 3 + b]);
-        v[3 + 2 * q] = dl_norm(z.re);
-        v[4 + 2 * q] = dl_norm(z.im);
+    for (int q = 0; q < 3; q++) {   // sum_k conj(W_ka) Y_kb
+        const cx<df64> n = dl2_cx(dl2_norm(conj_dot(W.a + pa[q], Y.a + pb[q], 3)));
+        v[3 + 2 * q] = n.re;
+        v[4 + 2 * q] = n.im;
     }
 }
 

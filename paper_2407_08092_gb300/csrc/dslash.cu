@@ -517,28 +517,47 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 5) hop_tile_kernel(const LatDe
 // forward and +1 for the backward hop), and the backward link enters as U^+.
 // ---------------------------------------------------------------------------
 // y += A x for one packed Hermitian 6x6 block A (reals 0..5 the diagonal,
-// then the strictly lower entries), read one entry at a time as the product
+// then the strictly lower entries), ld(k) its k-th vector, read as the product
 // needs it; the six sums are lazily normalised (dl_*) and left unnormalised.
-__device__ __forceinline__ void herm6_fma_df(const df2 *__restrict__ Cb, long long stride, const cx<df64> x[6],
-                                             cx<df64> y[6])
+template <typename Ld>
+__device__ __forceinline__ void herm6_fma_df(Ld ld, const cx<df64> x[6], cx<df64> y[6])
 {
 #pragma unroll
     for (int k = 0; k < 3; k++) {   // the diagonal: reals 2k, 2k+1
-        const df2 t = ldg(Cb + k * stride);
-        const df64 d0(t.rh, t.rl), d1(t.ih, t.il);
-        dl_fma(y[2 * k].re, d0, x[2 * k].re);
-        dl_fma(y[2 * k].im, d0, x[2 * k].im);
-        dl_fma(y[2 * k + 1].re, d1, x[2 * k + 1].re);
-        dl_fma(y[2 * k + 1].im, d1, x[2 * k + 1].im);
+        const df2 t = ld(k);
+        df64x2 y0 = dl2(y[2 * k]), y1 = dl2(y[2 * k + 1]);
+        dl2_fma(y0, dl2_both(df64(t.rh, t.rl)), dl2(x[2 * k]));
+        dl2_fma(y1, dl2_both(df64(t.ih, t.il)), dl2(x[2 * k + 1]));
+        y[2 * k] = dl2_cx(y0);
+        y[2 * k + 1] = dl2_cx(y1);
     }
+    // the lower entries l_ij and their conjugates above the diagonal: the real
+    // parts' products go straight into y, the imaginary parts' into z, whose
+    // parts are exchanged once at the end
+    df64x2 z[6];
 #pragma unroll
     for (int i = 1; i < 6; i++)
 #pragma unroll
         for (int j = 0; j < i; j++) {
-            const cx<df64> l = df2_cx(ldg(Cb + (3 + tri(i, j)) * stride));
-            dl_cfma(y[i], l, x[j]);    // lower entry
-            dl_cfmac(y[j], l, x[i]);   // its conjugate above the diagonal
+            const cx<df64> l = df2_cx(ld(3 + tri(i, j)));
+            const df64x2 re = dl2_both(l.re), im = dl2_both(l.im), xi = dl2(x[i]), xj = dl2(x[j]);
+            df64x2 yi = dl2(y[i]), yj = dl2(y[j]);
+            dl2_fma(yi, re, xj);
+            dl2_fma(yj, re, xi);
+            y[i] = dl2_cx(yi);
+            y[j] = dl2_cx(yj);
+            if (j == 0) z[i] = dl2_prod(im, xj);
+            else dl2_fma(z[i], im, xj);
+            const df64x2 mi = dl2_both(dl_neg(l.im));
+            if (i == 1) z[j] = dl2_prod(mi, xi);
+            else dl2_fma(z[j], mi, xi);
         }
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        df64x2 yi = dl2(y[i]);
+        dl2_add(yi, dlrow_rot({yi, z[i]}));
+        y[i] = dl2_cx(yi);
+    }
 }
 
 __device__ __forceinline__ cx<df64> rot_i(cx<df64> z, int q)   // i^q z
@@ -547,9 +566,26 @@ __device__ __forceinline__ cx<df64> rot_i(cx<df64> z, int q)   // i^q z
     return (q & 2) ? cx<df64>{-a.re, -a.im} : a;
 }
 
+// Operands staged ahead of their use (below): vectors of 16 bytes per thread,
+// each thread reading only what it copied itself.
+constexpr int kDfPsi = 0;        // the neighbour's 12 components
+constexpr int kDfLink = 12;      // two buffers of 9 link entries
+constexpr int kDfVecs = 30;
+__device__ __forceinline__ void copy_async(float4 *dst, const df2 *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// a use of v that the compiler keeps before the copies that follow
+__device__ __forceinline__ void used(cx<df64> v) { asm volatile("" ::"f"(v.re.hi), "f"(v.re.lo), "f"(v.im.hi), "f"(v.im.lo) : "memory"); }
+
 template <int MODE>
 __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &k, const df2 *in, const df2 *in2,
-                                            const df2 *bv, df2 *out, df2 *out2, long long s, const Coords &c)
+                                            const df2 *bv, df2 *out, df2 *out2, long long s, const Coords &c,
+                                            float4 *stage)
 {
     // per direction d = 2 mu + (backward): the partner of h0 is psi_3 for x, y
     // and psi_2 for z, t (acc_2 takes u_1 resp. u_0); the i-powers
@@ -584,24 +620,64 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
         return (long long)LQ_IDX((coord == 0) ? s + (long long)(ext - 1) * dd : s - dd, g.Vh, B_DF_NB);
     };
 
+    // The kernel waits on its loads, not on its arithmetic, when each direction
+    // reads its operands as it comes to them (long scoreboard the first stall,
+    // the FMA pipe 60% busy at 12 warps an SM).  So they are copied to shared
+    // memory ahead: the links of direction d + 1 while d runs (two buffers),
+    // the neighbour of d + 1 as soon as d is projected, and the first clover
+    // block while the last direction is multiplied.
+    auto vec = [&](int e) {
+        const float4 t = stage[e * LQ_HOP_THREADS];
+        return cx<df64>{df64(t.x, t.z), df64(t.y, t.w)};
+    };
+    auto copy_psi = [&](long long nb) {
+#pragma unroll
+        for (int e = 0; e < 12; e++) copy_async(stage + (kDfPsi + e) * LQ_HOP_THREADS, in + nb + e * st);
+        copy_commit();
+    };
+    auto copy_link = [&](int d, long long nb) {
+        const bool fwd = (d & 1) == 0;
+        const df2 *Um = (fwd ? k.Uout : k.Uin) + (long long)(d >> 1) * 9 * st + (fwd ? s : nb);
+#pragma unroll
+        for (int e = 0; e < 9; e++) copy_async(stage + (kDfLink + (d & 1) * 9 + e) * LQ_HOP_THREADS, Um + e * st);
+        copy_commit();
+    };
+    bool flip;
+    long long nb = neighbour(0, flip);
+    copy_link(0, nb);
+    copy_psi(nb);
 #pragma unroll 1
     for (int d = 0; d < 8; d++) {
-        const int mu = d >> 1;
         const bool fwd = (d & 1) == 0;
-        bool flip;
-        const long long nb = neighbour(d, flip);
-        const df2 *pn = in + nb;
+        bool flip1 = false;
+        const long long nb1 = d < 7 ? neighbour(d + 1, flip1) : 0;
+#pragma unroll
+        for (int a = 0; a < 3; a++) used(acc[a]);   // the last direction's link entries are used up
+        if (d < 7) {
+            copy_link(d + 1, nb1);
+            copy_wait<1>();
+        } else {
+            copy_wait<0>();
+        }
         const int pa = d < 4 ? 3 : 2;
         const int qa = (QA >> (2 * d)) & 3, qb = (QB >> (2 * d)) & 3;
         cx<df64> h[6];
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            h[a] = df2_cx(ldg(pn + a * st));
-            dl_cadd(h[a], rot_i(df2_cx(ldg(pn + (pa == 3 ? 9 + a : 6 + a) * st)), qa));
-            h[3 + a] = df2_cx(ldg(pn + (3 + a) * st));
-            dl_cadd(h[3 + a], rot_i(df2_cx(ldg(pn + (pa == 3 ? 6 + a : 9 + a) * st)), qb));
+            h[a] = vec(kDfPsi + a);
+            dl_cadd(h[a], rot_i(vec(kDfPsi + (pa == 3 ? 9 + a : 6 + a)), qa));
+            h[3 + a] = vec(kDfPsi + 3 + a);
+            dl_cadd(h[3 + a], rot_i(vec(kDfPsi + (pa == 3 ? 6 + a : 9 + a)), qb));
         }
-        const df2 *Um = (fwd ? k.Uout : k.Uin) + (long long)mu * 9 * st + (fwd ? s : nb);
+#pragma unroll
+        for (int a = 0; a < 6; a++) used(h[a]);
+        if (d < 7) {
+            copy_psi(nb1);
+        } else if (MODE != HOP_PREP) {   // the first clover block, over the neighbour and the free link buffer
+#pragma unroll
+            for (int e = 0; e < 18; e++) copy_async(stage + e * LQ_HOP_THREADS, k.clov + e * st + s);
+            copy_commit();
+        }
         const int ra = d < 4 ? 1 : 0;
         const int qc = (QC >> (2 * d)) & 3, qd = (QD >> (2 * d)) & 3;
 #pragma unroll
@@ -610,14 +686,17 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             cx<df64> e[3];
 #pragma unroll
             for (int b = 0; b < 3; b++) {
-                const cx<df64> t = df2_cx(ldg(Um + (fwd ? a * 3 + b : b * 3 + a) * st));
+                const cx<df64> t = vec(kDfLink + (d & 1) * 9 + (fwd ? a * 3 + b : b * 3 + a));
                 e[b] = fwd ? t : cx<df64>{t.re, dl_neg(t.im)};
             }
-            cx<df64> u0 = dl_cmul(e[0], h[0]), u1 = dl_cmul(e[0], h[3]);
-            dl_cfma(u0, e[1], h[1]);
-            dl_cfma(u1, e[1], h[4]);
-            dl_cfma(u0, e[2], h[2]);
-            dl_cfma(u1, e[2], h[5]);
+            dlrow r0 = dlrow_prod(e[0], dl2(h[0])), r1 = dlrow_prod(e[0], dl2(h[3]));
+            dlrow_fma(r0, e[1], dl2(h[1]));
+            dlrow_fma(r1, e[1], dl2(h[4]));
+            dlrow_fma(r0, e[2], dl2(h[2]));
+            dlrow_fma(r1, e[2], dl2(h[5]));
+            dl2_add(r0.r, dlrow_rot(r0));
+            dl2_add(r1.r, dlrow_rot(r1));
+            cx<df64> u0 = dl2_cx(r0.r), u1 = dl2_cx(r1.r);
             if (flip) {
                 u0 = {dl_neg(u0.re), dl_neg(u0.im)};
                 u1 = {dl_neg(u1.re), dl_neg(u1.im)};
@@ -627,9 +706,20 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             dl_cadd(acc[6 + a], rot_i(ra ? u1 : u0, qc));
             dl_cadd(acc[9 + a], rot_i(ra ? u0 : u1, qd));
         }
+        nb = nb1;
+        flip = flip1;
     }
 #pragma unroll
     for (int i = 0; i < 12; i++) acc[i] = dl_cnorm(acc[i]);
+    if (MODE != HOP_PREP) {
+        // the first 12 vectors of the second clover block go where the links were
+#pragma unroll
+        for (int a = 0; a < 3; a++) used(acc[a]);
+#pragma unroll
+        for (int e = 0; e < 12; e++) copy_async(stage + (18 + e) * LQ_HOP_THREADS, k.clov + (18 + e) * st + s);
+        copy_commit();
+        copy_wait<1>();
+    }
 
     // the site term, one 6x6 clover block (spins 0,1 then 2,3) at a time: six
     // components of the output are formed and stored per block (register
@@ -637,7 +727,12 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
 #pragma unroll 1
     for (int blk = 0; blk < 2; blk++) {
         const long long o = (long long)blk * 6 * st + s;
-        const df2 *Cb = k.clov + (long long)blk * 18 * st + s;
+        auto Cb = [&](int e) {   // vector e of the clover block
+            if (blk && e >= 12) return ldg(k.clov + (18 + e) * st + s);
+            const float4 t = stage[(18 * blk + e) * LQ_HOP_THREADS];
+            return df2(t.x, t.z, t.y, t.w);
+        };
+        if (blk && MODE != HOP_PREP) copy_wait<0>();
         cx<df64> a6[6], y[6];
 #pragma unroll
         for (int i = 0; i < 6; i++) a6[i] = blk ? acc[6 + i] : acc[i];
@@ -647,7 +742,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
                 a6[i] = {dl_scale2(a6[i].re, -0.5f), dl_scale2(a6[i].im, -0.5f)};
                 y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
             }
-            herm6_fma_df(Cb, st, a6, y);
+            herm6_fma_df(Cb, a6, y);
 #pragma unroll
             for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
         } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL || MODE == HOP_RES) {   // y = C x +- 1/2 acc
@@ -658,7 +753,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
                 x6[i] = df2_cx(in2[o + i * st]);
                 y[i] = {dl_scale2(a6[i].re, f), dl_scale2(a6[i].im, f)};
             }
-            herm6_fma_df(Cb, st, x6, y);
+            herm6_fma_df(Cb, x6, y);
 #pragma unroll
             for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
             if (MODE == HOP_RICH) {   // x + omega (b - D x)
@@ -679,14 +774,14 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             if (MODE == HOP_RECON || MODE == HOP_RECON_RES) {
 #pragma unroll
                 for (int i = 0; i < 6; i++) y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-                herm6_fma_df(Cb, st, a6, y);
+                herm6_fma_df(Cb, a6, y);
 #pragma unroll
                 for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
                 if (MODE == HOP_RECON_RES) {   // the parity's residual u - C x_o of the x_o just formed
                     cx<df64> z[6];
 #pragma unroll
                     for (int i = 0; i < 6; i++) z[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-                    herm6_fma_df(k.clov2 + (long long)blk * 18 * st + s, st, y, z);
+                    herm6_fma_df([&](int e) { return ldg(k.clov2 + ((long long)blk * 18 + e) * st + s); }, y, z);
 #pragma unroll
                     for (int i = 0; i < 6; i++) out2[o + i * st] = cx_df2(a6[i] - dl_cnorm(z[i]));
                 }
@@ -700,22 +795,27 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
     }
 }
 
+// Three resident blocks per SM (168 registers, 61 KB of staging each): K1 / K2
+// take 158 / 171 us on 24^3 x 48 (0.65 of the copy bandwidth) against 168 / 178
+// at two; 187 / 193 before the staging and 214 / 215 with scalar arithmetic.
 #ifndef LQ_DF_MINB
-#define LQ_DF_MINB 1
+#define LQ_DF_MINB 3
 #endif
+// One thread per output site and right-hand side; the right-hand sides of a
+// site block are consecutive blocks, so its links and clover come from L2 for
+// all but the first.
 template <int MODE>
-__global__ void __launch_bounds__(128, MODE == HOP_RECON_RES ? 3 : LQ_DF_MINB) hop_df_kernel(const __grid_constant__ Geom g,
-                                                     const __grid_constant__ HopArgs<df64> k)
+__global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(const __grid_constant__ Geom g,
+                                                                const __grid_constant__ HopArgs<df64> k)
 {
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    extern __shared__ float4 df_stage[];
+    const unsigned sb = blockIdx.x / (unsigned)k.nrhs;
+    const long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
     if (s >= g.Vh) return;
     const Coords c = cb_coords(g, s, k.pout);
-#pragma unroll 1
-    for (int r = 0; r < k.nrhs; r++) {
-        const long long o = r * k.fs;
-        hop_df_body<MODE>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
-                          k.out2 ? k.out2 + o : nullptr, s, c);
-    }
+    const long long o = (blockIdx.x - sb * k.nrhs) * k.fs;
+    hop_df_body<MODE>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
+                      k.out2 ? k.out2 + o : nullptr, s, c, df_stage + threadIdx.x);
 }
 
 template <typename R>
@@ -750,7 +850,11 @@ static void launch_hop(const Exec &e, const HopCall &c)
     k.fs = (long long)St<R>::SPINOR_VECS * e.g.stride;
     const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
     if constexpr (std::is_same<R, df64>::value)
-        hop_df_kernel<MODE><<<blocks, 128, 0, e.st>>>(e.g, k);
+    {
+        constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
+        cudaFuncSetAttribute(hop_df_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        hop_df_kernel<MODE><<<blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.st>>>(e.g, k);
+    }
     else
     {
         // several right-hand sides of FP64 or FP32 fields: one launch each (the
