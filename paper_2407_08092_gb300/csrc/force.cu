@@ -170,7 +170,10 @@ __device__ __forceinline__ M3<df64> load_mat(const df2 *__restrict__ m, long lon
     return A;
 }
 
-// one row of a product added to a row of sums: s_j += sum_k r_k B_kj
+// one row of a product added to a row of sums: s_j += sum_k r_k B_kj.  Each
+// product and each sum is renormalised: twelve products summed with their low
+// parts left to grow put the force 9.6e-15 from its 64-bit value, 6.2e-15 so
+// (5.2 against 5.6 ms on 24^3 x 48).
 __device__ __forceinline__ void row_fma(cx<df64> s[3], const cx<df64> r[3], const M3<df64> &B)
 {
 #pragma unroll
@@ -179,9 +182,9 @@ __device__ __forceinline__ void row_fma(cx<df64> s[3], const cx<df64> r[3], cons
         dlrow_fma(t, r[1], dl2(B.a[3 + j]));
         dlrow_fma(t, r[2], dl2(B.a[6 + j]));
         df64x2 u = dl2(s[j]);
-        dl2_add(u, t.r);
-        dl2_add(u, dlrow_rot(t));
-        s[j] = dl2_cx(u);
+        dl2_add(t.r, dlrow_rot(t));
+        dl2_add(u, dl2_norm(t.r));
+        s[j] = dl2_cx(dl2_norm(u));
     }
 }
 
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, 
         if (j == 4 || j == 6) continue;
         df2 *o = S.at(p, j < 4 ? j : j == 5 ? F_EM : F_EN, id);
 #pragma unroll
-        for (int k = 0; k < 9; k++) o[(long long)k * S.n] = cx_df2(dl_cnorm(acc.a[k]));
+        for (int k = 0; k < 9; k++) o[(long long)k * S.n] = cx_df2(acc.a[k]);
     }
 }
 
@@ -333,7 +336,10 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
 #pragma unroll
         for (int a = 0; a < 3; a++)
 #pragma unroll
-            for (int b = 0; b < 3; b++) dl_cfmac(acc.a[a * 3 + b], w[b], y[a]);
+            for (int b = 0; b < 3; b++) {
+                dl_cfmac(acc.a[a * 3 + b], w[b], y[a]);
+                acc.a[a * 3 + b] = dl_cnorm(acc.a[a * 3 + b]);   // eight terms of one size
+            }
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             y[a] = ld_comp(Yn, g.stride, s * 3 + a, cbn);
@@ -343,14 +349,17 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
 #pragma unroll
         for (int a = 0; a < 3; a++)
 #pragma unroll
-            for (int b = 0; b < 3; b++) dl_cfmac(acc.a[a * 3 + b], y[b], w[a]);
+            for (int b = 0; b < 3; b++) {
+                dl_cfmac(acc.a[a * 3 + b], y[b], w[a]);
+                acc.a[a * 3 + b] = dl_cnorm(acc.a[a * 3 + b]);   // eight terms of one size
+            }
     }
     {
         const bool wrap = mu == 3 && c[3] == g.L[3] - 1;
         const float f = (wrap && g.tbc < 0) ? 0.5f : -0.5f;
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            const cx<df64> t = dl_cnorm(acc.a[k]);
+            const cx<df64> t = acc.a[k];
             acc.a[k] = {dl_scale2(t.re, f), dl_scale2(t.im, f)};
         }
     }
@@ -386,15 +395,12 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
             }
             row_fma(acc.a + 3 * i, r, B);
         }
-        if (second)
-#pragma unroll
-            for (int k = 0; k < 9; k++) acc.a[k] = dl_cnorm(acc.a[k]);
     }
 
     double2 *o = G + (lex * 4 + mu) * 9;
 #pragma unroll
     for (int k = 0; k < 9; k++) {
-        const cx<df64> v = dl_cnorm(acc.a[k]);
+        const cx<df64> v = acc.a[k];
         o[k] = make_double2(coef * df_join(v.re.hi, v.re.lo), coef * df_join(v.im.hi, v.im.lo));
     }
 }
