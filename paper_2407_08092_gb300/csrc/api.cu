@@ -37,6 +37,10 @@ typedef std::complex<double> cd;
 
 static constexpr int MAX_RESTART = 256;
 static constexpr int RED_SLOTS = 2 * MAX_RESTART + 8;
+// Sites per parity up to which the FP32 GMRES queues the next step's operator
+// before it reads a step's scalars.  The GPU idles about 10 us a step while the
+// host reads them; the product queued ahead of a cycle's last step is wasted.
+static constexpr long long kAheadSites = 1LL << 18;
 
 struct lq_ctx {
     Geom g;
@@ -64,6 +68,7 @@ struct lq_ctx {
     double *h_pin_dev = nullptr;   // h_pin's device mapping (written by get_values)
     int *h_int = nullptr, *h_int_dev = nullptr;   // pinned host ints and their device mapping
     double *d_coef = nullptr;  // device coefficients [2 * RED_SLOTS]
+    cudaEvent_t ev = nullptr;  // marks the step whose scalars the host waits for
     double *d_s2 = nullptr;    // device: squared scales s_j^2 of the FP32 GMRES basis [RED_SLOTS]
     std::map<std::string, std::pair<void *, size_t>> ws;
     std::vector<void *> owned;
@@ -455,7 +460,8 @@ double arnoldi_cgs2(lq_ctx *c, int prec, void *V, int k, void *w, Hess &H)
 
 // The FP32 GMRES keeps its basis unnormalised: v_j = s_j V_j with the scales
 // s_j on the host, which saves the pass that would scale each new vector by
-// 1 / ||w||.  set_scale passes s_j^2 to the device for the CGS coefficients.
+// 1 / ||w||.  The CGS coefficients take s_j^2 on the device: set_scale passes
+// the first of a cycle, multi_axpy_finish leaves the others there.
 void set_scale(lq_ctx *c, int j, double s)
 {
     const double s2 = s * s;
@@ -468,14 +474,21 @@ void set_scale(lq_ctx *c, int j, double s)
 // sum_j h_jk v_j, i.e. w -= sum_j s_j^2 (V_j, w) V_j (the reduction applies
 // s_j^2); the new vector V_{k+1} = w has s_{k+1} = 1 / ||w||, and the true
 // h_{k+1,k} = s_k ||w||, which is returned.
-double arnoldi_scaled(lq_ctx *c, void *V, int k, void *w, Hess &H, double *s)
+// `ahead`, work that needs only the new vector, is queued before the host waits
+// for the coefficients, so that the GPU has work while the host reads them.
+template <typename F>
+double arnoldi_scaled(lq_ctx *c, void *V, int k, void *w, Hess &H, double *s, F &&ahead)
 {
     Exec e = c->ex();
     const int n = k + 1;
     multi_dot_finish(e, V, n, w, c->red, c->d_s2);   // s_j^2 (V_j, w) into red.out
-    multi_axpy_finish(e, V, n, c->red, -1, w, n);    // w -= sum_j ..., ||w||^2 into red.out[n]
+    // w -= sum_j ..., ||w||^2 into red.out[n], s_{k+1}^2 into d_s2[n], red.out to the host
+    multi_axpy_finish(e, V, n, c->red, -1, w, n, c->d_s2, c->h_pin_dev);
     ck_launch(c, "arnoldi");
-    const double *hv = fetch(c, 0, n + 1);
+    ck(c, cudaEventRecord(c->ev, c->st), "cudaEventRecord");
+    ahead();
+    ck(c, cudaEventSynchronize(c->ev), "cudaEventSynchronize");
+    const double *hv = c->h_pin;
     for (int j = 0; j < n; j++) H.h(j, k) = cd(hv[2 * j], hv[2 * j + 1]) * (s[k] / s[j]);
     const double nrm2 = hv[2 * n];
     if (!std::isfinite(nrm2)) fail(c, LQ_ERR_NAN, "NaN/Inf in the Arnoldi process");
@@ -536,10 +549,18 @@ KResult gmres(lq_ctx *c, int prec, const void *b, void *x, int m, int max_cycles
         }
         H.reset(beta);
         int nk = 0;
+        bool done_ahead = false;   // w = D_S V_k was queued during step k - 1
         for (int k = 0; k < m; k++) {
             void *w = vec_at(c, prec, V, k + 1);
-            op_schur(c, prec, vec_at(c, prec, V, k), w, t);
-            const double hk1 = scaled ? arnoldi_scaled(c, V, k, w, H, s) : arnoldi_cgs2(c, prec, V, k, w, H);
+            if (!done_ahead) op_schur(c, prec, vec_at(c, prec, V, k), w, t);
+            done_ahead = false;
+            auto next_product = [&] {
+                if (c->g.Vh > kAheadSites || k == m - 1) return;
+                op_schur(c, prec, w, vec_at(c, prec, V, k + 2), t);
+                done_ahead = true;
+            };
+            const double hk1 =
+                scaled ? arnoldi_scaled(c, V, k, w, H, s, next_product) : arnoldi_cgs2(c, prec, V, k, w, H);
             double colnorm2 = hk1 * hk1;
             for (int j = 0; j <= k; j++) colnorm2 += std::norm(H.h(j, k));
             H.h(k + 1, k) = hk1;
@@ -549,8 +570,7 @@ KResult gmres(lq_ctx *c, int prec, const void *b, void *x, int m, int max_cycles
             R.relres = est / bnorm;
             const bool breakdown = hk1 <= 1e-14 * std::sqrt(colnorm2);
             if (breakdown || (tol > 0 && est <= tol * bnorm) || k == m - 1) break;
-            if (scaled) set_scale(c, k + 1, s[k + 1]);
-            else axpby(e, prec, 0.0, 0.0, w, 1.0 / hk1, 0.0, w);
+            if (!scaled) axpby(e, prec, 0.0, 0.0, w, 1.0 / hk1, 0.0, w);
         }
         std::vector<cd> y = H.solve(nk);
         if (scaled)   // x += sum_j y_j v_j = sum_j (y_j s_j) V_j
@@ -1420,6 +1440,7 @@ lq_status lq_create(lq_ctx **out, const lq_lattice *lat, void *stream)
         ck(c, cudaHostGetDevicePointer((void **)&c->h_pin_dev, c->h_pin, 0), "cudaHostGetDevicePointer");
         ck(c, cudaMallocHost((void **)&c->h_int, sizeof(int) * 4), "cudaMallocHost");
         ck(c, cudaHostGetDevicePointer((void **)&c->h_int_dev, c->h_int, 0), "cudaHostGetDevicePointer");
+        ck(c, cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming), "cudaEventCreate");
     } catch (const Fail &f) {
         lq_destroy(c);
         return f.s;
@@ -1436,6 +1457,7 @@ lq_status lq_destroy(lq_ctx *c)
     for (void *p : c->owned)
         if (p) cudaFree(p);
     if (c->h_pin) cudaFreeHost(c->h_pin);
+    if (c->ev) cudaEventDestroy(c->ev);
     if (c->h_int) cudaFreeHost(c->h_int);
     for (cudaEvent_t ev : c->prof.pool) cudaEventDestroy(ev);
     delete c;

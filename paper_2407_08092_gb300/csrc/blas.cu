@@ -8,7 +8,10 @@
 //
 // Reductions are two-stage and deterministic: a fixed grid (set by the
 // lattice size alone) writes one partial per block and value, then one block
-// per value sums the partials in a fixed tree order in FP64.  Dot products are
+// per value sums the partials in a fixed tree order in FP64.  The grid gives
+// every thread one vector of an FP32 field until four blocks per SM are
+// reached: a thread per site, as small lattices had before, left an 8^4 field
+// to 8 blocks that read one vector after the other.  Dot products are
 // (v, w) = sum conj(v) w, the inner product of Algorithm 2.
 #include "lq_kernels.h"
 
@@ -19,7 +22,7 @@ static constexpr int MAXJ = 8;   // vectors per multi-dot launch
 
 int reduction_blocks(const Geom &g)
 {
-    long long b = (g.Vh + RT - 1) / RT;
+    const long long b = (6 * g.Vh + RT - 1) / RT;
     return (int)(b < 608 ? b : 608);
 }
 
@@ -94,7 +97,8 @@ __device__ __forceinline__ void block_sum(A v[N], A *sh /* [RT/32][N] */)
 // fixed order (warp w takes values w, w + 8, ..., each lane the blocks lane,
 // lane + 32, ...), scales value v by scale[v / 2] when a scale is given, and
 // writes them to out[v]: a deterministic second stage without a second launch.
-__device__ __forceinline__ void last_block_finish(double *partial, int pitch, int v0, int nval,
+// True in the threads of that last block, after a barrier that orders out[v].
+__device__ __forceinline__ bool last_block_finish(double *partial, int pitch, int v0, int nval,
                                                   const double *scale, double *out, unsigned *ticket)
 {
     __shared__ bool last;
@@ -104,7 +108,7 @@ __device__ __forceinline__ void last_block_finish(double *partial, int pitch, in
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last) return;
+    if (!last) return false;
     __threadfence();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int v = v0 + warp; v < v0 + nval; v += RT / 32) {
@@ -115,6 +119,8 @@ __device__ __forceinline__ void last_block_finish(double *partial, int pitch, in
         if (lane == 0) out[v] = scale ? a * scale[v >> 1] : a;
     }
     if (threadIdx.x == 0) *ticket = 0u;
+    __syncthreads();
+    return true;
 }
 
 // ---- multi-dot: partial[blk][2*(slot0+j) + re/im] = block share of (v_j, w) ------
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(RT, 4) multi_axpy_kernel(const typename Vec<R>
 __global__ void __launch_bounds__(RT, 4) multi_axpy_fin_kernel(const float4 *__restrict__ Vb, long long n, int nv,
                                                                const double *c, float sign, float4 *y,
                                                                double *partial, int pitch, int nrm_slot, double *out,
-                                                               unsigned *ticket)
+                                                               unsigned *ticket, double *scale, double *host)
 {
     __shared__ float sh[RT / 32];
     __shared__ float csr[256], csi[256];
@@ -216,7 +222,12 @@ __global__ void __launch_bounds__(RT, 4) multi_axpy_fin_kernel(const float4 *__r
         partial[(long long)blockIdx.x * pitch + 2 * nrm_slot] = (double)nrm[0];
         partial[(long long)blockIdx.x * pitch + 2 * nrm_slot + 1] = 0.0;
     }
-    last_block_finish(partial, pitch, 2 * nrm_slot, 2, nullptr, out, ticket);
+    if (!last_block_finish(partial, pitch, 2 * nrm_slot, 2, nullptr, out, ticket)) return;
+    for (int v = threadIdx.x; v < 2 * nrm_slot + 2; v += RT) host[v] = out[v];
+    if (threadIdx.x == 0) {
+        const double n2 = out[2 * nrm_slot];
+        scale[nrm_slot] = n2 > 0.0 ? 1.0 / n2 : 0.0;
+    }
 }
 
 template <typename R>
@@ -512,12 +523,14 @@ void multi_axpy(const Exec &e, int prec, const void *V, int nv, const double *c_
     }
 }
 
-void multi_axpy_finish(const Exec &e, const void *V, int nv, const RedScratch &r, int sign, void *y, int nrm_slot)
+void multi_axpy_finish(const Exec &e, const void *V, int nv, const RedScratch &r, int sign, void *y, int nrm_slot,
+                       double *scale, double *h_mapped)
 {
     Launch L_(e, K_AXPY_F32, (double)e.g.Vh * sp_bytes(P32) * (nv + 2), (double)e.g.Vh * 96 * nv);
     const int blocks = reduction_blocks(e.g);
     multi_axpy_fin_kernel<<<blocks, RT, 0, e.st>>>((const float4 *)V, nvec(e.g, P32), nv, r.out, (float)sign,
-                                                   (float4 *)y, r.partial, 2 * r.maxv, nrm_slot, r.out, r.ticket);
+                                                   (float4 *)y, r.partial, 2 * r.maxv, nrm_slot, r.out, r.ticket, scale,
+                                                   h_mapped);
 }
 
 template <int NJ>

@@ -262,9 +262,13 @@ void multi_axpy(const Exec &e, int prec, const void *V, int nv, const double *c_
 // reduction launches: multi_dot_finish writes scale_j * (v_j, w) for j < nv to
 // r.out slots 0 .. nv-1 (the last block of each launch sums the partials in a
 // fixed order); multi_axpy_finish then forms y = y + sign * sum_j r.out_j v_j and
-// writes ||y_new||^2 to r.out slot nrm_slot (summed the same way by its last block)
+// writes ||y_new||^2 to r.out slot nrm_slot (summed the same way by its last block),
+// which also leaves 1 / ||y_new||^2 (0 for a zero vector) in scale[nrm_slot] and
+// copies slots 0 .. nrm_slot to pinned host memory at its device mapping h_mapped:
+// an Arnoldi step takes no launches for its scalars
 void multi_dot_finish(const Exec &e, const void *V, int nv, const void *w, const RedScratch &r, const double *scale);
-void multi_axpy_finish(const Exec &e, const void *V, int nv, const RedScratch &r, int sign, void *y, int nrm_slot);
+void multi_axpy_finish(const Exec &e, const void *V, int nv, const RedScratch &r, int sign, void *y, int nrm_slot,
+                       double *scale, double *h_mapped);
 // partials of (v_j, w) = sum conj(v_j) w for j < nv into slots slot0 + j
 void multi_dot(const Exec &e, int prec, const void *V, int nv, const void *w, const RedScratch &r,
                int slot0);
