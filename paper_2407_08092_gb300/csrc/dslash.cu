@@ -31,9 +31,13 @@ static_assert(LQ_HOP_THREADS == kHopBlock, "hopping block size");
 #define LQ_HOP_BOUNDS __launch_bounds__(LQ_HOP_THREADS)
 #endif
 
+#ifndef LQ_F64_THREADS
+#define LQ_F64_THREADS 32
+#endif
+
 // one hop: acc += (1 -+ g_mu) W psi(nb), W = U_mu(x) (SIGN -1) or U_mu(x-mu)^+ (SIGN +1);
 // `bsign` is the fermion boundary factor of this hop
-template <int MU, int SIGN, typename R, typename SV, typename LV>
+template <int MU, int SIGN, bool FIRST = false, typename R, typename SV, typename LV>
 __device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *__restrict__ psi, const LV *__restrict__ U,
                                         long long link_site, long long nb, long long stride, R bsign)
 {
@@ -41,7 +45,7 @@ __device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *__restrict__ ps
     load_spinor(psi, stride, nb, p);
     cx<R> m[9];
     load_link(U, stride, MU, link_site, m);
-    hop_apply<MU, SIGN>(acc, p, m, bsign);
+    hop_apply<MU, SIGN, FIRST>(acc, p, m, bsign);
 }
 
 template <typename R>
@@ -72,8 +76,10 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
 {
     const long long st = g.stride;
     cx<R> acc[12];
+    constexpr bool SET = std::is_same<R, double>::value;   // FP32: the compiler's schedule is the better with a zeroed sum
+    if (!SET)
 #pragma unroll
-    for (int i = 0; i < 12; i++) acc[i] = {R(0), R(0)};
+        for (int i = 0; i < 12; i++) acc[i] = {R(0), R(0)};
     const R one = R(1);
 
     // x direction: the neighbour changes x, so its cb index is recomputed
@@ -82,7 +88,7 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
         const int xp = (c.x + 1 == g.L[0]) ? 0 : c.x + 1;
         const int xm = (c.x == 0) ? g.L[0] - 1 : c.x - 1;
         const long long nf = LQ_IDX(base + (xp >> 1), g.Vh, B_HOP_NB), nb = LQ_IDX(base + (xm >> 1), g.Vh, B_HOP_NB);
-        hop_dir<0, -1>(acc, in, Uout, s, nf, st, one);
+        hop_dir<0, -1, SET>(acc, in, Uout, s, nf, st, one);
         hop_dir<0, +1>(acc, in, Uin, nb, nb, st, one);
     }
     // y, z, t: x is unchanged, so the cb index moves by a fixed stride
@@ -509,12 +515,9 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 5) hop_tile_kernel(const LatDe
 // ---------------------------------------------------------------------------
 // df64 variant.  Each df64 operation is a chain of several FP32 instructions,
 // so the fully unrolled eight-direction body of hop_kernel would not fit the
-// instruction cache.  Here the eight hops share one loop body: the spin
-// projection and reconstruction of direction d are the table entries
-//   h0 = psi_0 + i^qa psi_pa,  h1 = psi_1 + i^qb psi_(5-pa)
-//   acc_2 += i^qc u_ra,        acc_3 += i^qd u_(1-ra)
-// (the same identities as `project` / `reconstruct` above, with s = -1 for the
-// forward and +1 for the backward hop), and the backward link enters as U^+.
+// instruction cache.  Here the eight hops share one loop body, the direction a
+// table index of the spin projection and reconstruction (spin.cuh); the
+// backward link enters as U^+.
 // ---------------------------------------------------------------------------
 // y += A x for one packed Hermitian 6x6 block A (reals 0..5 the diagonal,
 // then the strictly lower entries), ld(k) its k-th vector, read as the product
@@ -560,12 +563,6 @@ __device__ __forceinline__ void herm6_fma_df(Ld ld, const cx<df64> x[6], cx<df64
     }
 }
 
-__device__ __forceinline__ cx<df64> rot_i(cx<df64> z, int q)   // i^q z
-{
-    const cx<df64> a = (q & 1) ? cx<df64>{-z.im, z.re} : z;
-    return (q & 2) ? cx<df64>{-a.re, -a.im} : a;
-}
-
 // Operands staged ahead of their use (below): vectors of 16 bytes per thread,
 // each thread reading only what it copied itself.
 constexpr int kDfPsi = 0;        // the neighbour's 12 components
@@ -587,37 +584,20 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
                                             const df2 *bv, df2 *out, df2 *out2, long long s, const Coords &c,
                                             float4 *stage)
 {
-    // per direction d = 2 mu + (backward): the partner of h0 is psi_3 for x, y
-    // and psi_2 for z, t (acc_2 takes u_1 resp. u_0); the i-powers
-    //   qa = {1,3,0,2,1,3,2,0}, qb = {1,3,2,0,3,1,2,0},
-    //   qc = {3,1,2,0,3,1,2,0}, qd = {3,1,0,2,1,3,2,0}
-    // are packed two bits per direction (no local-memory tables).  The
+    // The directions run through one loop body (the tables of spin.cuh).  The
     // neighbour's components and the link's entries are read as the
     // projection and the product use them, and every sum is lazily normalised
     // (dl_*): acc is renormalised once, after the eight directions.
-    constexpr unsigned QA = 11661u, QB = 10029u, QC = 10023u, QD = 11655u;
     const long long st = g.stride;
     cx<df64> acc[12];
 #pragma unroll
     for (int i = 0; i < 12; i++) acc[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
 
-    // the neighbour's checkerboard index in direction d, and whether the time
-    // boundary flips the sign of the hop
+    // the neighbour in direction d, and whether the time boundary flips the hop's sign
     auto neighbour = [&](int d, bool &flip) {
-        const int mu = d >> 1;
-        const bool fwd = (d & 1) == 0;
-        flip = false;
-        if (mu == 0) {
-            const int xn = fwd ? (c.x + 1 == g.L[0] ? 0 : c.x + 1) : (c.x == 0 ? g.L[0] - 1 : c.x - 1);
-            return (long long)LQ_IDX(c.row * g.Lxh + (xn >> 1), g.Vh, B_DF_NB);
-        }
-        const int coord = mu == 1 ? c.y : mu == 2 ? c.z : c.t;
-        const int ext = g.L[mu];
-        const long long dd = mu == 1 ? (long long)g.Lxh
-                           : mu == 2 ? (long long)g.Lxh * g.L[1] : (long long)g.Lxh * g.L[1] * g.L[2];
-        if (mu == 3) flip = g.tbc < 0 && (fwd ? coord + 1 == ext : coord == 0);
-        if (fwd) return (long long)LQ_IDX((coord + 1 == ext) ? s - (long long)(ext - 1) * dd : s + dd, g.Vh, B_DF_NB);
-        return (long long)LQ_IDX((coord == 0) ? s + (long long)(ext - 1) * dd : s - dd, g.Vh, B_DF_NB);
+        const long long nb = hop_neighbour(g, c, s, d, flip, B_DF_NB);
+        flip = flip && g.tbc < 0;
+        return nb;
     };
 
     // The kernel waits on its loads, not on its arithmetic, when each direction
@@ -660,7 +640,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             copy_wait<0>();
         }
         const int pa = d < 4 ? 3 : 2;
-        const int qa = (QA >> (2 * d)) & 3, qb = (QB >> (2 * d)) & 3;
+        const int qa = (kHopQA >> (2 * d)) & 3, qb = (kHopQB >> (2 * d)) & 3;
         cx<df64> h[6];
 #pragma unroll
         for (int a = 0; a < 3; a++) {
@@ -679,7 +659,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             copy_commit();
         }
         const int ra = d < 4 ? 1 : 0;
-        const int qc = (QC >> (2 * d)) & 3, qd = (QD >> (2 * d)) & 3;
+        const int qc = (kHopQC >> (2 * d)) & 3, qd = (kHopQD >> (2 * d)) & 3;
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             // row a of U (forward) or of U^+ (backward): entries m[a*3+b] or conj(m[b*3+a])
@@ -848,7 +828,10 @@ static void launch_hop(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)St<R>::SPINOR_VECS * e.g.stride;
-    const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
+    // FP64 blocks are one warp: the FP64 pipe is the bound, so the sites have to
+    // spread evenly over the SMs (D_S on 16^4: 172 us with 64 threads, 155 with 32)
+    constexpr int threads = std::is_same<R, double>::value ? LQ_F64_THREADS : LQ_HOP_THREADS;
+    const unsigned blocks = (unsigned)((e.g.Vh + threads - 1) / threads);
     if constexpr (std::is_same<R, df64>::value)
     {
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
@@ -870,7 +853,7 @@ static void launch_hop(const Exec &e, const HopCall &c)
             if constexpr (std::is_same<R, float>::value && (MODE == HOP_K2 || MODE == HOP_RICH))
                 hop_kernel_occ<R, MODE><<<blocks, LQ_HOP_THREADS, 0, e.st>>>(e.g, kr);
             else
-                hop_kernel<R, MODE><<<blocks, LQ_HOP_THREADS, 0, e.st>>>(e.g, kr);
+                hop_kernel<R, MODE><<<blocks, threads, 0, e.st>>>(e.g, kr);
         }
     }
 }
@@ -977,6 +960,7 @@ void hop(const Exec &e, const HopCall &c)
     const double site_bytes = c.prec == PDF ? hop_site_bytes(c.mode, c.prec, c.nrhs)
                                             : c.nrhs * hop_site_bytes(c.mode, c.prec, 1);
     Launch L_(e, hop_class(c.mode, c.prec), (double)e.g.Vh * site_bytes, (double)e.g.Vh * c_hop_flops[c.mode] * c.nrhs);
+    if (hop_split(e, c)) return;
     switch (c.mode) {
         LQ_CASE(HOP_K1)
         LQ_CASE(HOP_K2)

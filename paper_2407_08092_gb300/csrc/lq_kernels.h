@@ -191,6 +191,9 @@ struct HopCall {
     int nrhs = 1;          // right-hand sides: in, in2, b, out are nrhs consecutive fields
 };
 void hop(const Exec &e, const HopCall &c);
+// the same by the kernels of small lattices (hop_split.cu); false, and nothing
+// done, where the one-thread kernels are the faster ones
+bool hop_split(const Exec &e, const HopCall &c);
 
 // One member lattice of a batched solve over lattices of different sizes: its
 // geometry, FP32 links and clover, and where its right-hand sides' fields sit
