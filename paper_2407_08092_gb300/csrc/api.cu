@@ -248,8 +248,10 @@ HopCall hopcall(lq_ctx *c, int mode, int prec, int pout)
 
 // ---- operators on internal fields ---------------------------------------------
 
-// out_e = D_S in_e (Eq. 3) via K1 (odd sites) and K2 (even sites); t: odd temporary
-void op_schur(lq_ctx *c, int prec, const void *in, void *out, void *t)
+// out_e = D_S in_e (Eq. 3) via K1 (odd sites) and K2 (even sites); t: odd temporary.
+// With `nat` the result goes there, in natural form, instead of to out (g5: with
+// spins 2 and 3 negated).
+void op_schur(lq_ctx *c, int prec, const void *in, void *out, void *t, void *nat = nullptr, bool g5 = false)
 {
     Exec e = c->ex();
     HopCall k1 = hopcall(c, HOP_K1, prec, 1);
@@ -262,6 +264,8 @@ void op_schur(lq_ctx *c, int prec, const void *in, void *out, void *t)
     k2.in2 = in;
     k2.out = out;
     k2.clov = Cp(c, prec, 0);
+    k2.nat = nat;
+    k2.nat_g5 = g5;
     hop(e, k2);
 }
 
@@ -284,21 +288,20 @@ void op_rich_sweep(lq_ctx *c, int prec, void *x, const void *b, double omega, vo
     hop(e, k2);
 }
 
-void op_full(lq_ctx *c, int prec, const void *ie, const void *io, void *oe, void *oo)
+// nat = D (ie, io), a natural full field
+void op_full(lq_ctx *c, int prec, const void *ie, const void *io, void *nat)
 {
     Exec e = c->ex();
-    HopCall a = hopcall(c, HOP_FULL, prec, 0);
-    a.in = io;
-    a.in2 = ie;
-    a.out = oe;
-    a.clov = Cp(c, prec, 0);
-    hop(e, a);
-    HopCall b = hopcall(c, HOP_FULL, prec, 1);
-    b.in = ie;
-    b.in2 = io;
-    b.out = oo;
-    b.clov = Cp(c, prec, 1);
-    hop(e, b);
+    for (int p = 0; p < 2; p++) {
+        HopCall a = hopcall(c, HOP_FULL, prec, p);
+        a.in = p ? ie : io;
+        a.in2 = p ? io : ie;
+        a.out = nullptr;
+        a.clov = Cp(c, prec, p);
+        a.nat = nat;
+        a.nat_full = true;
+        hop(e, a);
+    }
 }
 
 // bhat_e = b_e - D_eo D_oo^{-1} b_o
@@ -1522,34 +1525,27 @@ lq_status lq_apply(lq_ctx *c, int op, int prec, const void *in, void *out)
         need_gauge(c);
         Exec e = c->ex();
         void *a = field(c, prec, "apply:a"), *b = field(c, prec, "apply:b");
-        void *d = field(c, prec, "apply:d"), *f = field(c, prec, "apply:f");
         switch (op) {
         case LQ_OP_FULL:
             import_full(e, prec, in, a, b);
-            op_full(c, prec, a, b, d, f);
-            export_full(e, prec, d, f, out);
+            op_full(c, prec, a, b, out);
             break;
         case LQ_OP_SCHUR:
-            import_half(e, prec, in, a);
-            op_schur(c, prec, a, d, b);
-            export_half(e, prec, d, out);
+        case LQ_OP_SCHUR_DAG: {   // D_S^+ = g5 D_S g5
+            const bool dag = op == LQ_OP_SCHUR_DAG;
+            import_half(e, prec, in, a, dag);
+            op_schur(c, prec, a, nullptr, b, out, dag);
             break;
-        case LQ_OP_SCHUR_DAG:
-            import_half(e, prec, in, a);
-            gamma5(e, prec, a, a);
-            op_schur(c, prec, a, d, b);
-            gamma5(e, prec, d, d);
-            export_half(e, prec, d, out);
-            break;
+        }
         case LQ_OP_EE:
             import_half(e, prec, in, a);
-            clover_mul(e, prec, Cp(c, prec, 0), a, d);
-            export_half(e, prec, d, out);
+            clover_mul(e, prec, Cp(c, prec, 0), a, b);
+            export_half(e, prec, b, out);
             break;
         case LQ_OP_OO_INV:
             import_half(e, prec, in, a);
-            clover_mul(e, prec, Cip(c, prec), a, d);
-            export_half(e, prec, d, out);
+            clover_mul(e, prec, Cip(c, prec), a, b);
+            export_half(e, prec, b, out);
             break;
         default:
             fail(c, LQ_ERR_ARG, "bad op");

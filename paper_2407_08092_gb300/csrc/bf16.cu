@@ -72,29 +72,6 @@ __global__ void bf16_to_df_kernel(Geom g, const BfS4 *__restrict__ in, df2 *out)
     store_spinor(out, g.stride, s, d);
 }
 
-// natural [Vh][12] c128 <-> BF16 field of one parity
-__global__ void bf16_import_half_kernel(Geom g, const double2 *__restrict__ nat, BfS4 *f)
-{
-    const long long s = blockIdx.x * 256LL + threadIdx.x;
-    if (s >= g.Vh) return;
-    cx<float> v[12];
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-        const double2 t = nat[s * 12 + k];
-        v[k] = {(float)t.x, (float)t.y};
-    }
-    store_spinor(f, g.stride, s, v);
-}
-__global__ void bf16_export_half_kernel(Geom g, const BfS4 *__restrict__ f, double2 *nat)
-{
-    const long long s = blockIdx.x * 256LL + threadIdx.x;
-    if (s >= g.Vh) return;
-    cx<float> v[12];
-    load_spinor(f, g.stride, s, v);
-#pragma unroll
-    for (int k = 0; k < 12; k++) nat[s * 12 + k] = make_double2((double)v[k].re, (double)v[k].im);
-}
-
 // out = g5 in: spins 2, 3 (components 6..11) negated
 __global__ void bf16_gamma5_kernel(Geom g, const BfS4 *in, BfS4 *out)
 {
@@ -154,18 +131,6 @@ void bf16_convert(const Exec &e, int from, const void *in, int to, void *out)
     } else {
         bf16_to_df_kernel<<<b, 256, 0, e.st>>>(e.g, (const BfS4 *)in, (df2 *)out);
     }
-}
-
-void bf16_import_half(const Exec &e, const void *nat, void *f)
-{
-    Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + 48));
-    bf16_import_half_kernel<<<nb256(e.g.Vh), 256, 0, e.st>>>(e.g, (const double2 *)nat, (BfS4 *)f);
-}
-
-void bf16_export_half(const Exec &e, const void *f, void *nat)
-{
-    Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + 48));
-    bf16_export_half_kernel<<<nb256(e.g.Vh), 256, 0, e.st>>>(e.g, (const BfS4 *)f, (double2 *)nat);
 }
 
 void bf16_gamma5(const Exec &e, const void *in, void *out)

@@ -15,6 +15,7 @@
 
 #include "bf16.cuh"
 #include "lq_kernels.h"
+#include "nat.cuh"
 #include "spin.cuh"
 
 namespace lq {
@@ -64,15 +65,40 @@ struct HopArgs {
     int pout;
     int nrhs;        // right-hand sides sharing the links and clover of this launch
     long long fs;    // distance between consecutive right-hand sides' fields, in vectors
+    NatOut nat;      // natural output in the place of `out`
 };
+
+// all twelve components of a warp's sites in natural form, six at a time: seven
+// slots a row keep the shared-memory accesses free of bank conflicts
+constexpr int kNatRow = 7;
+template <typename SV, typename R>
+__device__ __forceinline__ void store_nat(const NatOut &o, double2 *tile, const SV *, long long s0, int n, int xbit,
+                                          const cx<R> v[12])
+{
+    const int lane = threadIdx.x & 31;
+    auto at = [](int r, int k) { return r * kNatRow + k; };
+#pragma unroll
+    for (int half = 0; half < 2; half++) {
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            double2 d = nat_value((const SV *)nullptr, v[6 * half + k]);
+            if (half) d = make_double2(flip_sign64(d.x, o.flip), flip_sign64(d.y, o.flip));
+            tile[at(lane, k)] = d;
+        }
+        __syncwarp();
+        nat_write6(o, tile, at, s0, n, xbit, half);
+    }
+}
 
 
 // SV, LV, CV: storage vectors of the spinors, links and clover blocks (the same
 // type for FP64, FP32 and df64; BF16 spinors and links with FP32 clover)
-template <typename R, int MODE, typename SV, typename LV, typename CV>
+template <typename R, int MODE, bool NAT = false, typename SV, typename LV, typename CV>
 __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV *Uin, const CV *clov, R omega,
                                          const SV *in, const SV *in2, const SV *bv, SV *out, long long s,
-                                         const Coords &c, const CV *clov2 = nullptr, SV *out2 = nullptr)
+                                         const Coords &c, const CV *clov2 = nullptr, SV *out2 = nullptr,
+                                         const NatOut &nat = NatOut(), double2 *tile = nullptr, int nvalid = 0)
 {
     const long long st = g.stride;
     cx<R> acc[12];
@@ -159,7 +185,8 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
             for (int i = 0; i < 12; i++) v[i] = y[i];
         }
     }
-    store_spinor(out, st, s, v);
+    if (NAT) store_nat(nat, tile, (const SV *)nullptr, s - min((int)(threadIdx.x & 31), nvalid - 1), nvalid, c.x & 1, v);
+    else store_spinor(out, st, s, v);
 }
 
 // One thread per output site.  The batched form (MULTI) loops over the
@@ -251,31 +278,50 @@ __device__ __forceinline__ void hop_body2(const Geom &g, const float4 *Uout, con
     }
 }
 
-template <typename R, int MODE>
+// The output site of a thread, and how many sites its warp has (its lanes from
+// there on shadow the last one): with natural output a warp stays whole.
+__device__ __forceinline__ long long warp_site(const Geom &g, int &nvalid)
+{
+    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x, s0 = s - (threadIdx.x & 31);
+    nvalid = (int)min(32LL, g.Vh - s0);
+    return min(s, g.Vh - 1);
+}
+template <typename R, int MODE, bool NAT>
+__device__ __forceinline__ void hop_site(const Geom &g, const HopArgs<R> &k)
+{
+    extern __shared__ __align__(16) double2 nat_tile[];
+    int nv = 0;
+    long long s;
+    if (NAT) {
+        s = warp_site(g, nv);
+        if (nv <= 0) return;
+    } else {
+        s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        if (s >= g.Vh) return;
+    }
+    const Coords c = cb_coords(g, s, k.pout);
+    double2 *tile = NAT ? nat_tile + (threadIdx.x >> 5) * 32 * kNatRow : nullptr;
+    if constexpr (std::is_same<R, float>::value)   // links and clover read once: no L1 allocation
+        hop_body<R, MODE, NAT>(g, (const F4S *)k.Uout, (const F4S *)k.Uin, (const F4S *)k.clov, k.omega, k.in, k.in2,
+                               k.b, k.out, s, c, (const F4S *)nullptr, (float4 *)nullptr, k.nat, tile, nv);
+    else
+        hop_body<R, MODE, NAT>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, k.clov2, k.out2, k.nat,
+                               tile, nv);
+}
+template <typename R, int MODE, bool NAT>
 __global__ void LQ_HOP_BOUNDS hop_kernel(Geom g, HopArgs<R> k)
 {
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (s >= g.Vh) return;
-    const Coords c = cb_coords(g, s, k.pout);
-    if constexpr (std::is_same<R, float>::value)   // links and clover read once: no L1 allocation
-        hop_body<R, MODE>(g, (const F4S *)k.Uout, (const F4S *)k.Uin, (const F4S *)k.clov, k.omega, k.in, k.in2,
-                          k.b, k.out, s, c);
-    else
-        hop_body<R, MODE>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, k.clov2, k.out2);
+    hop_site<R, MODE, NAT>(g, k);
 }
 
 // The same for FP32 K2 and its Richardson form, asked to fit six blocks per SM
 // (80 registers, a few bytes of spills): measured on GB300 on 32^3 x 64, K2
 // moves from 0.89 to 0.93 of the copy bandwidth this way, while K1 (78
 // registers unbounded) gains nothing.
-template <typename R, int MODE>
+template <typename R, int MODE, bool NAT>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_occ(Geom g, HopArgs<R> k)
 {
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (s >= g.Vh) return;
-    const Coords c = cb_coords(g, s, k.pout);
-    hop_body<R, MODE>(g, (const F4S *)k.Uout, (const F4S *)k.Uin, (const F4S *)k.clov, k.omega, k.in, k.in2, k.b,
-                      k.out, s, c);
+    hop_site<R, MODE, NAT>(g, k);
 }
 
 
@@ -287,15 +333,48 @@ struct HopArgsBF {
     const F4S *clov;   // FP32 clover blocks, read once
     float omega;
     int pout;
+    NatOut nat;
 };
+template <int MODE, bool NAT>
+__device__ __forceinline__ void hop_site_bf(const Geom &g, const HopArgsBF &k)
+{
+    extern __shared__ __align__(16) double2 nat_tile[];
+    int nv = 0;
+    long long s;
+    if (NAT) {
+        s = warp_site(g, nv);
+        if (nv <= 0) return;
+    } else {
+        s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        if (s >= g.Vh) return;
+    }
+    const Coords c = cb_coords(g, s, k.pout);
+    hop_body<float, MODE, NAT>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, (const F4S *)nullptr,
+                               (BfS4 *)nullptr, k.nat, NAT ? nat_tile + (threadIdx.x >> 5) * 32 * kNatRow : nullptr, nv);
+}
 template <int MODE>
 __global__ void LQ_HOP_BOUNDS hop_kernel_bf(Geom g, HopArgsBF k)
 {
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (s >= g.Vh) return;
-    const Coords c = cb_coords(g, s, k.pout);
-    hop_body<float, MODE>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c);
+    hop_site_bf<MODE, false>(g, k);
 }
+// K2 with natural output: held to the registers of the plain one (104 without the bound)
+__global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_bf_nat(Geom g, HopArgsBF k)
+{
+    hop_site_bf<HOP_K2, true>(g, k);
+}
+
+// shared memory of a block's natural output
+constexpr size_t nat_smem(int threads) { return (size_t)threads * kNatRow * sizeof(double2); }
+static NatOut nat_of(const HopCall &c)
+{
+    NatOut o;
+    o.p = (double2 *)c.nat;
+    o.full = c.nat_full;
+    o.flip = c.nat_g5 ? 0x80000000u : 0u;
+    return o;
+}
+// the modes that end a call on natural fields
+constexpr bool nat_mode(int mode) { return mode == HOP_K2 || mode == HOP_FULL || mode == HOP_RECON; }
 
 template <int MODE>
 static void launch_hop_bf(const Exec &e, const HopCall &c)
@@ -310,7 +389,14 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     k.clov = (const F4S *)c.clov;
     k.omega = (float)c.omega;
     k.pout = c.pout;
-    hop_kernel_bf<MODE><<<(unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS), LQ_HOP_THREADS, 0, e.st>>>(e.g, k);
+    k.nat = nat_of(c);
+    const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
+    if constexpr (MODE == HOP_K2)
+        if (c.nat) {
+            hop_kernel_bf_nat<<<blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.st>>>(e.g, k);
+            return;
+        }
+    hop_kernel_bf<MODE><<<blocks, LQ_HOP_THREADS, 0, e.st>>>(e.g, k);
 }
 
 // The batched hop over the right-hand sides of several lattices of different
@@ -579,10 +665,10 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group 
 // a use of v that the compiler keeps before the copies that follow
 __device__ __forceinline__ void used(cx<df64> v) { asm volatile("" ::"f"(v.re.hi), "f"(v.re.lo), "f"(v.im.hi), "f"(v.im.lo) : "memory"); }
 
-template <int MODE>
+template <int MODE, bool NAT>
 __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &k, const df2 *in, const df2 *in2,
                                             const df2 *bv, df2 *out, df2 *out2, long long s, const Coords &c,
-                                            float4 *stage)
+                                            float4 *stage, int nvalid)
 {
     // The directions run through one loop body (the tables of spin.cuh).  The
     // neighbour's components and the link's entries are read as the
@@ -770,8 +856,25 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
                 for (int i = 0; i < 6; i++) y[i] = a6[i];
             }
         }
+        if (NAT) {
+            // through the vectors of the staging area that block 0 has left (each
+            // lane's column turned by the component, against bank conflicts)
+            const int lane = threadIdx.x & 31;
+            double2 *tile = reinterpret_cast<double2 *>(stage - lane);
+            auto at = [](int r, int q) { return q * LQ_HOP_THREADS + ((r + q) & 31); };
+            const unsigned flip = blk ? k.nat.flip : 0u;
+            __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 6; i++) out[o + i * st] = cx_df2(y[i]);
+            for (int i = 0; i < 6; i++) {
+                const double2 d = nat_value((const df2 *)nullptr, y[i]);
+                tile[at(lane, i)] = make_double2(flip_sign64(d.x, flip), flip_sign64(d.y, flip));
+            }
+            __syncwarp();
+            nat_write6(k.nat, tile, at, s - min(lane, nvalid - 1), nvalid, c.x & 1, blk);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 6; i++) out[o + i * st] = cx_df2(y[i]);
+        }
     }
 }
 
@@ -784,18 +887,25 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
 // One thread per output site and right-hand side; the right-hand sides of a
 // site block are consecutive blocks, so its links and clover come from L2 for
 // all but the first.
-template <int MODE>
+template <int MODE, bool NAT>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ HopArgs<df64> k)
 {
     extern __shared__ float4 df_stage[];
     const unsigned sb = blockIdx.x / (unsigned)k.nrhs;
-    const long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
-    if (s >= g.Vh) return;
+    long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
+    int nv = 0;
+    if (NAT) {   // warps stay whole (warp_site)
+        nv = (int)min(32LL, g.Vh - (s - (threadIdx.x & 31)));
+        if (nv <= 0) return;
+        s = min(s, g.Vh - 1);
+    } else if (s >= g.Vh) {
+        return;
+    }
     const Coords c = cb_coords(g, s, k.pout);
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs;
-    hop_df_body<MODE>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
-                      k.out2 ? k.out2 + o : nullptr, s, c, df_stage + threadIdx.x);
+    hop_df_body<MODE, NAT>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
+                           k.out2 ? k.out2 + o : nullptr, s, c, df_stage + threadIdx.x, nv);
 }
 
 template <typename R>
@@ -832,11 +942,17 @@ static void launch_hop(const Exec &e, const HopCall &c)
     // spread evenly over the SMs (D_S on 16^4: 172 us with 64 threads, 155 with 32)
     constexpr int threads = std::is_same<R, double>::value ? LQ_F64_THREADS : LQ_HOP_THREADS;
     const unsigned blocks = (unsigned)((e.g.Vh + threads - 1) / threads);
+    k.nat = nat_of(c);
     if constexpr (std::is_same<R, df64>::value)
     {
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
-        cudaFuncSetAttribute(hop_df_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        hop_df_kernel<MODE><<<blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.st>>>(e.g, k);
+        auto launch = [&](auto kernel) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            kernel<<<blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.st>>>(e.g, k);
+        };
+        if constexpr (nat_mode(MODE))
+            if (c.nat) return launch(hop_df_kernel<MODE, true>);
+        launch(hop_df_kernel<MODE, false>);
     }
     else
     {
@@ -850,10 +966,20 @@ static void launch_hop(const Exec &e, const HopCall &c)
             kr.b = k.b ? k.b + o : nullptr;
             kr.out = k.out + o;
             kr.out2 = k.out2 ? k.out2 + o : nullptr;
-            if constexpr (std::is_same<R, float>::value && (MODE == HOP_K2 || MODE == HOP_RICH))
-                hop_kernel_occ<R, MODE><<<blocks, LQ_HOP_THREADS, 0, e.st>>>(e.g, kr);
-            else
-                hop_kernel<R, MODE><<<blocks, threads, 0, e.st>>>(e.g, kr);
+            const size_t sm = c.nat ? nat_smem(threads) : 0;
+            auto launch = [&](auto nat) {
+                constexpr bool NAT = decltype(nat)::value;
+                if constexpr (std::is_same<R, float>::value && (MODE == HOP_K2 || MODE == HOP_RICH))
+                    hop_kernel_occ<R, MODE, NAT><<<blocks, threads, sm, e.st>>>(e.g, kr);
+                else
+                    hop_kernel<R, MODE, NAT><<<blocks, threads, sm, e.st>>>(e.g, kr);
+            };
+            if constexpr (nat_mode(MODE)) {
+                if (c.nat) launch(std::true_type());
+                else launch(std::false_type());
+            } else {
+                launch(std::false_type());
+            }
         }
     }
 }
@@ -959,7 +1085,9 @@ void hop(const Exec &e, const HopCall &c)
     // counted once); FP64 and FP32 launch once per right-hand side
     const double site_bytes = c.prec == PDF ? hop_site_bytes(c.mode, c.prec, c.nrhs)
                                             : c.nrhs * hop_site_bytes(c.mode, c.prec, 1);
-    Launch L_(e, hop_class(c.mode, c.prec), (double)e.g.Vh * site_bytes, (double)e.g.Vh * c_hop_flops[c.mode] * c.nrhs);
+    // natural rows are complex doubles whatever the precision
+    const double nat_bytes = c.nat ? 192.0 - (double)spinor_bytes(e.g, c.prec) / e.g.stride : 0.0;
+    Launch L_(e, hop_class(c.mode, c.prec), (double)e.g.Vh * (site_bytes + nat_bytes), (double)e.g.Vh * c_hop_flops[c.mode] * c.nrhs);
     if (hop_split(e, c)) return;
     switch (c.mode) {
         LQ_CASE(HOP_K1)

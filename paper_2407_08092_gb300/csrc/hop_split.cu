@@ -19,6 +19,7 @@
 
 #include "bf16.cuh"
 #include "lq_kernels.h"
+#include "nat.cuh"
 #include "spin.cuh"
 
 namespace lq {
@@ -210,6 +211,7 @@ struct SplitArgs {
     R omega;
     int pout, nrhs;
     long long fs;
+    NatOut nat;
 };
 
 template <typename R, int MODE, typename SV, typename LV, typename CV>
@@ -291,7 +293,22 @@ __global__ void __launch_bounds__(kSplitThreads, std::is_same<R, df64>::value ? 
             }
         }
     }
-    if (on) st_comp(k.out + o, st, s, w, v);
+    if (k.nat.p) {   // 32 natural rows through shared memory, one vector a thread
+        double2 *tile = reinterpret_cast<double2 *>(split_sm);   // over U: 32 rows of 12 and a pad
+        double2 d = nat_value((const SV *)nullptr, v);
+        if (w >= 6) d = make_double2(flip_sign64(d.x, k.nat.flip), flip_sign64(d.y, k.nat.flip));
+        __syncthreads();
+        tile[lane * 13 + w] = d;
+        __syncthreads();
+        const int r = threadIdx.x / 12, c = threadIdx.x - 12 * r;
+        const long long q = sb * (long long)kSplitSites + r;
+        if (q < g.Vh) {
+            const long long row = k.nat.full ? 2 * q + (cb_coords(g, q, k.pout).x & 1) : q;
+            k.nat.p[row * 12 + c] = tile[r * 13 + c];
+        }
+    } else if (on) {
+        st_comp(k.out + o, st, s, w, v);
+    }
 }
 
 template <typename R, int MODE, typename SV, typename LV, typename CV>
@@ -311,6 +328,9 @@ static void launch_split(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)(spinor_bytes(e.g, c.prec) / sizeof(SV));
+    k.nat.p = (double2 *)c.nat;
+    k.nat.full = c.nat_full;
+    k.nat.flip = c.nat_g5 ? 0x80000000u : 0u;
     const unsigned blocks = (unsigned)((e.g.Vh + kSplitSites - 1) / kSplitSites) * (unsigned)c.nrhs;
     hop_split_kernel<R, MODE, SV, LV, CV><<<blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.st>>>(e.g, k);
 }

@@ -2,6 +2,7 @@
 // structure-of-arrays fields, precision conversion and the gamma_5 multiply.
 // (Sec. 2.4.5: odd-even reordering; the internal order is even sites first,
 // each parity in lexicographic order.)
+#include "bf16.cuh"
 #include "lq_kernels.h"
 
 namespace lq {
@@ -69,6 +70,18 @@ template <> struct Vec<P32> {
     }
 };
 
+template <> struct Vec<P16> {
+    static constexpr int N = 3;   // four complex components per 16-byte vector (import only)
+    typedef BfS4 T;
+    static __device__ __forceinline__ T from(const double2 *row, int k)
+    {
+        BfS4 t;
+#pragma unroll
+        for (int j = 0; j < 4; j++) t.c[j] = cx_bf({d2f_bits(row[4 * k + j].x), d2f_bits(row[4 * k + j].y)});
+        return t;
+    }
+};
+
 // row of the tile and internal site index of output item j of parity p
 // (FULL: lattice rows split by parity; else: a field of one parity, row = site)
 template <bool FULL>
@@ -90,14 +103,18 @@ __device__ __forceinline__ int tile_slot(int r)
 // natural [n][12] c128 -> internal field(s): f0 (FULL: even sites), f1 (odd sites)
 template <int PR, bool FULL>
 __global__ void __launch_bounds__(TT) import_tile_kernel(Geom g, const double2 *__restrict__ nat,
-                                                         typename Vec<PR>::T *f0, typename Vec<PR>::T *f1)
+                                                         typename Vec<PR>::T *f0, typename Vec<PR>::T *f1, bool g5)
 {
     __shared__ double2 tile[TS][TPAD];
     __shared__ unsigned char par[TS / 2];
     const long long n = FULL ? g.V : g.Vh;
     const long long r0 = (long long)blockIdx.x * TS;
     const int rows = (int)(n - r0 < TS ? n - r0 : TS);
-    for (int i = threadIdx.x; i < rows * 12; i += TT) tile[tile_slot<FULL>(i / 12)][i % 12] = __ldg(nat + r0 * 12 + i);
+    for (int i = threadIdx.x; i < rows * 12; i += TT) {
+        double2 t = __ldg(nat + r0 * 12 + i);
+        if (g5 && i % 12 >= 6) t = make_double2(-t.x, -t.y);
+        tile[tile_slot<FULL>(i / 12)][i % 12] = t;
+    }
     if (FULL && threadIdx.x < TS / 2 && 2 * (int)threadIdx.x < rows) par[threadIdx.x] = lex_parity(g, r0 + 2 * threadIdx.x);
     __syncthreads();
     constexpr int NV = Vec<PR>::N, PER = FULL ? TS / 2 : TS;
@@ -216,11 +233,11 @@ void import_links(const Exec &e, const void *U_nat, void *U64[2], void *U32[2], 
 
 // ---- spinors ----------------------------------------------------------------
 template <int PR, bool FULL>
-static void import_t(const Exec &e, const void *nat, void *f0, void *f1)
+static void import_t(const Exec &e, const void *nat, void *f0, void *f1, bool g5 = false)
 {
     typedef typename Vec<PR>::T T;
     const long long n = FULL ? e.g.V : e.g.Vh;
-    import_tile_kernel<PR, FULL><<<nblk(n, TS), TT, 0, e.st>>>(e.g, (const double2 *)nat, (T *)f0, (T *)f1);
+    import_tile_kernel<PR, FULL><<<nblk(n, TS), TT, 0, e.st>>>(e.g, (const double2 *)nat, (T *)f0, (T *)f1, g5);
 }
 template <int PR, bool FULL>
 static void export_t(const Exec &e, const void *f0, const void *f1, void *nat)
@@ -230,24 +247,17 @@ static void export_t(const Exec &e, const void *f0, const void *f1, void *nat)
     export_tile_kernel<PR, FULL><<<nblk(n, TS), TT, 0, e.st>>>(e.g, (const T *)f0, (const T *)f1, (double2 *)nat);
 }
 
-void import_half(const Exec &e, int prec, const void *nat, void *f)
+void import_half(const Exec &e, int prec, const void *nat, void *f, bool g5)
 {
-    if (prec == P16) {
-        bf16_import_half(e, nat, f);
-        return;
-    }
-    Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + (prec == P32 ? 96 : 192)));
-    if (prec == PDF) import_t<PDF, false>(e, nat, f, nullptr);
-    else if (prec == P64) import_t<P64, false>(e, nat, f, nullptr);
-    else import_t<P32, false>(e, nat, f, nullptr);
+    Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + (prec == P32 ? 96 : prec == P16 ? 48 : 192)));
+    if (prec == PDF) import_t<PDF, false>(e, nat, f, nullptr, g5);
+    else if (prec == P64) import_t<P64, false>(e, nat, f, nullptr, g5);
+    else if (prec == P16) import_t<P16, false>(e, nat, f, nullptr, g5);
+    else import_t<P32, false>(e, nat, f, nullptr, g5);
 }
 
 void export_half(const Exec &e, int prec, const void *f, void *nat)
 {
-    if (prec == P16) {
-        bf16_export_half(e, f, nat);
-        return;
-    }
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + (prec == P32 ? 96 : 192)));
     if (prec == PDF) export_t<PDF, false>(e, f, nullptr, nat);
     else if (prec == P64) export_t<P64, false>(e, f, nullptr, nat);

@@ -90,15 +90,14 @@ void import_links(const Exec &e, const void *U_nat, void *U64[2], void *U32[2], 
 void df64_to_f64(const Exec &e, const void *in, void *out, long long n);
 // BF16 12-real links of one parity from the FP32 ones
 void links_to_bf16(const Exec &e, const void *U32, void *U16);
-// BF16 fields (bf16.cu): conversions (one side BF16), natural half spinors,
-// gamma5 and axpby; the generic launchers below dispatch here for P16
+// BF16 fields (bf16.cu): conversions (one side BF16) and axpby; the generic
+// launchers below dispatch here for P16
 void bf16_convert(const Exec &e, int from, const void *in, int to, void *out);
-void bf16_import_half(const Exec &e, const void *nat, void *f);
-void bf16_export_half(const Exec &e, const void *f, void *nat);
 void bf16_gamma5(const Exec &e, const void *in, void *out);
 void bf16_axpby(const Exec &e, double ar, double ai, const void *x, double br, double bi, void *y, int nfields);
 // natural half spinor [Vh][12] c128 <-> internal field of one parity
-void import_half(const Exec &e, int prec, const void *nat, void *f);
+// (g5: with spins 2 and 3 negated)
+void import_half(const Exec &e, int prec, const void *nat, void *f, bool g5 = false);
 void export_half(const Exec &e, int prec, const void *f, void *nat);
 // natural full spinor [V][12] c128 <-> internal even and odd fields
 void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo);
@@ -189,6 +188,11 @@ struct HopCall {
     void *out2 = nullptr;          // HOP_RECON_RES: the output parity's residual
     double omega;          // HOP_RICH weight
     int nrhs = 1;          // right-hand sides: in, in2, b, out are nrhs consecutive fields
+    // natural output (HOP_K2 in any precision; HOP_FULL and HOP_RECON but in BF16; one
+    // right-hand side): complex-double rows in the place of `out`, those of a full
+    // lattice or of one parity, spins 2 and 3 negated on request
+    void *nat = nullptr;
+    bool nat_full = false, nat_g5 = false;
 };
 void hop(const Exec &e, const HopCall &c);
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
