@@ -239,6 +239,8 @@ HopCall hopcall(lq_ctx *c, int mode, int prec, int pout)
     h.mode = mode;
     h.prec = prec;
     h.pout = pout;
+    // the copies that this and the caller's Cp / Cip make now are read at once
+    h.after = prec == P64 ? c->links64 && c->clover64 : prec == P16 ? c->links16 : true;
     if (prec == P16) need_links16(c);
     if (prec == P64) need_links64(c);
     for (int p = 0; p < 2; p++)

@@ -127,16 +127,17 @@ __device__ __forceinline__ bool last_block_finish(double *partial, int pitch, in
 // (FIN: the last block also finishes the launch's values into out)
 template <typename R, int NJ, bool FIN = false>
 __global__ void __launch_bounds__(RT, 4) multi_dot_kernel(const typename Vec<R>::V *__restrict__ Vb, long long n,
-                                                          const typename Vec<R>::V *__restrict__ w, double *partial,
+                                                          const typename Vec<R>::V *w, double *partial,
                                                           int pitch, int slot0, const double *scale = nullptr,
                                                           double *out = nullptr, unsigned *ticket = nullptr)
 {
     __shared__ R sh[(RT / 32) * 2 * NJ];
+    if (FIN) after_previous();
     R acc[2 * NJ];
 #pragma unroll
     for (int i = 0; i < 2 * NJ; i++) acc[i] = R(0);
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
-        const auto wv = __ldg(w + i);
+        const auto wv = FIN ? w[i] : __ldg(w + i);   // FIN: written by the kernel before (after_previous)
 #pragma unroll
         for (int j = 0; j < NJ; j++) cdot_acc(__ldg(Vb + j * n + i), wv, acc[2 * j], acc[2 * j + 1]);
     }
@@ -196,6 +197,7 @@ __global__ void __launch_bounds__(RT, 4) multi_axpy_fin_kernel(const float4 *__r
 {
     __shared__ float sh[RT / 32];
     __shared__ float csr[256], csi[256];
+    after_previous();
     for (int j = threadIdx.x; j < nv; j += RT) {
         const double2 cj = reinterpret_cast<const double2 *>(c)[j];
         csr[j] = sign * (float)cj.x;
@@ -528,17 +530,16 @@ void multi_axpy_finish(const Exec &e, const void *V, int nv, const RedScratch &r
 {
     Launch L_(e, K_AXPY_F32, (double)e.g.Vh * sp_bytes(P32) * (nv + 2), (double)e.g.Vh * 96 * nv);
     const int blocks = reduction_blocks(e.g);
-    multi_axpy_fin_kernel<<<blocks, RT, 0, e.st>>>((const float4 *)V, nvec(e.g, P32), nv, r.out, (float)sign,
-                                                   (float4 *)y, r.partial, 2 * r.maxv, nrm_slot, r.out, r.ticket, scale,
-                                                   h_mapped);
+    launch_after(e, true, multi_axpy_fin_kernel, blocks, RT, 0, (const float4 *)V, nvec(e.g, P32), nv, r.out, (float)sign,
+                 (float4 *)y, r.partial, 2 * r.maxv, nrm_slot, r.out, r.ticket, scale, h_mapped);
 }
 
 template <int NJ>
 static void dot_fin_launch(const Exec &e, const RedScratch &r, const void *V, long long n, const void *w, int slot0,
                            const double *scale)
 {
-    multi_dot_kernel<float, NJ, true><<<r.blocks, RT, 0, e.st>>>((const float4 *)V, n, (const float4 *)w, r.partial,
-                                                                 2 * r.maxv, slot0, scale, r.out, r.ticket);
+    launch_after(e, true, multi_dot_kernel<float, NJ, true>, r.blocks, RT, 0, (const float4 *)V, n, (const float4 *)w, r.partial,
+                 2 * r.maxv, slot0, scale, r.out, r.ticket);
 }
 
 void multi_dot_finish(const Exec &e, const void *V, int nv, const void *w, const RedScratch &r, const double *scale)

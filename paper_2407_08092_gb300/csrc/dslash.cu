@@ -39,11 +39,11 @@ static_assert(LQ_HOP_THREADS == kHopBlock, "hopping block size");
 // one hop: acc += (1 -+ g_mu) W psi(nb), W = U_mu(x) (SIGN -1) or U_mu(x-mu)^+ (SIGN +1);
 // `bsign` is the fermion boundary factor of this hop
 template <int MU, int SIGN, bool FIRST = false, typename R, typename SV, typename LV>
-__device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *__restrict__ psi, const LV *__restrict__ U,
+__device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *psi, const LV *__restrict__ U,
                                         long long link_site, long long nb, long long stride, R bsign)
 {
     cx<R> p[12];
-    load_spinor(psi, stride, nb, p);
+    load_spinor_rw(psi, stride, nb, p);   // the kernel before wrote it: not through the read-only path (after_previous)
     cx<R> m[9];
     load_link(U, stride, MU, link_site, m);
     hop_apply<MU, SIGN, FIRST>(acc, p, m, bsign);
@@ -311,6 +311,7 @@ __device__ __forceinline__ void hop_site(const Geom &g, const HopArgs<R> &k)
 template <typename R, int MODE, bool NAT>
 __global__ void LQ_HOP_BOUNDS hop_kernel(Geom g, HopArgs<R> k)
 {
+    after_previous();
     hop_site<R, MODE, NAT>(g, k);
 }
 
@@ -321,6 +322,7 @@ __global__ void LQ_HOP_BOUNDS hop_kernel(Geom g, HopArgs<R> k)
 template <typename R, int MODE, bool NAT>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_occ(Geom g, HopArgs<R> k)
 {
+    after_previous();
     hop_site<R, MODE, NAT>(g, k);
 }
 
@@ -355,11 +357,13 @@ __device__ __forceinline__ void hop_site_bf(const Geom &g, const HopArgsBF &k)
 template <int MODE>
 __global__ void LQ_HOP_BOUNDS hop_kernel_bf(Geom g, HopArgsBF k)
 {
+    after_previous();
     hop_site_bf<MODE, false>(g, k);
 }
 // K2 with natural output: held to the registers of the plain one (104 without the bound)
 __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_bf_nat(Geom g, HopArgsBF k)
 {
+    after_previous();
     hop_site_bf<HOP_K2, true>(g, k);
 }
 
@@ -393,10 +397,10 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
     if constexpr (MODE == HOP_K2)
         if (c.nat) {
-            hop_kernel_bf_nat<<<blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.st>>>(e.g, k);
+            launch_after(e, c.after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
             return;
         }
-    hop_kernel_bf<MODE><<<blocks, LQ_HOP_THREADS, 0, e.st>>>(e.g, k);
+    launch_after(e, c.after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
 }
 
 // The batched hop over the right-hand sides of several lattices of different
@@ -654,14 +658,6 @@ __device__ __forceinline__ void herm6_fma_df(Ld ld, const cx<df64> x[6], cx<df64
 constexpr int kDfPsi = 0;        // the neighbour's 12 components
 constexpr int kDfLink = 12;      // two buffers of 9 link entries
 constexpr int kDfVecs = 30;
-__device__ __forceinline__ void copy_async(float4 *dst, const df2 *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 // a use of v that the compiler keeps before the copies that follow
 __device__ __forceinline__ void used(cx<df64> v) { asm volatile("" ::"f"(v.re.hi), "f"(v.re.lo), "f"(v.im.hi), "f"(v.im.lo) : "memory"); }
 
@@ -892,6 +888,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(cons
                                                                 const __grid_constant__ HopArgs<df64> k)
 {
     extern __shared__ float4 df_stage[];
+    after_previous();
     const unsigned sb = blockIdx.x / (unsigned)k.nrhs;
     long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
     int nv = 0;
@@ -948,7 +945,7 @@ static void launch_hop(const Exec &e, const HopCall &c)
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
         auto launch = [&](auto kernel) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            kernel<<<blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.st>>>(e.g, k);
+            launch_after(e, c.after, kernel, blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.g, k);
         };
         if constexpr (nat_mode(MODE))
             if (c.nat) return launch(hop_df_kernel<MODE, true>);
@@ -970,9 +967,9 @@ static void launch_hop(const Exec &e, const HopCall &c)
             auto launch = [&](auto nat) {
                 constexpr bool NAT = decltype(nat)::value;
                 if constexpr (std::is_same<R, float>::value && (MODE == HOP_K2 || MODE == HOP_RICH))
-                    hop_kernel_occ<R, MODE, NAT><<<blocks, threads, sm, e.st>>>(e.g, kr);
+                    launch_after(e, c.after, hop_kernel_occ<R, MODE, NAT>, blocks, threads, sm, e.g, kr);
                 else
-                    hop_kernel<R, MODE, NAT><<<blocks, threads, sm, e.st>>>(e.g, kr);
+                    launch_after(e, c.after, hop_kernel<R, MODE, NAT>, blocks, threads, sm, e.g, kr);
             };
             if constexpr (nat_mode(MODE)) {
                 if (c.nat) launch(std::true_type());

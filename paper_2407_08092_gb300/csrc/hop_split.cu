@@ -9,8 +9,10 @@
 //      whose entries it loaded before step 1.
 // The operations and their order are those of the one-thread kernels.
 //
-// lq_apply of D_S in us, twelve threads against one, at 2048 sites a parity: df64
-// 18.8 / 39.3, FP32 18.6 / 20.7, FP64 37 / 88, BF16 18.8 / 20.8; at 9216: 29 / 43,
+// lq_apply of D_S in us, twelve threads against one and before the launches
+// overlapped (launch_after: df64 at 2048 sites 18.8 -> 14.4), at 2048 sites a
+// parity: df64 18.8 / 39.3, FP32 18.6 / 20.7, FP64 37 / 88, BF16 18.8 / 20.8; at
+// 9216: 29 / 43,
 // 18.7 / 24.8, 63 / 88, 20.8 / 24.9; at 24576: 58 / 56, 31.0 / 29.0, 162 / 132,
 // 32 / 27.  The larger the lattice, the less it needs the extra threads, which
 // pass the eight half spinors through shared memory and idle while others work.
@@ -128,7 +130,7 @@ __device__ __forceinline__ void half_hop(const SV *psi, const LV *U, long long s
 {
     constexpr int MU = D >> 1, SIGN = (D & 1) ? +1 : -1;
     cx<R> p[12], m[9], h[6];
-    load_spinor(psi, st, nb, p);
+    load_spinor_rw(psi, st, nb, p);
     load_link(U, st, MU, link, m);
     project<MU, SIGN>(p, h);
     transport<SIGN>(m, h, sign, u);
@@ -167,10 +169,10 @@ struct HalfHop<df64, df2, df2> {
         for (int k = 0; k < 9; k++) m[k] = df2_cx(ldg(Um + k * st));
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            h[a] = df2_cx(ldg(psi + a * st + nb));
-            dl_cadd(h[a], rot_i(df2_cx(ldg(psi + (d < 4 ? 9 + a : 6 + a) * st + nb)), qa));
-            h[3 + a] = df2_cx(ldg(psi + (3 + a) * st + nb));
-            dl_cadd(h[3 + a], rot_i(df2_cx(ldg(psi + (d < 4 ? 6 + a : 9 + a) * st + nb)), qb));
+            h[a] = df2_cx(psi[a * st + nb]);
+            dl_cadd(h[a], rot_i(df2_cx(psi[(d < 4 ? 9 + a : 6 + a) * st + nb]), qa));
+            h[3 + a] = df2_cx(psi[(3 + a) * st + nb]);
+            dl_cadd(h[3 + a], rot_i(df2_cx(psi[(d < 4 ? 6 + a : 9 + a) * st + nb]), qb));
         }
 #pragma unroll
         for (int a = 0; a < 3; a++) {
@@ -220,6 +222,7 @@ __global__ void __launch_bounds__(kSplitThreads, std::is_same<R, df64>::value ? 
 {
     typedef HalfHop<R, SV, LV> H;
     extern __shared__ __align__(16) unsigned char split_sm[];
+    after_previous();
     cx<R> *U = reinterpret_cast<cx<R> *>(split_sm);        // [direction][6][site]
     cx<R> *X = U + 48 * kSplitSites;                       // [12][site]: what the clover blocks multiply
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -332,7 +335,7 @@ static void launch_split(const Exec &e, const HopCall &c)
     k.nat.full = c.nat_full;
     k.nat.flip = c.nat_g5 ? 0x80000000u : 0u;
     const unsigned blocks = (unsigned)((e.g.Vh + kSplitSites - 1) / kSplitSites) * (unsigned)c.nrhs;
-    hop_split_kernel<R, MODE, SV, LV, CV><<<blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.st>>>(e.g, k);
+    launch_after(e, c.after, hop_split_kernel<R, MODE, SV, LV, CV>, blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.g, k);
 }
 
 bool hop_split(const Exec &e, const HopCall &c)

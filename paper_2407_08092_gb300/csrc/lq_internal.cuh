@@ -596,6 +596,13 @@ __device__ __forceinline__ void load_link(const double2 *__restrict__ U, long lo
         m[k] = {t.x, t.y};
     }
 }
+// SU(3): third row = conj(row0 x row1)
+__device__ __forceinline__ void third_row(cx<float> m[9])
+{
+    m[6] = cconj(cmul(m[1], m[5]) - cmul(m[2], m[4]));
+    m[7] = cconj(cmul(m[2], m[3]) - cmul(m[0], m[5]));
+    m[8] = cconj(cmul(m[0], m[4]) - cmul(m[1], m[3]));
+}
 template <typename P>   // const float4 (cached) or const F4S (read once)
 __device__ __forceinline__ void load_link_f(const P *__restrict__ U, long long stride, int mu, long long s,
                                             cx<float> m[9])
@@ -606,10 +613,7 @@ __device__ __forceinline__ void load_link_f(const P *__restrict__ U, long long s
         m[2 * k] = {t.x, t.y};
         m[2 * k + 1] = {t.z, t.w};
     }
-    // SU(3): third row = conj(row0 x row1)
-    m[6] = cconj(cmul(m[1], m[5]) - cmul(m[2], m[4]));
-    m[7] = cconj(cmul(m[2], m[3]) - cmul(m[0], m[5]));
-    m[8] = cconj(cmul(m[0], m[4]) - cmul(m[1], m[3]));
+    third_row(m);
 }
 __device__ __forceinline__ void load_link(const float4 *__restrict__ U, long long stride, int mu, long long s,
                                           cx<float> m[9])
@@ -712,6 +716,29 @@ __device__ __forceinline__ Coords cb_coords(const Geom &g, long long s, int pari
     c.t = (int)(r2 / g.L[2]);
     c.x = 2 * xh + ((c.y + c.z + c.t + parity) & 1);
     return c;
+}
+
+// asynchronous 16-byte copies to shared memory, in groups that complete in order
+__device__ __forceinline__ void copy_async(float4 *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// First statement of a kernel that launch_after (lq_kernels.h) starts while the
+// kernel before it still runs: waits until that one has finished and its writes
+// are visible, then lets the kernel after this one be brought in likewise.  A
+// kernel is brought in only when all blocks of the one before have passed this
+// point, so what earlier kernels wrote is there in any case; what the one before
+// wrote is read with plain loads, since the compiler may move a read-only load
+// (__ldg) across the wait.
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------

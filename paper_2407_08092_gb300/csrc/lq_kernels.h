@@ -76,6 +76,28 @@ struct Launch {
     }
 };
 
+// Launches a kernel that begins with after_previous() behind another kernel of
+// the same call: its blocks take their places while the other one drains, which
+// saves most of the gap between two dependent launches.  Plainly (after = false),
+// when all that is on the stream has finished: for the first kernel of a call and
+// behind a kernel that wrote what this one reads through the read-only path.
+template <typename... P, typename... A>
+inline void launch_after(const Exec &e, bool after, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                         const A &...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = after ? 1 : 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = e.st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Bytes of one internal per-parity spinor field in a precision.
 inline size_t spinor_bytes(const Geom &g, int prec)
 {
@@ -193,6 +215,7 @@ struct HopCall {
     // lattice or of one parity, spins 2 and 3 negated on request
     void *nat = nullptr;
     bool nat_full = false, nat_g5 = false;
+    bool after = true;     // launch_after: not behind a kernel that made links or clover blocks of this call
 };
 void hop(const Exec &e, const HopCall &c);
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
