@@ -1028,6 +1028,7 @@ void group_setup(lq_group *G, const std::vector<int> &nrhs, int m)
         d.off = mf;
         d.fs = fs;
         d.nrhs = nrhs[l];
+        d.first = N;
         mf += nrhs[l] * fs;
         N += nrhs[l];
         maxfs = fs > maxfs ? fs : maxfs;
@@ -1077,7 +1078,7 @@ void group_setup(lq_group *G, const std::vector<int> &nrhs, int m)
     k.active = (int *)galloc(G, sizeof(int) * N);
     k.kused = (int *)galloc(G, sizeof(int) * N);
     k.nanflag = (int *)galloc(G, sizeof(int));
-    k.scale = (double *)galloc(G, sizeof(double) * N);
+    k.scale = (double *)galloc(G, sizeof(double) * (size_t)N * (m + 1));
     k.est = (double *)galloc(G, sizeof(double) * N);
     k.target = (double *)galloc(G, sizeof(double) * N);
     G->mbr.assign(M, BatchRed{});
@@ -1099,14 +1100,16 @@ void group_setup(lq_group *G, const std::vector<int> &nrhs, int m)
     G->tune.tuned = false;
 }
 
-// out = D_S in for every system (two persistent launches over the work table)
-void group_schur(lq_group *G, const void *in, void *out)
+// out = D_S (s in) for every system (two persistent launches over the work table),
+// s its normaliser of basis vector k (k < 0: 1)
+void group_schur(lq_group *G, const void *in, void *out, int k = -1)
 {
     Exec e = gexec(G);
-    hop_group(e, HOP_K1, G->desc, G->tiles, G->ntiles, G->tune.grid, G->tune.spt, G->tune.rpt, in, nullptr, G->T,
-              G->k1_bytes, G->k1_flops);
-    hop_group(e, HOP_K2, G->desc, G->tiles, G->ntiles, G->tune.grid, G->tune.spt, G->tune.rpt, G->T, in, out,
-              G->k2_bytes, G->k2_flops);
+    const double *s = k < 0 ? nullptr : G->ks.scale + k;
+    hop_group(e, HOP_K1, G->desc, G->tiles, G->ntiles, G->tune.grid, G->tune.spt, G->tune.rpt, in, nullptr, G->T, s,
+              G->m + 1, G->k1_bytes, G->k1_flops);
+    hop_group(e, HOP_K2, G->desc, G->tiles, G->ntiles, G->tune.grid, G->tune.spt, G->tune.rpt, G->T, in, out, s,
+              G->m + 1, G->k2_bytes, G->k2_flops);
 }
 
 void group_set_blas(lq_group *G, int blocks)
@@ -1193,9 +1196,9 @@ void group_tune(lq_group *G)
 // One cycle of batched GMRES(m) in FP32 on D_S (Algorithm 2 for each system), in
 // three kinds of segment, each a fixed launch sequence without host
 // synchronisation:
-//   start:  r = B - D_S X, beta = ||r||, g = beta e_1, V_0 = r / beta
+//   start:  V_0 = B - D_S X, beta = ||V_0||, g = beta e_1, v_0 = V_0 / beta
 //   steps:  Arnoldi steps [k0, k1): w = D_S v_k, one Gram-Schmidt pass with the
-//           new norm fused, Givens on the device, v_{k+1}
+//           new norm fused, Givens on the device, V_{k+1} = w and its normaliser
 //   finish: y = R^{-1} g, X += V y
 static constexpr int BATCH_SEG = 4;   // Arnoldi steps per segment
 
@@ -1207,7 +1210,6 @@ void group_start(lq_group *G)
     bnorm(e, P32, G->S, G->V, G->N, G->br, 0);
     bfinish(e, G->br, G->N, 0, 1);
     ks_init(e, G->ks, G->br.out, G->br.pitch);
-    bscale(e, G->S, G->V, G->ks.scale, G->V, G->N);
 }
 
 void group_steps(lq_group *G, int k0, int k1)
@@ -1215,14 +1217,14 @@ void group_steps(lq_group *G, int k0, int k1)
     Exec e = gexec(G);
     auto Vj = [&](int j) { return (char *)G->V + (size_t)j * G->mf * 16; };
     for (int k = k0; k < k1; k++) {
-        group_schur(G, Vj(k), Vj(k + 1));
+        group_schur(G, Vj(k), Vj(k + 1), k);
         const int nv = k + 1;
         bdot(e, G->S, G->V, G->mf, nv, Vj(k + 1), G->N, G->br, 0);
         bfinish(e, G->br, G->N, 0, nv);
-        baxpy(e, G->S, G->V, G->mf, nv, G->br.out, G->br.pitch / 2, -1, Vj(k + 1), G->N, &G->br, nv);
+        baxpy(e, G->S, G->V, G->mf, nv, G->br.out, G->br.pitch / 2, -1, Vj(k + 1), G->N, &G->br, nv, G->ks.scale,
+              G->m + 1);
         bfinish(e, G->br, G->N, nv, 1);
         ks_step(e, G->ks, k, 1, G->br.out, G->br.pitch);
-        bscale(e, G->S, Vj(k + 1), G->ks.scale, Vj(k + 1), G->N);
     }
 }
 

@@ -106,15 +106,17 @@ template <bool NORM>
 __global__ void __launch_bounds__(BT, 4) baxpy_kernel(const float4 *__restrict__ V, long long vjs,
                                                       const longlong2 *seg, long long n, int nv,
                                                       const double2 *__restrict__ c, int cstride, float sign,
-                                                      float4 *y, double *partial, int pitch, int slot)
+                                                      float4 *y, double *partial, int pitch, int slot,
+                                                      const double *__restrict__ scale, int sstride)
 {
     __shared__ float csr[256], csi[256];
     __shared__ float sh[BT / 32];
     const int r = blockIdx.y;
     for (int j = threadIdx.x; j < nv; j += BT) {
         const double2 cj = c[(long long)r * cstride + j];
-        csr[j] = sign * (float)cj.x;
-        csi[j] = sign * (float)cj.y;
+        const double sj = scale ? scale[(long long)r * sstride + j] : 1.0;
+        csr[j] = sign * (float)(sj * sj * cj.x);
+        csi[j] = sign * (float)(sj * sj * cj.y);
     }
     __syncthreads();
     long long off, len;
@@ -226,24 +228,6 @@ __global__ void __launch_bounds__(BT) bfinish_kernel(const double *__restrict__ 
     }
 }
 
-// y_r = s_r x_r (FP32 fields, device scale per system)
-__global__ void __launch_bounds__(BT) bscale_kernel(const float4 *x, const longlong2 *seg, long long n,
-                                                    const double *s, float4 *y)
-{
-    const int r = blockIdx.y;
-    long long off, len;
-    seg_of(seg, n, r, off, len);
-    const float f = (float)s[r];
-    for (long long i = blockIdx.x * (long long)BT + threadIdx.x; i < len; i += (long long)gridDim.x * BT) {
-        float4 v = x[off + i];
-        v.x *= f;
-        v.y *= f;
-        v.z *= f;
-        v.w *= f;
-        y[off + i] = v;
-    }
-}
-
 // y_r = x_r - y_r (FP32 fields)
 __global__ void __launch_bounds__(BT) bxmy_kernel(const float4 *__restrict__ x, const longlong2 *seg, long long n,
                                                   float4 *y)
@@ -274,7 +258,10 @@ __device__ __forceinline__ double cd_abs(cdbl a) { return hypot(a.re, a.im); }
 
 // Start of a cycle: beta_r = sqrt(nrm2_r); g_r = beta e_1; the cycle of a
 // right-hand side whose residual already meets its target (or is 0) stays
-// inactive.  scale_r = 1/beta (0 when inactive).
+// inactive.  scale_r0 = 1/beta (0 when inactive): the basis is stored
+// unnormalised, v_j = scale_j V_j, which saves the pass that would scale each new
+// vector; D_S takes the factor on its input (hop_group), so that ||V_j|| stays the
+// size of a Hessenberg entry, and a system that has left the cycle multiplies by 0.
 __global__ void ks_init_kernel(int N, int m, const double *nrm2, int nstride, const double *target, double2 *g,
                                int *active, int *kused, double *scale, double *est)
 {
@@ -285,7 +272,7 @@ __global__ void ks_init_kernel(int N, int m, const double *nrm2, int nstride, co
     const bool on = beta > target[r] && beta > 0.0 && isfinite(beta);
     active[r] = on ? 1 : 0;
     kused[r] = 0;
-    scale[r] = on ? 1.0 / beta : 0.0;
+    scale[(long long)r * (m + 1)] = on ? 1.0 / beta : 0.0;
     est[r] = beta;
 }
 
@@ -295,15 +282,17 @@ __global__ void ks_init_kernel(int N, int m, const double *nrm2, int nstride, co
 // ||w||^2 in slot k+1.
 // Rotates the new Hessenberg column, updates g, and decides whether the cycle
 // continues for this right-hand side (residual estimate above target, no
-// breakdown).  scale_r = 1/h_{k+1,k} normalises the next basis vector.
+// breakdown).  The dots are those of the stored vectors, (V_j, w): h_jk takes
+// scale_j.  scale_{k+1} = 1/h_{k+1,k} normalises the next basis vector.
 __global__ void ks_step_kernel(int N, int m, int k, int passes, const double *dots, int dstride, const double *target,
                                double2 *H, double *cs, double2 *sn, double2 *g, int *active, int *kused,
                                double *scale, double *est, int *nanflag)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
+    double *sr = scale + (long long)r * (m + 1);
     if (!active[r]) {
-        scale[r] = 0.0;
+        sr[k + 1] = 0.0;
         return;
     }
     const double *d = dots + (long long)r * dstride;
@@ -314,27 +303,33 @@ __global__ void ks_step_kernel(int N, int m, int k, int passes, const double *do
     const double hk1 = sqrt(d[2 * (passes == 2 ? 2 * k + 2 : k + 1)]);
     double colnorm2 = hk1 * hk1;
     for (int j = 0; j <= k; j++) {
-        const double re = d[2 * j] + (passes == 2 ? d[2 * (k + 1 + j)] : 0.0);
-        const double im = d[2 * j + 1] + (passes == 2 ? d[2 * (k + 1 + j) + 1] : 0.0);
+        const double re = sr[j] * (d[2 * j] + (passes == 2 ? d[2 * (k + 1 + j)] : 0.0));
+        const double im = sr[j] * (d[2 * j + 1] + (passes == 2 ? d[2 * (k + 1 + j) + 1] : 0.0));
         Hr[(long long)k * (m + 1) + j] = make_double2(re, im);
         colnorm2 += re * re + im * im;
     }
     if (!isfinite(colnorm2)) {
         atomicAdd(nanflag, 1);
         active[r] = 0;
-        scale[r] = 0.0;
+        sr[k + 1] = 0.0;
         return;
     }
-    // previous rotations on the new column
-    for (int i = 0; i < k; i++) {
-        const double2 a2 = Hr[(long long)k * (m + 1) + i], b2 = Hr[(long long)k * (m + 1) + i + 1];
-        const cdbl a = {a2.x, a2.y}, b = {b2.x, b2.y}, s = {snr[i].x, snr[i].y};
-        const cdbl sb = cd_mul(s, b), sca = cd_mul(cd_conj(s), a);
-        Hr[(long long)k * (m + 1) + i] = make_double2(csr[i] * a.re + sb.re, csr[i] * a.im + sb.im);
-        Hr[(long long)k * (m + 1) + i + 1] = make_double2(-sca.re + csr[i] * b.re, -sca.im + csr[i] * b.im);
+    // previous rotations on the new column, the entry they pass on in a register
+    cdbl a;
+    {
+        const double2 a2 = Hr[(long long)k * (m + 1)];
+        a = {a2.x, a2.y};
     }
-    const double2 a2 = Hr[(long long)k * (m + 1) + k];
-    const cdbl a = {a2.x, a2.y}, b = {hk1, 0.0};
+#pragma unroll 4
+    for (int i = 0; i < k; i++) {
+        const double2 b2 = Hr[(long long)k * (m + 1) + i + 1], s2 = snr[i];
+        const cdbl b = {b2.x, b2.y}, s = {s2.x, s2.y};
+        const double ci = csr[i];
+        const cdbl sb = cd_mul(s, b), sca = cd_mul(cd_conj(s), a);
+        Hr[(long long)k * (m + 1) + i] = make_double2(ci * a.re + sb.re, ci * a.im + sb.im);
+        a = {-sca.re + ci * b.re, -sca.im + ci * b.im};
+    }
+    const cdbl b = {hk1, 0.0};
     const double t = sqrt(a.re * a.re + a.im * a.im + hk1 * hk1);
     double c;
     cdbl s;
@@ -362,12 +357,13 @@ __global__ void ks_step_kernel(int N, int m, int k, int passes, const double *do
     const bool breakdown = hk1 <= 1e-14 * sqrt(colnorm2);
     const bool go = !breakdown && e > target[r] && k + 1 < m;
     active[r] = go ? 1 : 0;
-    scale[r] = go ? 1.0 / hk1 : 0.0;
+    sr[k + 1] = go ? 1.0 / hk1 : 0.0;
 }
 
-// y_r = R^{-1} g over the kused_r columns; zeros beyond (coefficients of x += V y)
+// y_r = R^{-1} g over the kused_r columns, zeros beyond, times the basis vectors'
+// normalisers: the coefficients of x += V y
 __global__ void ks_solve_kernel(int N, int m, const double2 *H, const double2 *g, const int *kused, double2 *y,
-                                int ystride)
+                                int ystride, const double *scale)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
@@ -388,6 +384,10 @@ __global__ void ks_solve_kernel(int N, int m, const double2 *H, const double2 *g
         const double den = hii.re * hii.re + hii.im * hii.im;
         const cdbl q = cd_mul(acc, cd_conj(hii));
         yr[i] = make_double2(q.re / den, q.im / den);
+    }
+    for (int j = 0; j < n; j++) {
+        const double sj = scale[(long long)r * (m + 1) + j];
+        yr[j] = make_double2(sj * yr[j].x, sj * yr[j].y);
     }
 }
 
@@ -430,17 +430,17 @@ void bdot(const Exec &e, const Segs &S, const void *V, long long vjs, int nv, co
 }
 
 void baxpy(const Exec &e, const Segs &S, const void *V, long long vjs, int nv, const double *c, int cstride,
-           int sign, void *y, int N, BatchRed *br, int slot)
+           int sign, void *y, int N, BatchRed *br, int slot, const double *scale, int sstride)
 {
     Launch L_(e, K_AXPY_F32, S.sites * 96.0 * (nv + 2), S.sites * 96 * nv);
     const int blocks = br ? br->blocks : S.blocks;
     const dim3 grid(blocks, N);
     if (br)
         baxpy_kernel<true><<<grid, BT, 0, e.st>>>((const float4 *)V, vjs, S.seg, S.n, nv, (const double2 *)c,
-                                                  cstride, (float)sign, (float4 *)y, br->partial, br->pitch, slot);
+                                                  cstride, (float)sign, (float4 *)y, br->partial, br->pitch, slot, scale, sstride);
     else
         baxpy_kernel<false><<<grid, BT, 0, e.st>>>((const float4 *)V, vjs, S.seg, S.n, nv, (const double2 *)c,
-                                                   cstride, (float)sign, (float4 *)y, nullptr, 0, slot);
+                                                   cstride, (float)sign, (float4 *)y, nullptr, 0, slot, scale, sstride);
 }
 
 void bnorm(const Exec &e, int prec, const Segs &S, const void *w, int N, BatchRed &br, int slot)
@@ -459,12 +459,6 @@ void bfinish(const Exec &e, BatchRed &br, int N, int first, int count)
     Launch L_(e, K_FINISH, (double)N * br.blocks * 2 * count * 8.0);
     bfinish_kernel<<<dim3(2 * count, N), BT, 0, e.st>>>(br.partial, br.blocks, br.pitch, 2 * first, br.out,
                                                         br.pitch);
-}
-
-void bscale(const Exec &e, const Segs &S, const void *x, const double *s, void *y, int N)
-{
-    Launch L_(e, K_AXPY_F32, S.sites * 192.0);
-    bscale_kernel<<<dim3(S.blocks, N), BT, 0, e.st>>>((const float4 *)x, S.seg, S.n, s, (float4 *)y);
 }
 
 void bxmy(const Exec &e, const Segs &S, const void *x, void *y, int N)
@@ -490,7 +484,7 @@ void ks_step(const Exec &e, const KState &k, int step, int passes, const double 
 void ks_solve(const Exec &e, const KState &k)
 {
     Launch L_(e, K_FINISH, 0.0);
-    ks_solve_kernel<<<(k.N + 31) / 32, 32, 0, e.st>>>(k.N, k.m, k.H, k.g, k.kused, k.y, k.m);
+    ks_solve_kernel<<<(k.N + 31) / 32, 32, 0, e.st>>>(k.N, k.m, k.H, k.g, k.kused, k.y, k.m, k.scale);
 }
 
 int batch_blocks(long long maxlen, int N) { return bblocks(maxlen, N); }

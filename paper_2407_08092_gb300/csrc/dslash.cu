@@ -94,7 +94,8 @@ __device__ __forceinline__ void store_nat(const NatOut &o, double2 *tile, const 
 
 // SV, LV, CV: storage vectors of the spinors, links and clover blocks (the same
 // type for FP64, FP32 and df64; BF16 spinors and links with FP32 clover)
-template <typename R, int MODE, bool NAT = false, typename SV, typename LV, typename CV>
+// (SCALED, for K1 and K2: omega is a factor of the input field)
+template <typename R, int MODE, bool NAT = false, bool SCALED = false, typename SV, typename LV, typename CV>
 __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV *Uin, const CV *clov, R omega,
                                          const SV *in, const SV *in2, const SV *bv, SV *out, long long s,
                                          const Coords &c, const CV *clov2 = nullptr, SV *out2 = nullptr,
@@ -145,7 +146,7 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
     cx<R> v[12];
     if (MODE == HOP_K1) {
 #pragma unroll
-        for (int i = 0; i < 12; i++) acc[i] = R(-0.5) * acc[i];
+        for (int i = 0; i < 12; i++) acc[i] = (SCALED ? R(-0.5) * omega : R(-0.5)) * acc[i];
         clover_apply<R>(clov, st, s, acc, v);
     } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL || MODE == HOP_RES) {
         cx<R> x[12];
@@ -153,7 +154,7 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
         clover_apply<R>(clov, st, s, x, v);
         const R f = (MODE == HOP_FULL || MODE == HOP_RES) ? R(-0.5) : R(0.5);
 #pragma unroll
-        for (int i = 0; i < 12; i++) v[i] = v[i] + f * acc[i];
+        for (int i = 0; i < 12; i++) v[i] = (SCALED ? omega * v[i] : v[i]) + f * acc[i];
         if (MODE == HOP_RICH) {
             cx<R> bb[12];
             load_spinor(bv, st, s, bb);
@@ -213,7 +214,7 @@ template <int MODE>
 __device__ __forceinline__ void hop_body2(const Geom &g, const float4 *Uout, const float4 *Uin, const float4 *clov,
                                           const float4 *in0, const float4 *in1, const float4 *in20,
                                           const float4 *in21, float4 *out0, float4 *out1, bool two, long long s,
-                                          const Coords &c)
+                                          const Coords &c, float sc0, float sc1)
 {
     const long long st = g.stride;
     cx<float> a0[12], a1[12];
@@ -253,12 +254,12 @@ __device__ __forceinline__ void hop_body2(const Geom &g, const float4 *Uout, con
     cx<float> v[12], x[12];
     if (MODE == HOP_K1) {
 #pragma unroll
-        for (int i = 0; i < 12; i++) a0[i] = -0.5f * a0[i];
+        for (int i = 0; i < 12; i++) a0[i] = -0.5f * sc0 * a0[i];
         clover_apply<float>(clov, st, s, a0, v);
         store_spinor(out0, st, s, v);
         if (two) {
 #pragma unroll
-            for (int i = 0; i < 12; i++) a1[i] = -0.5f * a1[i];
+            for (int i = 0; i < 12; i++) a1[i] = -0.5f * sc1 * a1[i];
             clover_apply<float>(clov, st, s, a1, v);
             store_spinor(out1, st, s, v);
         }
@@ -266,13 +267,13 @@ __device__ __forceinline__ void hop_body2(const Geom &g, const float4 *Uout, con
         load_spinor_rw(in20, st, s, x);
         clover_apply<float>(clov, st, s, x, v);
 #pragma unroll
-        for (int i = 0; i < 12; i++) v[i] = v[i] + 0.5f * a0[i];
+        for (int i = 0; i < 12; i++) v[i] = sc0 * v[i] + 0.5f * a0[i];
         store_spinor(out0, st, s, v);
         if (two) {
             load_spinor_rw(in21, st, s, x);
             clover_apply<float>(clov, st, s, x, v);
 #pragma unroll
-            for (int i = 0; i < 12; i++) v[i] = v[i] + 0.5f * a1[i];
+            for (int i = 0; i < 12; i++) v[i] = sc1 * v[i] + 0.5f * a1[i];
             store_spinor(out1, st, s, v);
         }
     }
@@ -413,13 +414,20 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
 #else
 #define LQ_GROUP_BOUNDS __launch_bounds__(LQ_HOP_THREADS)
 #endif
+// the factor of system r's input field (null: 1)
+__device__ __forceinline__ float scale_of(const double *scale, int stride, int r)
+{
+    return scale ? (float)scale[(long long)r * stride] : 1.0f;
+}
 template <int MODE, int RPT>
 __global__ void LQ_GROUP_BOUNDS hop_group_kernel(const LatDesc *__restrict__ d,
                                                                    const int4 *__restrict__ tiles, int ntiles,
-                                                                   const float4 *in, const float4 *in2, float4 *out)
+                                                                   const float4 *in, const float4 *in2, float4 *out,
+                                                                   const double *scale, int sstride)
 {
     constexpr int pout = MODE == HOP_K1 ? 1 : 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int t0 = (int)((long long)ntiles * blockIdx.x / gridDim.x), t1 = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
+    for (int t = t0; t < t1; t++) {
         const int4 w = __ldg(tiles + t);
         const LatDesc *L = d + w.x;
         const Geom g = L->g;
@@ -428,15 +436,17 @@ __global__ void LQ_GROUP_BOUNDS hop_group_kernel(const LatDesc *__restrict__ d,
         if (s >= g.Vh || r >= L->nrhs) continue;
         const Coords c = cb_coords(g, s, pout);
         const long long o = L->off + r * L->fs;
+        const float sc = scale_of(scale, sstride, L->first + r);
         if (RPT == 1) {
-            hop_body<float, MODE>(g, L->U[pout], L->U[1 - pout], L->clov[pout], 0.0f, in + o,
-                                  in2 ? in2 + o : nullptr, (const float4 *)nullptr, out + o, s, c);
+            hop_body<float, MODE, false, true>(g, L->U[pout], L->U[1 - pout], L->clov[pout], sc, in + o,
+                                               in2 ? in2 + o : nullptr, (const float4 *)nullptr, out + o, s, c);
         } else {
             // the second right-hand side, when it exists (else the first is read twice, stored once)
             const bool two = r + 1 < L->nrhs;
             const long long o1 = two ? o + L->fs : o;
             hop_body2<MODE>(g, L->U[pout], L->U[1 - pout], L->clov[pout], in + o, in + o1,
-                            in2 ? in2 + o : nullptr, in2 ? in2 + o1 : nullptr, out + o, out + o1, two, s, c);
+                            in2 ? in2 + o : nullptr, in2 ? in2 + o1 : nullptr, out + o, out + o1, two, s, c, sc,
+                            two ? scale_of(scale, sstride, L->first + r + 1) : 0.0f);
         }
     }
 }
@@ -500,7 +510,8 @@ __device__ __forceinline__ void tile_hop(cx<float> acc[12], const float4 *__rest
 template <int MODE, int S>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, 5) hop_tile_kernel(const LatDesc *__restrict__ d,
                                                                      const int4 *__restrict__ tiles, int ntiles,
-                                                                     const float4 *in, const float4 *in2, float4 *out)
+                                                                     const float4 *in, const float4 *in2, float4 *out,
+                                                                     const double *scale, int sstride)
 {
     static_assert(MODE == HOP_K1 || MODE == HOP_K2, "K1 or K2");
     constexpr int R = LQ_HOP_THREADS / S;   // right-hand-side lanes
@@ -586,16 +597,17 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 5) hop_tile_kernel(const LatDe
             tile_hop<3, -1>(acc, pin, st, tile_nb[6 * S + x], tile_sm, S, x, tile_bc[x]);
             tile_hop<3, +1>(acc, pin, st, tile_nb[7 * S + x], tile_sm, S, x, tile_bc[S + x]);
             cx<float> v[12];
+            const float sc = scale_of(scale, sstride, L->first + r);
             if (MODE == HOP_K1) {
 #pragma unroll
-                for (int i = 0; i < 12; i++) acc[i] = -0.5f * acc[i];
+                for (int i = 0; i < 12; i++) acc[i] = -0.5f * sc * acc[i];
                 tile_clover(tile_sm, S, x, acc, v);
             } else {
                 cx<float> xs[12];
                 load_spinor_rw(in2 + o, st, s, xs);
                 tile_clover(tile_sm, S, x, xs, v);
 #pragma unroll
-                for (int i = 0; i < 12; i++) v[i] = v[i] + 0.5f * acc[i];
+                for (int i = 0; i < 12; i++) v[i] = sc * v[i] + 0.5f * acc[i];
             }
             store_spinor(out + o, st, s, v);
         }
@@ -1046,7 +1058,8 @@ int hop_group_resident(int rpt, int spt)
 }
 
 void hop_group(const Exec &e, int mode, const LatDesc *desc, const int4 *tiles, int ntiles, int grid, int spt,
-               int rpt, const void *in, const void *in2, void *out, double bytes, double flops)
+               int rpt, const void *in, const void *in2, void *out, const double *scale, int sstride, double bytes,
+               double flops)
 {
     Launch L_(e, mode == HOP_K1 ? K_HOP_K1_F32 : K_HOP_K2_F32, bytes, flops);
     const dim3 block(spt, LQ_HOP_THREADS / spt);
@@ -1055,18 +1068,18 @@ void hop_group(const Exec &e, int mode, const LatDesc *desc, const int4 *tiles, 
     if (rpt == 0) {   // staged links and clover, every right-hand side of the tile's lattice
         const size_t sm = tile_smem(spt);
         if (spt == 64) {
-            if (mode == HOP_K1) hop_tile_kernel<HOP_K1, 64><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o);
-            else hop_tile_kernel<HOP_K2, 64><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o);
+            if (mode == HOP_K1) hop_tile_kernel<HOP_K1, 64><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
+            else hop_tile_kernel<HOP_K2, 64><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
         } else {
-            if (mode == HOP_K1) hop_tile_kernel<HOP_K1, 32><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o);
-            else hop_tile_kernel<HOP_K2, 32><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o);
+            if (mode == HOP_K1) hop_tile_kernel<HOP_K1, 32><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
+            else hop_tile_kernel<HOP_K2, 32><<<grid, block, sm, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
         }
         return;
     }
-    if (mode == HOP_K1 && rpt == 2) hop_group_kernel<HOP_K1, 2><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o);
-    else if (mode == HOP_K1) hop_group_kernel<HOP_K1, 1><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o);
-    else if (rpt == 2) hop_group_kernel<HOP_K2, 2><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o);
-    else hop_group_kernel<HOP_K2, 1><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o);
+    if (mode == HOP_K1 && rpt == 2) hop_group_kernel<HOP_K1, 2><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
+    else if (mode == HOP_K1) hop_group_kernel<HOP_K1, 1><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
+    else if (rpt == 2) hop_group_kernel<HOP_K2, 2><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
+    else hop_group_kernel<HOP_K2, 1><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
 }
 
 void hop(const Exec &e, const HopCall &c)

@@ -232,6 +232,7 @@ struct LatDesc {
     long long off;           // float4 vectors
     long long fs;            // float4 vectors per field (6 * stride)
     int nrhs;
+    int first;               // the batch's system of its first right-hand side
 };
 // threads per block of the hopping kernels
 constexpr int kHopBlock = 128;
@@ -246,9 +247,12 @@ int hop_group_resident(int rpt, int spt);
 // and clover blocks are staged in shared memory and applied to every
 // right-hand side of the lattice (first right-hand side 0).
 // A persistent grid of `grid` blocks of (spt, kHopBlock / spt) threads
-// walks the table; mode HOP_K1 (odd output) or HOP_K2 (even output), FP32.
+// walks the table; mode HOP_K1 (odd output) or HOP_K2 (even output), FP32.  With
+// `scale` (device) the field that D_S multiplies is scale[r * sstride] times the
+// stored one of system r: K1 takes it on `in`, K2 on `in2`.
 void hop_group(const Exec &e, int mode, const LatDesc *desc, const int4 *tiles, int ntiles, int grid, int spt,
-               int rpt, const void *in, const void *in2, void *out, double bytes, double flops);
+               int rpt, const void *in, const void *in2, void *out, const double *scale, int sstride, double bytes,
+               double flops);
 // FP32 hopping-launch byte and flop counts of `sites` output sites with nrhs
 // right-hand sides sharing links and clover
 double hop_bytes(int mode, int prec, int nrhs, double sites);
@@ -332,7 +336,7 @@ struct KState {
     int *active;      // [N] cycle continues for this right-hand side
     int *kused;       // [N] Arnoldi steps taken this cycle
     int *nanflag;     // NaN/Inf seen
-    double *scale;    // [N] normaliser of the newest basis vector (0 when inactive)
+    double *scale;    // [N][m+1] normalisers of the basis vectors, stored unnormalised (0 once inactive)
     double *est;      // [N] residual estimate |g_{k+1}|
     double *target;   // [N] absolute residual target of the cycle
 };
@@ -350,11 +354,11 @@ struct Segs {
 // FP32 batched BLAS; basis vector j of system r at V + j * vjs + off_r
 void bdot(const Exec &e, const Segs &S, const void *V, long long vjs, int nv, const void *w, int N, BatchRed &br,
           int slot0);
+// (scale, [N] rows of sstride: the coefficient of v_j is scale_j^2 c_j)
 void baxpy(const Exec &e, const Segs &S, const void *V, long long vjs, int nv, const double *c, int cstride,
-           int sign, void *y, int N, BatchRed *br, int slot);
+           int sign, void *y, int N, BatchRed *br, int slot, const double *scale = nullptr, int sstride = 0);
 void bnorm(const Exec &e, int prec, const Segs &S, const void *w, int N, BatchRed &br, int slot);   // P32 or PDF
 void bfinish(const Exec &e, BatchRed &br, int N, int first, int count);
-void bscale(const Exec &e, const Segs &S, const void *x, const double *s, void *y, int N);
 void bxmy(const Exec &e, const Segs &S, const void *x, void *y, int N);   // y = x - y
 void ks_init(const Exec &e, const KState &k, const double *nrm2, int nstride);
 void ks_step(const Exec &e, const KState &k, int step, int passes, const double *dots, int dstride);
