@@ -379,7 +379,7 @@ static NatOut nat_of(const HopCall &c)
     return o;
 }
 // the modes that end a call on natural fields
-constexpr bool nat_mode(int mode) { return mode == HOP_K2 || mode == HOP_FULL || mode == HOP_RECON; }
+constexpr bool nat_mode(int mode) { return mode == HOP_K2 || mode == HOP_FULL; }
 
 template <int MODE>
 static void launch_hop_bf(const Exec &e, const HopCall &c)
@@ -426,6 +426,7 @@ __global__ void LQ_GROUP_BOUNDS hop_group_kernel(const LatDesc *__restrict__ d,
                                                                    const double *scale, int sstride)
 {
     constexpr int pout = MODE == HOP_K1 ? 1 : 0;
+    // consecutive entries, so that a site block's right-hand sides find its links in L1
     const int t0 = (int)((long long)ntiles * blockIdx.x / gridDim.x), t1 = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
     for (int t = t0; t < t1; t++) {
         const int4 w = __ldg(tiles + t);
@@ -673,7 +674,11 @@ constexpr int kDfVecs = 30;
 // a use of v that the compiler keeps before the copies that follow
 __device__ __forceinline__ void used(cx<df64> v) { asm volatile("" ::"f"(v.re.hi), "f"(v.re.lo), "f"(v.im.hi), "f"(v.im.lo) : "memory"); }
 
-template <int MODE, bool NAT>
+// IO, how the fields stand: the output natural (kNat), the neighbours' field in
+// FP32 (kIn32: its values are exact in df64, and a site reads half the bytes), the
+// output rounded to FP32 (kOut32)
+constexpr int kNat = 1, kIn32 = 2, kOut32 = 4;
+template <int MODE, int IO>
 __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &k, const df2 *in, const df2 *in2,
                                             const df2 *bv, df2 *out, df2 *out2, long long s, const Coords &c,
                                             float4 *stage, int nvalid)
@@ -706,8 +711,13 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
     };
     auto copy_psi = [&](long long nb) {
 #pragma unroll
-        for (int e = 0; e < 12; e++) copy_async(stage + (kDfPsi + e) * LQ_HOP_THREADS, in + nb + e * st);
+        for (int e = 0; e < (IO & kIn32 ? 6 : 12); e++) copy_async(stage + (kDfPsi + e) * LQ_HOP_THREADS, in + nb + e * st);
         copy_commit();
+    };
+    auto psi = [&](int e) {   // component e of the neighbour
+        if (!(IO & kIn32)) return vec(kDfPsi + e);
+        const float4 t = stage[(kDfPsi + (e >> 1)) * LQ_HOP_THREADS];
+        return cx<df64>{df64(e & 1 ? t.z : t.x, 0.0f), df64(e & 1 ? t.w : t.y, 0.0f)};
     };
     auto copy_link = [&](int d, long long nb) {
         const bool fwd = (d & 1) == 0;
@@ -738,10 +748,10 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
         cx<df64> h[6];
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            h[a] = vec(kDfPsi + a);
-            dl_cadd(h[a], rot_i(vec(kDfPsi + (pa == 3 ? 9 + a : 6 + a)), qa));
-            h[3 + a] = vec(kDfPsi + 3 + a);
-            dl_cadd(h[3 + a], rot_i(vec(kDfPsi + (pa == 3 ? 6 + a : 9 + a)), qb));
+            h[a] = psi(a);
+            dl_cadd(h[a], rot_i(psi(pa == 3 ? 9 + a : 6 + a), qa));
+            h[3 + a] = psi(3 + a);
+            dl_cadd(h[3 + a], rot_i(psi(pa == 3 ? 6 + a : 9 + a), qb));
         }
 #pragma unroll
         for (int a = 0; a < 6; a++) used(h[a]);
@@ -864,7 +874,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
                 for (int i = 0; i < 6; i++) y[i] = a6[i];
             }
         }
-        if (NAT) {
+        if (IO & kNat) {
             // through the vectors of the staging area that block 0 has left (each
             // lane's column turned by the component, against bank conflicts)
             const int lane = threadIdx.x & 31;
@@ -879,6 +889,12 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
             }
             __syncwarp();
             nat_write6(k.nat, tile, at, s - min(lane, nvalid - 1), nvalid, c.x & 1, blk);
+        } else if (IO & kOut32) {
+            float4 *f = reinterpret_cast<float4 *>(out) + (long long)blk * 3 * st + s;
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                f[i * st] = make_float4(df_to_float(y[2 * i].re), df_to_float(y[2 * i].im), df_to_float(y[2 * i + 1].re),
+                                        df_to_float(y[2 * i + 1].im));
         } else {
 #pragma unroll
             for (int i = 0; i < 6; i++) out[o + i * st] = cx_df2(y[i]);
@@ -895,7 +911,7 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
 // One thread per output site and right-hand side; the right-hand sides of a
 // site block are consecutive blocks, so its links and clover come from L2 for
 // all but the first.
-template <int MODE, bool NAT>
+template <int MODE, int IO>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ HopArgs<df64> k)
 {
@@ -904,7 +920,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(cons
     const unsigned sb = blockIdx.x / (unsigned)k.nrhs;
     long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
     int nv = 0;
-    if (NAT) {   // warps stay whole (warp_site)
+    if (IO & kNat) {   // warps stay whole (warp_site)
         nv = (int)min(32LL, g.Vh - (s - (threadIdx.x & 31)));
         if (nv <= 0) return;
         s = min(s, g.Vh - 1);
@@ -913,8 +929,30 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(cons
     }
     const Coords c = cb_coords(g, s, k.pout);
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs;
-    hop_df_body<MODE, NAT>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
+    hop_df_body<MODE, IO>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
                            k.out2 ? k.out2 + o : nullptr, s, c, df_stage + threadIdx.x, nv);
+}
+
+// one parity's FP32 field as its rows of a natural full field
+__global__ void __launch_bounds__(LQ_HOP_THREADS) export_parity_kernel(Geom g, const float4 *f, int parity, NatOut nat)
+{
+    extern __shared__ __align__(16) double2 nat_tile[];
+    int nv;
+    const long long s = warp_site(g, nv);
+    if (nv <= 0) return;
+    cx<float> v[12];
+    load_spinor_rw(f, g.stride, s, v);
+    store_nat(nat, nat_tile + (threadIdx.x >> 5) * 32 * kNatRow, f, s - min((int)(threadIdx.x & 31), nv - 1), nv,
+              cb_coords(g, s, parity).x & 1, v);
+}
+void export_parity(const Exec &e, const void *f, int parity, void *nat)
+{
+    Launch L_(e, K_LAYOUT, (double)e.g.Vh * (96 + 192));
+    NatOut o;
+    o.p = (double2 *)nat;
+    o.full = 1;
+    export_parity_kernel<<<(unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS), LQ_HOP_THREADS,
+                           nat_smem(LQ_HOP_THREADS), e.st>>>(e.g, (const float4 *)f, parity, o);
 }
 
 template <typename R>
@@ -959,9 +997,13 @@ static void launch_hop(const Exec &e, const HopCall &c)
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             launch_after(e, c.after, kernel, blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.g, k);
         };
+        if constexpr (MODE == HOP_PREP)
+            if (c.out32) return launch(hop_df_kernel<MODE, kOut32>);
+        if constexpr (MODE == HOP_RECON)
+            if (c.in32) return launch(hop_df_kernel<MODE, kNat | kIn32>);
         if constexpr (nat_mode(MODE))
-            if (c.nat) return launch(hop_df_kernel<MODE, true>);
-        launch(hop_df_kernel<MODE, false>);
+            if (c.nat) return launch(hop_df_kernel<MODE, kNat>);
+        launch(hop_df_kernel<MODE, 0>);
     }
     else
     {
@@ -1096,7 +1138,8 @@ void hop(const Exec &e, const HopCall &c)
     const double site_bytes = c.prec == PDF ? hop_site_bytes(c.mode, c.prec, c.nrhs)
                                             : c.nrhs * hop_site_bytes(c.mode, c.prec, 1);
     // natural rows are complex doubles whatever the precision
-    const double nat_bytes = c.nat ? 192.0 - (double)spinor_bytes(e.g, c.prec) / e.g.stride : 0.0;
+    const double nat_bytes = (c.nat ? 192.0 - (double)spinor_bytes(e.g, c.prec) / e.g.stride : 0.0) -
+                             96.0 * (c.in32 + c.out32);
     Launch L_(e, hop_class(c.mode, c.prec), (double)e.g.Vh * (site_bytes + nat_bytes), (double)e.g.Vh * c_hop_flops[c.mode] * c.nrhs);
     if (hop_split(e, c)) return;
     switch (c.mode) {

@@ -338,13 +338,18 @@ static void launch_split(const Exec &e, const HopCall &c)
     launch_after(e, c.after, hop_split_kernel<R, MODE, SV, LV, CV>, blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.g, k);
 }
 
-bool hop_split(const Exec &e, const HopCall &c)
+bool hop_split_takes(const Geom &g, int prec, int nrhs)
 {
     // sites up to which twelve threads are the faster: at 16384 df64 42.9 / 43.2 us
     // and FP32 25.9 / 27.6, at 18432 df64 44.7 / 43.3; FP64 86 / 88 at 10368 and
     // 114 / 92 at 16384; BF16 23.8 / 24.9 at 10368 and 26.9 / 24.9 at 13824
-    const long long most = c.prec == P16 ? 10368 : c.prec == P64 ? 12288 : 16384;
-    if (e.g.Vh * c.nrhs > most) return false;
+    const long long most = prec == P16 ? 10368 : prec == P64 ? 12288 : 16384;
+    return g.Vh * nrhs <= most;
+}
+
+bool hop_split(const Exec &e, const HopCall &c)
+{
+    if (!hop_split_takes(e.g, c.prec, c.nrhs)) return false;
 #define LQ_CASE(M)                                                                              \
     case M:                                                                                     \
         if (c.prec == P64) launch_split<double, M, double2, double2, double2>(e, c);            \

@@ -124,6 +124,8 @@ void export_half(const Exec &e, int prec, const void *f, void *nat);
 // natural full spinor [V][12] c128 <-> internal even and odd fields
 void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo);
 void export_full(const Exec &e, int prec, const void *fe, const void *fo, void *nat);
+// the rows of one parity of a natural full field from an FP32 field (dslash.cu)
+void export_parity(const Exec &e, const void *f, int parity, void *nat);
 // precision conversion between internal fields
 void convert(const Exec &e, int from, const void *in, int to, void *out);
 // out = g5 in (negates spins 2 and 3); in == out allowed
@@ -210,17 +212,21 @@ struct HopCall {
     void *out2 = nullptr;          // HOP_RECON_RES: the output parity's residual
     double omega;          // HOP_RICH weight
     int nrhs = 1;          // right-hand sides: in, in2, b, out are nrhs consecutive fields
-    // natural output (HOP_K2 in any precision; HOP_FULL and HOP_RECON but in BF16; one
-    // right-hand side): complex-double rows in the place of `out`, those of a full
-    // lattice or of one parity, spins 2 and 3 negated on request
+    // natural output (HOP_K2 in any precision, HOP_FULL but in BF16, HOP_RECON with
+    // in32; one right-hand side): complex-double rows in the place of `out`, those of
+    // a full lattice or of one parity, spins 2 and 3 negated on request
     void *nat = nullptr;
     bool nat_full = false, nat_g5 = false;
+    // df64 beyond hop_split's sizes, one right-hand side: HOP_PREP writes an FP32
+    // field, HOP_RECON with natural output reads `in` in FP32
+    bool in32 = false, out32 = false;
     bool after = true;     // launch_after: not behind a kernel that made links or clover blocks of this call
 };
 void hop(const Exec &e, const HopCall &c);
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
 // done, where the one-thread kernels are the faster ones
 bool hop_split(const Exec &e, const HopCall &c);
+bool hop_split_takes(const Geom &g, int prec, int nrhs);
 
 // One member lattice of a batched solve over lattices of different sizes: its
 // geometry, FP32 links and clover, and where its right-hand sides' fields sit
