@@ -13,7 +13,7 @@
 // intermediate live in shared memory, where the hops read their neighbours;
 // links and clover blocks come from block-major FP32 copies (below), so that
 // the sites of one block are contiguous and the half-steps re-read them from
-// L2 in whole cache lines.
+// L2 in whole cache lines, ahead of their use.
 //
 // The residual r = b - D x each block solve starts from is kept up to date
 // block by block instead of by applying D to the whole lattice before every
@@ -27,6 +27,8 @@
 //   r_B <- r_B + 1/2 sum over out-of-block neighbours of (1 -+ g_mu) W e'.
 // Each launch stores its blocks' even residual and its correction e; the next
 // launch of the other colour adds the face hops of e in a prologue.
+#include <type_traits>
+
 #include "lq_kernels.h"
 #include "spin.cuh"
 
@@ -98,51 +100,32 @@ __device__ __forceinline__ void st_sm(float2 *f, int i, const cx<float> v[12])
     for (int c = 0; c < 12; c++) f[c * SAP_THREADS + i] = make_float2(v[c].re, v[c].im);
 }
 
-// one direction of the block-local hopping sum at the site with local
-// coordinates l (parity p, global coordinates G, block-major index base + i):
-// the neighbour is read from the shared-memory field `src` of the other parity
-// when it lies in the block
-template <int MU>
-__device__ __forceinline__ void sap_hop_dir(const SapArgs &a, const float2 *src, const int l[4], const int G[4],
-                                            int p, long long base, int i, cx<float> acc[12])
+// The block-local neighbours of the i-th block site of parity p (local coordinates
+// l): byte d of .x (d < 4) and .y is the index of the site at direction
+// d = 2 mu + (backward), or kOut when that one lies outside the block; .z bit 0 / 1:
+// the hop to +t / -t crosses the lattice's time boundary (one block spans t).
+constexpr unsigned kOut = 0x80u;
+__device__ __forceinline__ uint3 sap_neighbours(const SapArgs &a, const int l[4])
 {
-    const int ext = a.b[MU], L = a.g.L[MU];
-    const bool whole = ext == L;   // the block spans the direction: the wrap stays inside
+    uint3 n = make_uint3(0u, 0u, 0u);
 #pragma unroll
-    for (int dir = 0; dir < 2; dir++) {
-        const int ln = dir == 0 ? l[MU] + 1 : l[MU] - 1;
-        const bool in = whole || (ln >= 0 && ln < ext);
-        if (!in) continue;
-        int q[4] = {l[0], l[1], l[2], l[3]};
-        q[MU] = (ln + ext) % ext;
-        const int nbi = (int)LQ_IDX((q[0] + a.b[0] * (q[1] + a.b[1] * (q[2] + a.b[2] * q[3]))) >> 1, a.bvh,
-                                    B_SAP_LOCAL);
-        cx<float> psi[12];
-        ld_sm(src, nbi, psi);
-        cx<float> m[9];
-        float s = 1.0f;
-        if (dir == 0) {
-            load_link(a.Ub[p], a.g.stride, MU, LQ_IDX(base + i, a.g.Vh, B_SAP_GLOBAL), m);
-            if (MU == 3 && G[3] + 1 == L) s = (float)a.g.tbc;
-            hop_apply<MU, -1>(acc, psi, m, s);
-        } else {   // the link of the neighbour at -mu, which lies in the block
-            load_link(a.Ub[1 - p], a.g.stride, MU, LQ_IDX(base + nbi, a.g.Vh, B_SAP_GLOBAL), m);
-            if (MU == 3 && G[3] == 0) s = (float)a.g.tbc;
-            hop_apply<MU, +1>(acc, psi, m, s);
+    for (int mu = 0; mu < 4; mu++) {
+        const int ext = a.b[mu];
+        const bool whole = ext == a.g.L[mu];   // the block spans the direction: the wrap stays inside
+#pragma unroll
+        for (int back = 0; back < 2; back++) {
+            int q[4] = {l[0], l[1], l[2], l[3]};
+            const bool edge = back ? q[mu] == 0 : q[mu] + 1 == ext;
+            q[mu] = back ? (edge ? ext - 1 : q[mu] - 1) : (edge ? 0 : q[mu] + 1);
+            const unsigned idx = (unsigned)LQ_IDX((q[0] + a.b[0] * (q[1] + a.b[1] * (q[2] + a.b[2] * q[3]))) >> 1,
+                                                  a.bvh, B_SAP_LOCAL);
+            const unsigned v = (edge && !whole ? kOut : idx) << (8 * ((2 * mu + back) & 3));
+            if (mu < 2) n.x |= v;
+            else n.y |= v;
+            if (mu == 3 && edge && whole) n.z |= 1u << back;
         }
     }
-}
-
-// acc = sum over the in-block neighbours of (1 -+ g_mu) W psi
-__device__ __forceinline__ void sap_hop(const SapArgs &a, const float2 *src, const int l[4], const int G[4], int p,
-                                        long long base, int i, cx<float> acc[12])
-{
-#pragma unroll
-    for (int k = 0; k < 12; k++) acc[k] = {0.0f, 0.0f};
-    sap_hop_dir<0>(a, src, l, G, p, base, i, acc);
-    sap_hop_dir<1>(a, src, l, G, p, base, i, acc);
-    sap_hop_dir<2>(a, src, l, G, p, base, i, acc);
-    sap_hop_dir<3>(a, src, l, G, p, base, i, acc);
+    return n;
 }
 
 // The hops across the two faces of the block normal to MU: for every site on
@@ -220,13 +203,15 @@ __device__ __forceinline__ void sap_sum3(float v[3], float *sh)
     }
 }
 
-#ifndef LQ_SAP_MINB
-#define LQ_SAP_MINB 4
-#endif
-
-// The CTA asks for four resident blocks per SM (at most 128 registers, no spills); the
-// MR iterate and residual live in shared memory, not in registers.  The solve
-// is one loop over half-steps, each one hop into one parity followed by its
+// Three resident blocks per SM (168 registers): the MR iterate and residual and
+// the odd intermediate live in shared memory, and the registers hold loads ahead
+// of their use: a link is read while the direction before it is computed, also
+// across half-steps, and the first clover block during the last direction.  It
+// waits on those loads all the same (long scoreboard the first stall, the issue
+// slots 42% busy): SAP(3, 4) on 24^3 x 48 takes 1525 us, 1641 at four blocks (128
+// registers), 1697 at two, and 1807 with the operands copied to a shared-memory
+// ring five steps ahead, whose copies cost more issue than they save waiting.  The
+// solve is one loop over half-steps, each one hop into one parity followed by its
 // epilogue, so that a single copy of the hop code serves all of them (the
 // instruction cache holds it):
 //   (face) the block's residual rin plus the face hops of e', staged in smE / smO
@@ -235,6 +220,9 @@ __device__ __forceinline__ void sap_sum3(float v[3], float *sh)
 //   2j+2   odd:  t = D_oo^{-1} (-1/2 H_oe res)                     (MR step j)
 //   2j+3   even: p = C res + 1/2 H_eo t; alpha; e += alpha res; res -= alpha p
 //   2m+2   odd:  e_o = D_oo^{-1} (r_o + 1/2 H_oe e_e); x += e; store e and res
+#ifndef LQ_SAP_MINB
+#define LQ_SAP_MINB 3
+#endif
 __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(SapArgs a)
 {
     __shared__ float2 smE[12 * SAP_THREADS];   // even: r_e, r_hat, then the MR residual
@@ -250,22 +238,43 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
         sap_local(a, i, 0, le);
         sap_local(a, i, 1, lo);
     }
+    const uint3 ne = sap_neighbours(a, le), no = sap_neighbours(a, lo);
     const long long st = a.g.stride;
     const long long base = sap_block_base(a, O);
     const long long sb = on ? LQ_IDX(base + i, a.g.Vh, B_SAP_GLOBAL) : 0;   // block-major index of the thread's sites
+    // lattice indices of the thread's sites
+    long long cbe = 0, cbo = 0;
+    if (on) {
+        const int Ge[4] = {O[0] + le[0], O[1] + le[1], O[2] + le[2], O[3] + le[3]};
+        const int Go[4] = {O[0] + lo[0], O[1] + lo[1], O[2] + lo[2], O[3] + lo[3]};
+        cbe = sap_global_cb(a.g, Ge);
+        cbo = sap_global_cb(a.g, Go);
+    }
     const int last = 2 * a.m + 2;
     const bool face = a.eface[0] != nullptr;
+
+    // the output parity of half-step ph > 0, and the byte of a packed neighbour table
+    auto parity_of = [&](int ph) { return ph < last && (ph & 1) ? 0 : 1; };
+    auto neighbour = [&](int p, int d) {
+        const unsigned w = d < 4 ? (p ? no.x : ne.x) : (p ? no.y : ne.y);
+        return (w >> (8 * (d & 3))) & 0xFFu;
+    };
+    // the link of direction d into parity p: its own forward, the neighbour's at -mu
+    // backward (any valid one where the neighbour lies outside the block)
+    float4 link[3];
+    auto load_next = [&](int p, int d) {
+        const bool back = d & 1;
+        const long long at = back ? LQ_IDX(base + (neighbour(p, d) & 0x7Fu), a.g.Vh, B_SAP_GLOBAL) : sb;
+        const float4 *u = a.Ub[back ? 1 - p : p] + (long long)(d >> 1) * 3 * st + at;
+#pragma unroll
+        for (int k = 0; k < 3; k++) link[k] = ldg(u + k * st);
+    };
     if (face) {
         if (on) {
-            int G[4];
             cx<float> v[12];
-#pragma unroll
-            for (int mu = 0; mu < 4; mu++) G[mu] = O[mu] + le[mu];
-            load_spinor_rw(a.rin[0], st, sap_global_cb(a.g, G), v);
+            load_spinor_rw(a.rin[0], st, cbe, v);
             st_sm(smE, i, v);
-#pragma unroll
-            for (int mu = 0; mu < 4; mu++) G[mu] = O[mu] + lo[mu];
-            if (a.rin[1]) load_spinor_rw(a.rin[1], st, sap_global_cb(a.g, G), v);
+            if (a.rin[1]) load_spinor_rw(a.rin[1], st, cbo, v);
             else
 #pragma unroll
                 for (int k = 0; k < 12; k++) v[k] = {0.0f, 0.0f};
@@ -281,70 +290,104 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
         sap_face<3>(a, O, smE, smO);
         __syncthreads();
     }
+    if (on) {   // half-step 0; r_o is kept for the last one
+        cx<float> v[12], pv[12];
+        if (face) ld_sm(smO, i, v);
+        else load_spinor_rw(a.rin[1], st, cbo, v);
+        store_spinor(a.ro, st, cbo, v);
+        clover_apply<float>(a.Ci, st, sb, v, pv);
+        st_sm(smO, i, pv);
+    }
+    load_next(0, 0);
+    __syncthreads();
 #pragma unroll 1
-    for (int ph = 0; ph <= last; ph++) {
-        const int p = (ph == 1 || (ph > 1 && ph < last && (ph & 1))) ? 0 : 1;   // output parity
-        int l[4], G[4];
-#pragma unroll
-        for (int mu = 0; mu < 4; mu++) {
-            l[mu] = p ? lo[mu] : le[mu];
-            G[mu] = O[mu] + l[mu];
-        }
-        const long long cb = on ? sap_global_cb(a.g, G) : 0;
+    for (int ph = 1; ph <= last; ph++) {
+        const int p = parity_of(ph);   // output parity
+        // the hops from the other parity
         cx<float> w[12];
-        if (on && ph > 0) sap_hop(a, p ? (ph == last ? smX : smE) : smO, l, G, p, base, i, w);
-        float d[3] = {0.0f, 0.0f, 0.0f};
-        cx<float> pv[12];
-        if (on) {
-            cx<float> v[12];
-            if (ph == 0) {   // r_o, kept for the last half-step
-                if (face) ld_sm(smO, i, v);
-                else load_spinor_rw(a.rin[1], st, cb, v);
-                store_spinor(a.ro, st, cb, v);
+#pragma unroll
+        for (int k = 0; k < 12; k++) w[k] = {0.0f, 0.0f};
+        const float2 *src = p ? (ph == last ? smX : smE) : smO;
+        const float4 *C = (p ? a.Ci : a.Ce) + sb;
+        float4 c0[9];   // the first clover block
+        auto hop = [&](auto D) {
+            constexpr int d = decltype(D)::value;
+            cx<float> m[9];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                m[2 * k] = {link[k].x, link[k].y};
+                m[2 * k + 1] = {link[k].z, link[k].w};
             }
-            if (p == 1) {   // odd output: D_oo^{-1} (...)
-                if (ph == last) {
-                    load_spinor_rw(a.ro, st, cb, v);
+            if (d < 7) {
+                load_next(p, d + 1);
+            } else if (ph > 1) {
 #pragma unroll
-                    for (int k = 0; k < 12; k++) v[k] = v[k] + 0.5f * w[k];
-                } else if (ph > 0) {
-#pragma unroll
-                    for (int k = 0; k < 12; k++) v[k] = -0.5f * w[k];
-                }
-                clover_apply<float>(a.Ci, st, sb, v, pv);
-                if (ph < last) {
-                    st_sm(smO, i, pv);
-                } else {   // x += e on both parities of the site pair; store e and the residual
-                    store_spinor(a.eout[1], st, cb, pv);
-                    load_spinor_rw(a.x[1], st, cb, v);
-#pragma unroll
-                    for (int k = 0; k < 12; k++) v[k] = v[k] + pv[k];
-                    store_spinor(a.x[1], st, cb, v);
-                    int Ge[4];
-#pragma unroll
-                    for (int mu = 0; mu < 4; mu++) Ge[mu] = O[mu] + le[mu];
-                    const long long cbe = sap_global_cb(a.g, Ge);
-                    ld_sm(smE, i, v);
-                    store_spinor(a.rout_e, st, cbe, v);
-                    ld_sm(smX, i, pv);
-                    store_spinor(a.eout[0], st, cbe, pv);
-                    load_spinor_rw(a.x[0], st, cbe, v);
-#pragma unroll
-                    for (int k = 0; k < 12; k++) v[k] = v[k] + pv[k];
-                    store_spinor(a.x[0], st, cbe, v);
-                }
-            } else if (ph == 1) {   // r_hat = r_e + 1/2 H_eo (D_oo^{-1} r_o), e = 0
+                for (int k = 0; k < 9; k++) c0[k] = ldg(C + k * st);
+            }
+            const unsigned nb = neighbour(p, d);
+            if (!on || nb == kOut) return;
+            cx<float> psi[12];
+            ld_sm(src, (int)nb, psi);
+            third_row(m);
+            const bool cross = d >= 6 && (((p ? no.z : ne.z) >> (d & 1)) & 1u);
+            hop_apply<(d >> 1), (d & 1) ? +1 : -1>(w, psi, m, cross ? (float)a.g.tbc : 1.0f);
+        };
+        hop(std::integral_constant<int, 0>());
+        hop(std::integral_constant<int, 1>());
+        hop(std::integral_constant<int, 2>());
+        hop(std::integral_constant<int, 3>());
+        hop(std::integral_constant<int, 4>());
+        hop(std::integral_constant<int, 5>());
+        hop(std::integral_constant<int, 6>());
+        hop(std::integral_constant<int, 7>());
+        if (ph == 1) {   // r_hat = r_e + 1/2 H_eo (D_oo^{-1} r_o), e = 0
+            if (on) {
+                cx<float> v[12];
                 if (face) ld_sm(smE, i, v);   // r_e from the prologue
-                else load_spinor_rw(a.rin[0], st, cb, v);
+                else load_spinor_rw(a.rin[0], st, cbe, v);
 #pragma unroll
                 for (int k = 0; k < 12; k++) v[k] = v[k] + 0.5f * w[k];
                 st_sm(smE, i, v);
 #pragma unroll
                 for (int k = 0; k < 12; k++) v[k] = {0.0f, 0.0f};
                 st_sm(smX, i, v);
-            } else if (ph > 1) {   // p = C res + 1/2 H_eo t and the dot products
+            }
+            load_next(1, 0);
+            __syncthreads();
+            continue;
+        }
+        // what the clover blocks multiply: the residual (even) or the hops (odd)
+        cx<float> v[12], pv[12];
+        if (on) {
+            if (p == 0) {
                 ld_sm(smE, i, v);
-                clover_apply<float>(a.Ce, st, sb, v, pv);
+            } else if (ph == last) {
+                load_spinor_rw(a.ro, st, cbo, v);
+#pragma unroll
+                for (int k = 0; k < 12; k++) v[k] = v[k] + 0.5f * w[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < 12; k++) v[k] = -0.5f * w[k];
+            }
+        }
+        if (on) {
+            float c[36];
+#pragma unroll
+            for (int blk = 0; blk < 2; blk++) {
+#pragma unroll
+                for (int k = 0; k < 9; k++) {
+                    c[4 * k] = c0[k].x;
+                    c[4 * k + 1] = c0[k].y;
+                    c[4 * k + 2] = c0[k].z;
+                    c[4 * k + 3] = c0[k].w;
+                    if (blk == 0) c0[k] = ldg(C + (9 + k) * st);
+                }
+                herm6_apply<float>(c, v + 6 * blk, pv + 6 * blk);
+            }
+        }
+        if (p == 0) {   // p = C res + 1/2 H_eo t, the dot products and the MR update
+            float d[3] = {0.0f, 0.0f, 0.0f};
+            if (on)
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
                     pv[k] = pv[k] + 0.5f * w[k];
@@ -352,14 +395,10 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
                     d[1] = fmaf(pv[k].re, v[k].im, fmaf(-pv[k].im, v[k].re, d[1]));   // Im (p, res)
                     d[2] = fmaf(pv[k].re, pv[k].re, fmaf(pv[k].im, pv[k].im, d[2]));  // (p, p)
                 }
-            }
-        }
-        if (p == 0 && ph > 1) {   // the MR update after an even half-step
             sap_sum3(d, red);
             const float ar = d[2] > 0.0f ? d[0] / d[2] : 0.0f, ai = d[2] > 0.0f ? d[1] / d[2] : 0.0f;
             if (on) {
-                cx<float> v[12], e[12];
-                ld_sm(smE, i, v);
+                cx<float> e[12];
                 ld_sm(smX, i, e);
 #pragma unroll
                 for (int k = 0; k < 12; k++) {
@@ -369,7 +408,24 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
                 st_sm(smE, i, v);
                 st_sm(smX, i, e);
             }
+        } else if (on && ph < last) {
+            st_sm(smO, i, pv);
+        } else if (on) {   // x += e on both parities of the site pair; store e and the residual
+            store_spinor(a.eout[1], st, cbo, pv);
+            load_spinor_rw(a.x[1], st, cbo, v);
+#pragma unroll
+            for (int k = 0; k < 12; k++) v[k] = v[k] + pv[k];
+            store_spinor(a.x[1], st, cbo, v);
+            ld_sm(smE, i, v);
+            store_spinor(a.rout_e, st, cbe, v);
+            ld_sm(smX, i, pv);
+            store_spinor(a.eout[0], st, cbe, pv);
+            load_spinor_rw(a.x[0], st, cbe, v);
+#pragma unroll
+            for (int k = 0; k < 12; k++) v[k] = v[k] + pv[k];
+            store_spinor(a.x[0], st, cbe, v);
         }
+        if (ph < last) load_next(parity_of(ph + 1), 0);
         __syncthreads();
     }
 }
