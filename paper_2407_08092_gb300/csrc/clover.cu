@@ -18,7 +18,7 @@
 // from df64 by clover_to_f64 when an FP64 operator first needs them.  The
 // field strengths F of the six planes come from three passes over plaquettes
 // (one thread per (site, plane) each, into scratch arrays), then one thread
-// per site assembles the two 6x6 blocks.
+// per site and 6x6 block assembles it.
 #include "leaves.cuh"
 #include "lq_kernels.h"
 
@@ -221,11 +221,12 @@ __device__ __forceinline__ cx<df64> f_entry(const float2 *__restrict__ Fb, long 
 // The entries are formed in their packed order and stored four at a time (two
 // df2 and one FP32 float4), so only four of a block's 36 entries are held in
 // registers at once.  diag = 4 + m0 and h come as df64 pairs split on the host.
-// Four resident blocks per SM (128 registers, a few bytes of spills) against
-// two unbounded: 0.60 against 0.74 ms per launch of assembly and inverse on
-// 32^3 x 64, on average.
+// One thread per site and block (the two blocks of a site in one CTA, whose L1 serves
+// the second reading of F), five CTAs per SM (96 registers): 180 us on 24^3 x 48, 187
+// at four and 192 at six; a thread that made both blocks took 230 (0.55 of the copy
+// bandwidth, waiting on its loads).
 #ifndef LQ_CLA_MINB
-#define LQ_CLA_MINB 4
+#define LQ_CLA_MINB 5
 #endif
 __global__ void __launch_bounds__(128, LQ_CLA_MINB) clover_assemble_kernel(Geom g, const float2 *__restrict__ Fb, df64 diag,
                                                               df64 h, df2 *Ce, df2 *Co, float4 *C32e, float4 *C32o)
@@ -240,8 +241,8 @@ __global__ void __launch_bounds__(128, LQ_CLA_MINB) clover_assemble_kernel(Geom 
     const long long cb = lex >> 1;
     df2 *C = parity ? Co : Ce;
     float4 *C32 = parity ? C32o : C32e;
-#pragma unroll 1
-    for (int b = 0; b < 2; b++) {
+    const int b = threadIdx.y;
+    {
         const bool plus = b == 0;
         // G_l entries (a, c) for this block
         auto G = [&](int l, int a, int cc) {
@@ -455,7 +456,7 @@ void clover_build(const Exec &e, const void *Udf[2], double csw, double m0, void
     Launch L_(e, K_CLOVER, (double)e.g.V * (6 * 72 + 72 * (8 + 4)));
     const double dg = 4.0 + m0, hh = 0.5 * csw;
     const float dg_hi = (float)dg, hh_hi = (float)hh;
-    clover_assemble_kernel<<<blocks_for(e.g.V, 128), 128, 0, e.st>>>(
+    clover_assemble_kernel<<<blocks_for(e.g.V, 64), dim3(64, 2), 0, e.st>>>(
         e.g, (const float2 *)Fscratch, df64(dg_hi, (float)(dg - (double)dg_hi)), df64(hh_hi, (float)(hh - (double)hh_hi)),
         (df2 *)Cdf[0], (df2 *)Cdf[1], (float4 *)C32[0], (float4 *)C32[1]);
 }
