@@ -128,6 +128,24 @@ __device__ __forceinline__ uint3 sap_neighbours(const SapArgs &a, const int l[4]
     return n;
 }
 
+// Reals 12 Q .. 12 Q + 11 of a packed Hermitian 6x6 block applied to x: the parts in
+// turn are herm6_apply, operation for operation.
+template <int Q>
+__device__ __forceinline__ void herm6_part(const float4 c[3], const cx<float> *x, cx<float> *y)
+{
+    const float a[12] = {c[0].x, c[0].y, c[0].z, c[0].w, c[1].x, c[1].y, c[1].z, c[1].w, c[2].x, c[2].y, c[2].z, c[2].w};
+    if (Q == 0)
+#pragma unroll
+        for (int i = 0; i < 6; i++) y[i] = a[i] * x[i];
+#pragma unroll
+    for (int e = Q == 0 ? 6 : 0; e < 12; e += 2) {
+        const int t = (12 * Q + e - 6) / 2, i = t < 1 ? 1 : t < 3 ? 2 : t < 6 ? 3 : t < 10 ? 4 : 5, j = t - tri(i, 0);
+        const cx<float> l = {a[e], a[e + 1]};
+        y[i] = cfma(l, x[j], y[i]);
+        y[j] = cfmac(l, x[i], y[j]);
+    }
+}
+
 // The hops across the two faces of the block normal to MU: for every site on
 // a face, 1/2 (1 -+ g_mu) W e' of its neighbour outside the block is added to
 // the site's residual in shared memory (smE even, smO odd).  The work items
@@ -204,16 +222,16 @@ __device__ __forceinline__ void sap_sum3(float v[3], float *sh)
 }
 
 // Three resident blocks per SM (168 registers): the MR iterate and residual and
-// the odd intermediate live in shared memory, and the registers hold loads ahead
-// of their use: a link is read while the direction before it is computed, also
-// across half-steps, and the first clover block during the last direction.  It
-// waits on those loads all the same (long scoreboard the first stall, the issue
-// slots 42% busy): SAP(3, 4) on 24^3 x 48 takes 1525 us, 1641 at four blocks (128
-// registers), 1697 at two, and 1807 with the operands copied to a shared-memory
-// ring five steps ahead, whose copies cost more issue than they save waiting.  The
-// solve is one loop over half-steps, each one hop into one parity followed by its
-// epilogue, so that a single copy of the hop code serves all of them (the
-// instruction cache holds it):
+// the odd intermediate live in shared memory, and the registers hold what comes
+// from global memory four chunks (directions, or thirds of a clover block) ahead
+// of its use, also across half-steps, since the loads' latency is what the kernel
+// waits for.  SAP(3, 4) on 24^3 x 48: 1641 us at four blocks (128 registers) with
+// each link loaded where it is used, 1552 so at three, 1525 with the link of the
+// next direction loaded ahead, 1393 two chunks ahead, 1353 four; 1807 with the
+// operands copied to a shared-memory ring, whose copies cost more issue than they
+// save waiting.  The solve is one loop over half-steps, each one hop into one
+// parity followed by its epilogue, so that a single copy of the hop code serves
+// all of them (the instruction cache holds it):
 //   (face) the block's residual rin plus the face hops of e', staged in smE / smO
 //   0      odd:  D_oo^{-1} r_o                               (no hop; r_o kept in ro)
 //   1      even: r_hat = r_e + 1/2 H_eo (D_oo^{-1} r_o); e = 0
@@ -259,16 +277,32 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
         const unsigned w = d < 4 ? (p ? no.x : ne.x) : (p ? no.y : ne.y);
         return (w >> (8 * (d & 3))) & 0xFFu;
     };
-    // the link of direction d into parity p: its own forward, the neighbour's at -mu
-    // backward (any valid one where the neighbour lies outside the block)
-    float4 link[3];
-    auto load_next = [&](int p, int d) {
-        const bool back = d & 1;
-        const long long at = back ? LQ_IDX(base + (neighbour(p, d) & 0x7Fu), a.g.Vh, B_SAP_GLOBAL) : sb;
-        const float4 *u = a.Ub[back ? 1 - p : p] + (long long)(d >> 1) * 3 * st + at;
+    // The operands from global memory, in chunks of three vectors: of half-step ph
+    // the links of directions 0..7 (its own forward, the neighbour's at -mu backward,
+    // any valid one where that lies outside the block), then the clover blocks (8..13,
+    // none in half-step 1); chunks beyond are those of the next half-step.
+    auto load_chunk = [&](int ph, int c, float4 *dst) {
+        const int n = ph == 1 ? 8 : 14;
+        if (c >= n) {
+            c -= n;
+            ph++;
+        }
+        if (ph > last) return;
+        const int p = parity_of(ph);
+        const float4 *u;
+        if (c < 8) {
+            const bool back = c & 1;
+            u = a.Ub[back ? 1 - p : p] + (long long)(c >> 1) * 3 * st +
+                (back ? LQ_IDX(base + (neighbour(p, c) & 0x7Fu), a.g.Vh, B_SAP_GLOBAL) : sb);
+        } else {
+            u = (p ? a.Ci : a.Ce) + (long long)(c - 8) * 3 * st + sb;
+        }
 #pragma unroll
-        for (int k = 0; k < 3; k++) link[k] = ldg(u + k * st);
+        for (int k = 0; k < 3; k++) dst[k] = ldg(u + k * st);
     };
+    float4 B[4][3], E[2][3];   // chunks c in B[c & 3], but 12 and 13 in E
+#pragma unroll
+    for (int c = 0; c < 4; c++) load_chunk(1, c, B[c]);
     if (face) {
         if (on) {
             cx<float> v[12];
@@ -298,7 +332,6 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
         clover_apply<float>(a.Ci, st, sb, v, pv);
         st_sm(smO, i, pv);
     }
-    load_next(0, 0);
     __syncthreads();
 #pragma unroll 1
     for (int ph = 1; ph <= last; ph++) {
@@ -308,22 +341,15 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
 #pragma unroll
         for (int k = 0; k < 12; k++) w[k] = {0.0f, 0.0f};
         const float2 *src = p ? (ph == last ? smX : smE) : smO;
-        const float4 *C = (p ? a.Ci : a.Ce) + sb;
-        float4 c0[9];   // the first clover block
         auto hop = [&](auto D) {
             constexpr int d = decltype(D)::value;
             cx<float> m[9];
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                m[2 * k] = {link[k].x, link[k].y};
-                m[2 * k + 1] = {link[k].z, link[k].w};
+                m[2 * k] = {B[d & 3][k].x, B[d & 3][k].y};
+                m[2 * k + 1] = {B[d & 3][k].z, B[d & 3][k].w};
             }
-            if (d < 7) {
-                load_next(p, d + 1);
-            } else if (ph > 1) {
-#pragma unroll
-                for (int k = 0; k < 9; k++) c0[k] = ldg(C + k * st);
-            }
+            load_chunk(ph, d + 4, B[d & 3]);
             const unsigned nb = neighbour(p, d);
             if (!on || nb == kOut) return;
             cx<float> psi[12];
@@ -352,12 +378,15 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
                 for (int k = 0; k < 12; k++) v[k] = {0.0f, 0.0f};
                 st_sm(smX, i, v);
             }
-            load_next(1, 0);
             __syncthreads();
             continue;
         }
+        load_chunk(ph, 12, E[0]);
+        load_chunk(ph, 13, E[1]);
         // what the clover blocks multiply: the residual (even) or the hops (odd)
         cx<float> v[12], pv[12];
+#pragma unroll
+        for (int k = 0; k < 12; k++) v[k] = {0.0f, 0.0f};
         if (on) {
             if (p == 0) {
                 ld_sm(smE, i, v);
@@ -370,21 +399,16 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
                 for (int k = 0; k < 12; k++) v[k] = -0.5f * w[k];
             }
         }
-        if (on) {
-            float c[36];
-#pragma unroll
-            for (int blk = 0; blk < 2; blk++) {
-#pragma unroll
-                for (int k = 0; k < 9; k++) {
-                    c[4 * k] = c0[k].x;
-                    c[4 * k + 1] = c0[k].y;
-                    c[4 * k + 2] = c0[k].z;
-                    c[4 * k + 3] = c0[k].w;
-                    if (blk == 0) c0[k] = ldg(C + (9 + k) * st);
-                }
-                herm6_apply<float>(c, v + 6 * blk, pv + 6 * blk);
-            }
-        }
+        herm6_part<0>(B[0], v, pv);
+        load_chunk(ph, 14, B[0]);
+        herm6_part<1>(B[1], v, pv);
+        load_chunk(ph, 15, B[1]);
+        herm6_part<2>(B[2], v, pv);
+        load_chunk(ph, 16, B[2]);
+        herm6_part<0>(B[3], v + 6, pv + 6);
+        load_chunk(ph, 17, B[3]);
+        herm6_part<1>(E[0], v + 6, pv + 6);
+        herm6_part<2>(E[1], v + 6, pv + 6);
         if (p == 0) {   // p = C res + 1/2 H_eo t, the dot products and the MR update
             float d[3] = {0.0f, 0.0f, 0.0f};
             if (on)
@@ -425,7 +449,6 @@ __global__ void __launch_bounds__(SAP_THREADS, LQ_SAP_MINB) sap_block_kernel(Sap
             for (int k = 0; k < 12; k++) v[k] = v[k] + pv[k];
             store_spinor(a.x[0], st, cbe, v);
         }
-        if (ph < last) load_next(parity_of(ph + 1), 0);
         __syncthreads();
     }
 }
