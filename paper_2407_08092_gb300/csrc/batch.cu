@@ -254,7 +254,6 @@ struct cdbl {
 };
 __device__ __forceinline__ cdbl cd_mul(cdbl a, cdbl b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
 __device__ __forceinline__ cdbl cd_conj(cdbl a) { return {a.re, -a.im}; }
-__device__ __forceinline__ double cd_abs(cdbl a) { return hypot(a.re, a.im); }
 
 // Start of a cycle: beta_r = sqrt(nrm2_r); g_r = beta e_1; the cycle of a
 // right-hand side whose residual already meets its target (or is 0) stays
@@ -329,18 +328,19 @@ __global__ void ks_step_kernel(int N, int m, int k, int passes, const double *do
         Hr[(long long)k * (m + 1) + i] = make_double2(ci * a.re + sb.re, ci * a.im + sb.im);
         a = {-sca.re + ci * b.re, -sca.im + ci * b.im};
     }
+    // one thread's chain of FP64 roots and quotients is what this kernel takes:
+    // each is formed once
     const cdbl b = {hk1, 0.0};
-    const double t = sqrt(a.re * a.re + a.im * a.im + hk1 * hk1);
+    const double a2 = a.re * a.re + a.im * a.im;
     double c;
     cdbl s;
-    if (cd_abs(a) == 0.0) {
+    if (a2 == 0.0) {
         c = 0.0;
         s = {1.0, 0.0};
     } else {
-        const double aa = cd_abs(a);
-        c = aa / t;
-        s = cd_mul({a.re / aa, a.im / aa}, cd_conj(b));
-        s = {s.re / t, s.im / t};
+        const double aa = sqrt(a2), it = 1.0 / sqrt(a2 + hk1 * hk1), f = hk1 * it / aa;
+        c = aa * it;
+        s = {a.re * f, a.im * f};
     }
     csr[k] = c;
     snr[k] = make_double2(s.re, s.im);
@@ -351,10 +351,10 @@ __global__ void ks_step_kernel(int N, int m, int k, int passes, const double *do
     const cdbl ng = cd_mul(cd_conj(s), gk);
     gr[k] = make_double2(c * gk.re, c * gk.im);
     gr[k + 1] = make_double2(-ng.re, -ng.im);
-    const double e = hypot(ng.re, ng.im);
+    const double e = sqrt(ng.re * ng.re + ng.im * ng.im);
     est[r] = e;
     kused[r] = k + 1;
-    const bool breakdown = hk1 <= 1e-14 * sqrt(colnorm2);
+    const bool breakdown = hk1 * hk1 <= 1e-28 * colnorm2;
     const bool go = !breakdown && e > target[r] && k + 1 < m;
     active[r] = go ? 1 : 0;
     sr[k + 1] = go ? 1.0 / hk1 : 0.0;
