@@ -671,6 +671,7 @@ __device__ __forceinline__ void herm6_fma_df(Ld ld, const cx<df64> x[6], cx<df64
 constexpr int kDfPsi = 0;        // the neighbour's 12 components
 constexpr int kDfLink = 12;      // two buffers of 9 link entries
 constexpr int kDfVecs = 30;
+constexpr int kDfSites = LQ_HOP_THREADS / 2;   // sites of a block: two threads each
 // a use of v that the compiler keeps before the copies that follow
 __device__ __forceinline__ void used(cx<df64> v) { asm volatile("" ::"f"(v.re.hi), "f"(v.re.lo), "f"(v.im.hi), "f"(v.im.lo) : "memory"); }
 
@@ -686,8 +687,10 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
     // The directions run through one loop body (the tables of spin.cuh).  The
     // neighbour's components and the link's entries are read as the
     // projection and the product use them, and every sum is lazily normalised
-    // (dl_*): acc is renormalised once, after the eight directions.
+    // (dl_*): the two halves' sums are added and renormalised once.
     const long long st = g.stride;
+    const int half = threadIdx.x / kDfSites, d0 = 4 * half, d1 = d0 + 4;
+    const bool on = (int)(threadIdx.x & 31) < nvalid;   // shadowing lanes store nothing
     cx<df64> acc[12];
 #pragma unroll
     for (int i = 0; i < 12; i++) acc[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
@@ -703,8 +706,8 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
     // reads its operands as it comes to them (long scoreboard the first stall,
     // the FMA pipe 60% busy at 12 warps an SM).  So they are copied to shared
     // memory ahead: the links of direction d + 1 while d runs (two buffers),
-    // the neighbour of d + 1 as soon as d is projected, and the first clover
-    // block while the last direction is multiplied.
+    // the neighbour of d + 1 as soon as d is projected, and the clover block
+    // while the last direction is multiplied.
     auto vec = [&](int e) {
         const float4 t = stage[e * LQ_HOP_THREADS];
         return cx<df64>{df64(t.x, t.z), df64(t.y, t.w)};
@@ -727,17 +730,17 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
         copy_commit();
     };
     bool flip;
-    long long nb = neighbour(0, flip);
-    copy_link(0, nb);
+    long long nb = neighbour(d0, flip);
+    copy_link(d0, nb);
     copy_psi(nb);
 #pragma unroll 1
-    for (int d = 0; d < 8; d++) {
+    for (int d = d0; d < d1; d++) {
         const bool fwd = (d & 1) == 0;
         bool flip1 = false;
-        const long long nb1 = d < 7 ? neighbour(d + 1, flip1) : 0;
+        const long long nb1 = d + 1 < d1 ? neighbour(d + 1, flip1) : 0;
 #pragma unroll
         for (int a = 0; a < 3; a++) used(acc[a]);   // the last direction's link entries are used up
-        if (d < 7) {
+        if (d + 1 < d1) {
             copy_link(d + 1, nb1);
             copy_wait<1>();
         } else {
@@ -755,11 +758,11 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
         }
 #pragma unroll
         for (int a = 0; a < 6; a++) used(h[a]);
-        if (d < 7) {
+        if (d + 1 < d1) {
             copy_psi(nb1);
-        } else if (MODE != HOP_PREP) {   // the first clover block, over the neighbour and the free link buffer
+        } else if (MODE != HOP_PREP) {   // the clover block, over the neighbour and the free link buffer
 #pragma unroll
-            for (int e = 0; e < 18; e++) copy_async(stage + e * LQ_HOP_THREADS, k.clov + e * st + s);
+            for (int e = 0; e < 18; e++) copy_async(stage + e * LQ_HOP_THREADS, k.clov + (18 * half + e) * st + s);
             copy_commit();
         }
         const int ra = d < 4 ? 1 : 0;
@@ -793,124 +796,126 @@ __device__ __forceinline__ void hop_df_body(const Geom &g, const HopArgs<df64> &
         nb = nb1;
         flip = flip1;
     }
+    // each half hands the other its sums of the other's spins, through the second
+    // link buffer, which the last direction has left
 #pragma unroll
-    for (int i = 0; i < 12; i++) acc[i] = dl_cnorm(acc[i]);
-    if (MODE != HOP_PREP) {
-        // the first 12 vectors of the second clover block go where the links were
-#pragma unroll
-        for (int a = 0; a < 3; a++) used(acc[a]);
-#pragma unroll
-        for (int e = 0; e < 12; e++) copy_async(stage + (18 + e) * LQ_HOP_THREADS, k.clov + (18 + e) * st + s);
-        copy_commit();
-        copy_wait<1>();
+    for (int i = 0; i < 6; i++) {
+        const cx<df64> v = half ? acc[i] : acc[6 + i];
+        stage[(kDfLink + 9 + i) * LQ_HOP_THREADS] = make_float4(v.re.hi, v.im.hi, v.re.lo, v.im.lo);
     }
+    __syncthreads();
+    cx<df64> a6[6], y[6];
+    const float4 *other = stage + (half ? -kDfSites : kDfSites);
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        const float4 t = other[(kDfLink + 9 + i) * LQ_HOP_THREADS];
+        a6[i] = half ? acc[6 + i] : acc[i];
+        dl_cadd(a6[i], {df64(t.x, t.z), df64(t.y, t.w)});
+        a6[i] = dl_cnorm(a6[i]);
+    }
+    if (MODE != HOP_PREP) copy_wait<0>();
 
-    // the site term, one 6x6 clover block (spins 0,1 then 2,3) at a time: six
-    // components of the output are formed and stored per block (register
-    // arrays are selected by the block, never indexed by it)
-#pragma unroll 1
-    for (int blk = 0; blk < 2; blk++) {
-        const long long o = (long long)blk * 6 * st + s;
-        auto Cb = [&](int e) {   // vector e of the clover block
-            if (blk && e >= 12) return ldg(k.clov + (18 + e) * st + s);
-            const float4 t = stage[(18 * blk + e) * LQ_HOP_THREADS];
-            return df2(t.x, t.z, t.y, t.w);
-        };
-        if (blk && MODE != HOP_PREP) copy_wait<0>();
-        cx<df64> a6[6], y[6];
+    // the site term of the half's two spins, one 6x6 clover block
+    const long long o = (long long)half * 6 * st + s;
+    auto Cb = [&](int e) {   // vector e of the clover block
+        const float4 t = stage[e * LQ_HOP_THREADS];
+        return df2(t.x, t.z, t.y, t.w);
+    };
+    if (MODE == HOP_K1) {   // y = C (-1/2 acc)
 #pragma unroll
-        for (int i = 0; i < 6; i++) a6[i] = blk ? acc[6 + i] : acc[i];
-        if (MODE == HOP_K1) {   // y = C (-1/2 acc)
+        for (int i = 0; i < 6; i++) {
+            a6[i] = {dl_scale2(a6[i].re, -0.5f), dl_scale2(a6[i].im, -0.5f)};
+            y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+        }
+        herm6_fma_df(Cb, a6, y);
 #pragma unroll
-            for (int i = 0; i < 6; i++) {
-                a6[i] = {dl_scale2(a6[i].re, -0.5f), dl_scale2(a6[i].im, -0.5f)};
-                y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-            }
+        for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
+    } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL || MODE == HOP_RES) {   // y = C x +- 1/2 acc
+        const float f = (MODE == HOP_FULL || MODE == HOP_RES) ? -0.5f : 0.5f;
+        cx<df64> x6[6];
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            x6[i] = df2_cx(in2[o + i * st]);
+            y[i] = {dl_scale2(a6[i].re, f), dl_scale2(a6[i].im, f)};
+        }
+        herm6_fma_df(Cb, x6, y);
+#pragma unroll
+        for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
+        if (MODE == HOP_RICH) {   // x + omega (b - D x)
+#pragma unroll
+            for (int i = 0; i < 6; i++) y[i] = x6[i] + k.omega * (df2_cx(ldg(bv + o + i * st)) - y[i]);
+        }
+        if (MODE == HOP_RES) {   // b - D x
+#pragma unroll
+            for (int i = 0; i < 6; i++) y[i] = df2_cx(ldg(bv + o + i * st)) - y[i];
+        }
+    } else {   // y = in2 + 1/2 acc, and for the reconstruction C^{-1} of that
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            cx<df64> t = df2_cx(in2[o + i * st]);
+            dl_cadd(t, {dl_scale2(a6[i].re, 0.5f), dl_scale2(a6[i].im, 0.5f)});
+            a6[i] = dl_cnorm(t);
+        }
+        if (MODE == HOP_RECON || MODE == HOP_RECON_RES) {
+#pragma unroll
+            for (int i = 0; i < 6; i++) y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
             herm6_fma_df(Cb, a6, y);
 #pragma unroll
             for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
-        } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL || MODE == HOP_RES) {   // y = C x +- 1/2 acc
-            const float f = (MODE == HOP_FULL || MODE == HOP_RES) ? -0.5f : 0.5f;
-            cx<df64> x6[6];
+            if (MODE == HOP_RECON_RES) {   // the parity's residual u - C x_o of the x_o just formed
+                cx<df64> z[6];
 #pragma unroll
-            for (int i = 0; i < 6; i++) {
-                x6[i] = df2_cx(in2[o + i * st]);
-                y[i] = {dl_scale2(a6[i].re, f), dl_scale2(a6[i].im, f)};
+                for (int i = 0; i < 6; i++) z[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
+                herm6_fma_df([&](int e) { return ldg(k.clov2 + ((long long)half * 18 + e) * st + s); }, y, z);
+#pragma unroll
+                for (int i = 0; i < 6; i++)
+                    if (on) out2[o + i * st] = cx_df2(a6[i] - dl_cnorm(z[i]));
             }
-            herm6_fma_df(Cb, x6, y);
-#pragma unroll
-            for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
-            if (MODE == HOP_RICH) {   // x + omega (b - D x)
-#pragma unroll
-                for (int i = 0; i < 6; i++) y[i] = x6[i] + k.omega * (df2_cx(ldg(bv + o + i * st)) - y[i]);
-            }
-            if (MODE == HOP_RES) {   // b - D x
-#pragma unroll
-                for (int i = 0; i < 6; i++) y[i] = df2_cx(ldg(bv + o + i * st)) - y[i];
-            }
-        } else {   // y = in2 + 1/2 acc, and for the reconstruction C^{-1} of that
-#pragma unroll
-            for (int i = 0; i < 6; i++) {
-                cx<df64> t = df2_cx(in2[o + i * st]);
-                dl_cadd(t, {dl_scale2(a6[i].re, 0.5f), dl_scale2(a6[i].im, 0.5f)});
-                a6[i] = dl_cnorm(t);
-            }
-            if (MODE == HOP_RECON || MODE == HOP_RECON_RES) {
-#pragma unroll
-                for (int i = 0; i < 6; i++) y[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-                herm6_fma_df(Cb, a6, y);
-#pragma unroll
-                for (int i = 0; i < 6; i++) y[i] = dl_cnorm(y[i]);
-                if (MODE == HOP_RECON_RES) {   // the parity's residual u - C x_o of the x_o just formed
-                    cx<df64> z[6];
-#pragma unroll
-                    for (int i = 0; i < 6; i++) z[i] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
-                    herm6_fma_df([&](int e) { return ldg(k.clov2 + ((long long)blk * 18 + e) * st + s); }, y, z);
-#pragma unroll
-                    for (int i = 0; i < 6; i++) out2[o + i * st] = cx_df2(a6[i] - dl_cnorm(z[i]));
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 6; i++) y[i] = a6[i];
-            }
-        }
-        if (IO & kNat) {
-            // through the vectors of the staging area that block 0 has left (each
-            // lane's column turned by the component, against bank conflicts)
-            const int lane = threadIdx.x & 31;
-            double2 *tile = reinterpret_cast<double2 *>(stage - lane);
-            auto at = [](int r, int q) { return q * LQ_HOP_THREADS + ((r + q) & 31); };
-            const unsigned flip = blk ? k.nat.flip : 0u;
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 6; i++) {
-                const double2 d = nat_value((const df2 *)nullptr, y[i]);
-                tile[at(lane, i)] = make_double2(flip_sign64(d.x, flip), flip_sign64(d.y, flip));
-            }
-            __syncwarp();
-            nat_write6(k.nat, tile, at, s - min(lane, nvalid - 1), nvalid, c.x & 1, blk);
-        } else if (IO & kOut32) {
-            float4 *f = reinterpret_cast<float4 *>(out) + (long long)blk * 3 * st + s;
-#pragma unroll
-            for (int i = 0; i < 3; i++)
-                f[i * st] = make_float4(df_to_float(y[2 * i].re), df_to_float(y[2 * i].im), df_to_float(y[2 * i + 1].re),
-                                        df_to_float(y[2 * i + 1].im));
         } else {
 #pragma unroll
-            for (int i = 0; i < 6; i++) out[o + i * st] = cx_df2(y[i]);
+            for (int i = 0; i < 6; i++) y[i] = a6[i];
         }
+    }
+    if (IO & kNat) {
+        // through the vectors that the clover block has left (each
+        // lane's column turned by the component, against bank conflicts)
+        const int lane = threadIdx.x & 31;
+        double2 *tile = reinterpret_cast<double2 *>(stage - lane);
+        auto at = [](int r, int q) { return q * LQ_HOP_THREADS + ((r + q) & 31); };
+        const unsigned flip = half ? k.nat.flip : 0u;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+            const double2 d = nat_value((const df2 *)nullptr, y[i]);
+            tile[at(lane, i)] = make_double2(flip_sign64(d.x, flip), flip_sign64(d.y, flip));
+        }
+        __syncwarp();
+        nat_write6(k.nat, tile, at, s - min(lane, nvalid - 1), nvalid, c.x & 1, half);
+    } else if (IO & kOut32) {
+        float4 *f = reinterpret_cast<float4 *>(out) + (long long)half * 3 * st + s;
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+            if (on) f[i * st] = make_float4(df_to_float(y[2 * i].re), df_to_float(y[2 * i].im), df_to_float(y[2 * i + 1].re),
+                                    df_to_float(y[2 * i + 1].im));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 6; i++)
+            if (on) out[o + i * st] = cx_df2(y[i]);
     }
 }
 
-// Three resident blocks per SM (168 registers, 61 KB of staging each): K1 / K2
-// take 158 / 171 us on 24^3 x 48 (0.65 of the copy bandwidth) against 168 / 178
-// at two; 187 / 193 before the staging and 214 / 215 with scalar arithmetic.
+// Two threads per output site and right-hand side: the first takes the directions
+// along x and y and the site term of spins 0 and 1, the second those along z and t
+// and spins 2 and 3.  One thread's chain is half as long so, which a lattice of
+// about one wave of blocks waits for, and the sums need fewer registers: lq_apply of
+// D_S takes 45.7 us on 18x10x14x22 and 350 on 24^3 x 48, against 56.3 and 367 with
+// one thread a site (whose K1 / K2 took 158 / 171 us on 24^3 x 48, 187 / 193 before
+// the staging and 214 / 215 with scalar arithmetic).  Three resident blocks per SM
+// (61 KB of staging each).  The right-hand sides of a site block are consecutive
+// blocks, so its links and clover come from L2 for all but the first.
 #ifndef LQ_DF_MINB
 #define LQ_DF_MINB 3
 #endif
-// One thread per output site and right-hand side; the right-hand sides of a
-// site block are consecutive blocks, so its links and clover come from L2 for
-// all but the first.
 template <int MODE, int IO>
 __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(const __grid_constant__ Geom g,
                                                                 const __grid_constant__ HopArgs<df64> k)
@@ -918,15 +923,10 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(cons
     extern __shared__ float4 df_stage[];
     after_previous();
     const unsigned sb = blockIdx.x / (unsigned)k.nrhs;
-    long long s = sb * (long long)LQ_HOP_THREADS + threadIdx.x;
-    int nv = 0;
-    if (IO & kNat) {   // warps stay whole (warp_site)
-        nv = (int)min(32LL, g.Vh - (s - (threadIdx.x & 31)));
-        if (nv <= 0) return;
-        s = min(s, g.Vh - 1);
-    } else if (s >= g.Vh) {
-        return;
-    }
+    // blocks stay whole: threads beyond the last site shadow it
+    long long s = sb * (long long)kDfSites + threadIdx.x % kDfSites;
+    const int nv = (int)min(32LL, g.Vh - (s - (threadIdx.x & 31)));
+    s = min(s, g.Vh - 1);
     const Coords c = cb_coords(g, s, k.pout);
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs;
     hop_df_body<MODE, IO>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
@@ -988,22 +988,24 @@ static void launch_hop(const Exec &e, const HopCall &c)
     // FP64 blocks are one warp: the FP64 pipe is the bound, so the sites have to
     // spread evenly over the SMs (D_S on 16^4: 172 us with 64 threads, 155 with 32)
     constexpr int threads = std::is_same<R, double>::value ? LQ_F64_THREADS : LQ_HOP_THREADS;
-    const unsigned blocks = (unsigned)((e.g.Vh + threads - 1) / threads);
+    constexpr int sites = std::is_same<R, df64>::value ? kDfSites : threads;   // of a block
+    const unsigned blocks = (unsigned)((e.g.Vh + sites - 1) / sites);
     k.nat = nat_of(c);
     if constexpr (std::is_same<R, df64>::value)
     {
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
-        auto launch = [&](auto kernel) {
+        auto launch = [&](auto io) {
+            auto kernel = hop_df_kernel<MODE, decltype(io)::value>;
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
             launch_after(e, c.after, kernel, blocks * (unsigned)c.nrhs, LQ_HOP_THREADS, sm, e.g, k);
         };
         if constexpr (MODE == HOP_PREP)
-            if (c.out32) return launch(hop_df_kernel<MODE, kOut32>);
+            if (c.out32) return launch(std::integral_constant<int, kOut32>());
         if constexpr (MODE == HOP_RECON)
-            if (c.in32) return launch(hop_df_kernel<MODE, kNat | kIn32>);
+            if (c.in32) return launch(std::integral_constant<int, kNat | kIn32>());
         if constexpr (nat_mode(MODE))
-            if (c.nat) return launch(hop_df_kernel<MODE, kNat>);
-        launch(hop_df_kernel<MODE, 0>);
+            if (c.nat) return launch(std::integral_constant<int, kNat>());
+        launch(std::integral_constant<int, 0>());
     }
     else
     {

@@ -7,7 +7,7 @@
 //   2. warp c < 12 sums the eight contributions to component c;
 //   3. warp c forms component c of the site term, one row of a 6x6 clover block,
 //      whose entries it loaded before step 1.
-// The operations and their order are those of the one-thread kernels.
+// The operations are those of the larger lattices' kernels.
 //
 // lq_apply of D_S in us, twelve threads against one and before the launches
 // overlapped (launch_after: df64 at 2048 sites 18.8 -> 14.4), at 2048 sites a
@@ -340,10 +340,11 @@ static void launch_split(const Exec &e, const HopCall &c)
 
 bool hop_split_takes(const Geom &g, int prec, int nrhs)
 {
-    // sites up to which twelve threads are the faster: at 16384 df64 42.9 / 43.2 us
-    // and FP32 25.9 / 27.6, at 18432 df64 44.7 / 43.3; FP64 86 / 88 at 10368 and
+    // sites up to which twelve threads are the faster (for df64 than two): df64
+    // 23.0 / 24.1 us at 9216, 31.4 / 31.1 at 13824, 39.2 / 35.1 at 16384; FP32
+    // 25.9 / 27.6 at 16384 and 31.0 / 29.0 at 24576; FP64 86 / 88 at 10368 and
     // 114 / 92 at 16384; BF16 23.8 / 24.9 at 10368 and 26.9 / 24.9 at 13824
-    const long long most = prec == P16 ? 10368 : prec == P64 ? 12288 : 16384;
+    const long long most = prec == P16 ? 10368 : prec == P32 ? 16384 : 12288;
     return g.Vh * nrhs <= most;
 }
 
