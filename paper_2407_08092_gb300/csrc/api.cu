@@ -307,16 +307,17 @@ void op_full(lq_ctx *c, int prec, const void *ie, const void *io, void *nat)
 }
 
 // bhat_e = b_e - D_eo D_oo^{-1} b_o
-// (out32: bhat is an FP32 field)
-void op_prepare(lq_ctx *c, int prec, const void *be, const void *bo, void *bhat, void *t, bool out32 = false)
+// (out32: bhat is an FP32 field; n: of n consecutive fields)
+void op_prepare(lq_ctx *c, int prec, const void *be, const void *bo, void *bhat, void *t, bool out32 = false, int n = 1)
 {
     Exec e = c->ex();
-    clover_mul(e, prec, Cip(c, prec), bo, t);
+    clover_mul(e, prec, Cip(c, prec), bo, t, n);
     HopCall p = hopcall(c, HOP_PREP, prec, 0);
     p.in = t;
     p.in2 = be;
     p.out = bhat;
     p.out32 = out32;
+    p.nrhs = n;
     hop(e, p);
 }
 
@@ -335,8 +336,9 @@ void op_reconstruct(lq_ctx *c, int prec, const void *bo, const void *xe, void *x
 // The reconstruction of Eq. 2 together with the full system's residual r = b - D x
 // (prec FP64 or df64): x_o = D_oo^{-1} u with u = b_o - D_oe x_e, and in the same
 // launch r_o = u - D_oo x_o; then r_e = b_e - D_ee x_e - D_eo x_o in one launch.
+// (n: of n consecutive fields)
 void op_reconstruct_residual(lq_ctx *c, int prec, const void *be, const void *bo, const void *xe, void *xo,
-                             void *re, void *ro)
+                             void *re, void *ro, int n = 1)
 {
     Exec e = c->ex();
     HopCall r = hopcall(c, HOP_RECON_RES, prec, 1);
@@ -346,6 +348,7 @@ void op_reconstruct_residual(lq_ctx *c, int prec, const void *be, const void *bo
     r.clov = Cip(c, prec);
     r.clov2 = Cp(c, prec, 1);
     r.out2 = ro;
+    r.nrhs = n;
     hop(e, r);
     HopCall q = hopcall(c, HOP_RES, prec, 0);
     q.in = xo;
@@ -353,6 +356,7 @@ void op_reconstruct_residual(lq_ctx *c, int prec, const void *be, const void *bo
     q.b = be;
     q.out = re;
     q.clov = Cp(c, prec, 0);
+    q.nrhs = n;
     hop(e, q);
 }
 
@@ -1930,8 +1934,8 @@ lq_status lq_solve_group(lq_group *G, const lq_solver_params *p, const int *n_rh
             for (int r = 0; r < n; r++) {
                 import_full(e, PDF, (const char *)b[l] + r * q.nat, q.BE + r * q.fw, q.BO + r * q.fw);
                 import_full(e, PDF, (const char *)x[l] + r * q.nat, q.XE + r * q.fw, q.XO + r * q.fw);
-                op_prepare(ml, PDF, q.BE + r * q.fw, q.BO + r * q.fw, q.BH + r * q.fw, q.T);
             }
+            op_prepare(ml, PDF, q.BE, q.BO, q.BH, q.T, false, n);
         }
         // df64 norms of one field per right-hand side, all members, into out[N]
         auto norms = [&](char *MW::*f, std::vector<double> &out) {
@@ -1979,10 +1983,7 @@ lq_status lq_solve_group(lq_group *G, const lq_solver_params *p, const int *n_rh
             if (all || it == p->max_restarts) break;
             // correction: D_S e = R to smooth_tol (relative) with batched FP32 GMRES
             for (int l = 0; l < M; l++) {
-                Exec e = G->mem[l]->ex();
-                const long long fs = 6 * G->mem[l]->g.stride;
-                for (int r = 0; r < n_rhs[l]; r++)
-                    convert(e, PDF, w[l].R + r * w[l].fw, P32, (float4 *)G->B + G->off[l] + r * fs);
+                convert(G->mem[l]->ex(), PDF, w[l].R, P32, (float4 *)G->B + G->off[l], n_rhs[l]);
             }
             ck(c, cudaMemsetAsync(G->X, 0, (size_t)G->mf * 16, G->st), "cudaMemsetAsync");
             for (int k = 0; k < N; k++) {
@@ -2012,39 +2013,30 @@ lq_status lq_solve_group(lq_group *G, const lq_solver_params *p, const int *n_rh
             for (int l = 0; l < M; l++) {
                 lq_ctx *ml = G->mem[l];
                 Exec e = ml->ex();
-                const long long fs = 6 * ml->g.stride;
-                for (int r = 0; r < n_rhs[l]; r++)
-                    convert(e, P32, (const float4 *)G->X + G->off[l] + r * fs, PDF, w[l].E + r * w[l].fw);
+                convert(e, P32, (const float4 *)G->X + G->off[l], PDF, w[l].E, n_rhs[l]);
                 axpby(e, PDF, 1.0, 0.0, w[l].E, 1.0, 0.0, w[l].XE, n_rhs[l]);
             }
         }
         not_conv = !all;
-        // reconstruct (Eq. 2), export, true residual of every right-hand side
+        // reconstruct (Eq. 2), export, true residual of every right-hand side (even
+        // part into R, odd into E, which the iteration has left)
         for (int l = 0; l < M; l++) {
             lq_ctx *ml = G->mem[l];
-            Exec e = ml->ex();
             const MW &q = w[l];
-            void *ye = field(ml, PDF, "bw:ye"), *yo = field(ml, PDF, "bw:yo");
-            for (int r = 0; r < n_rhs[l]; r++) {
-                const int k = G->first[l] + r;
-                op_reconstruct_residual(ml, PDF, q.BE + r * q.fw, q.BO + r * q.fw, q.XE + r * q.fw,
-                                        q.XO + r * q.fw, ye, yo);
-                export_full(e, PDF, q.XE + r * q.fw, q.XO + r * q.fw, (char *)x[l] + r * q.nat);
-                norm2(e, PDF, ye, ml->red, 0);
-                norm2(e, PDF, yo, ml->red, 1);
-                norm2(e, PDF, q.BE + r * q.fw, ml->red, 2);
-                norm2(e, PDF, q.BO + r * q.fw, ml->red, 3);
-                reduce_finish(e, ml->red, 0, 4);
-                const double *hv = fetch(ml, 0, 4);
-                const double bb = hv[4] + hv[6];
-                st[k].rel_resid_true = bb > 0 ? std::sqrt((hv[0] + hv[2]) / bb) : 0.0;
-                if (!std::isfinite(st[k].rel_resid_true)) fail(c, LQ_ERR_NAN, "NaN/Inf in a true residual");
-                st[k].cycles = outer[k];
-                st[k].iters = outer[k];
-                st[k].inner_iters = inner[k];
-            }
+            op_reconstruct_residual(ml, PDF, q.BE, q.BO, q.XE, q.XO, q.R, q.E, n_rhs[l]);
+            for (int r = 0; r < n_rhs[l]; r++)
+                export_full(ml->ex(), PDF, q.XE + r * q.fw, q.XO + r * q.fw, (char *)x[l] + r * q.nat);
         }
-        ck(c, cudaStreamSynchronize(G->st), "cudaStreamSynchronize");
+        std::vector<double> ro;
+        norms(&MW::R, rn);
+        norms(&MW::E, ro);
+        for (int k = 0; k < N; k++) {
+            st[k].rel_resid_true = bn[k] > 0 ? std::sqrt(rn[k] * rn[k] + ro[k] * ro[k]) / bn[k] : 0.0;
+            if (!std::isfinite(st[k].rel_resid_true)) fail(c, LQ_ERR_NAN, "NaN/Inf in a true residual");
+            st[k].cycles = outer[k];
+            st[k].iters = outer[k];
+            st[k].inner_iters = inner[k];
+        }
     });
     if (stats) {
         const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();

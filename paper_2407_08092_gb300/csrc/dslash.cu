@@ -961,6 +961,8 @@ __global__ void __launch_bounds__(256) clover_mul_kernel(Geom g, const typename 
 {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.Vh) return;
+    in += blockIdx.y * St<R>::SPINOR_VECS * g.stride;
+    out += blockIdx.y * St<R>::SPINOR_VECS * g.stride;
     cx<R> x[12], y[12];
     load_spinor_rw(in, g.stride, s, x);
     clover_apply<R>(C, g.stride, s, x, y);
@@ -1163,11 +1165,12 @@ void hop(const Exec &e, const HopCall &c)
 #undef LQ_CASE
 }
 
-void clover_mul(const Exec &e, int prec, const void *clov, const void *in, void *out)
+void clover_mul(const Exec &e, int prec, const void *clov, const void *in, void *out, int nfields)
 {
-    Launch L_(e, K_HOP_OTHER, (double)e.g.Vh * (prec != P32 ? 192.0 * 2 + 576.0 : 96.0 * 2 + 288.0),
-              (double)e.g.Vh * 552);
-    const unsigned blocks = (unsigned)((e.g.Vh + 255) / 256);
+    Launch L_(e, K_HOP_OTHER,
+              (double)e.g.Vh * (prec != P32 ? nfields * 192.0 * 2 + 576.0 : nfields * 96.0 * 2 + 288.0),
+              (double)e.g.Vh * nfields * 552);
+    const dim3 blocks((unsigned)((e.g.Vh + 255) / 256), nfields);
     if (prec == P64)
         clover_mul_kernel<double><<<blocks, 256, 0, e.st>>>(e.g, (const double2 *)clov, (const double2 *)in,
                                                            (double2 *)out);

@@ -318,10 +318,13 @@ __global__ void df2d_kernel(Geom g, const df2 *__restrict__ in, double2 *out)
     for (int c = 0; c < 12; c++) out[c * g.stride + s] = from_df2(ldg(in + c * g.stride + s));
 }
 // FP32 -> df64 is exact (lo = 0); df64 -> FP32 rounds hi + lo once
+// (field blockIdx.y of consecutive ones)
 __global__ void f2df_kernel(Geom g, const float4 *__restrict__ in, df2 *out)
 {
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.Vh) return;
+    in += blockIdx.y * 6 * g.stride;
+    out += blockIdx.y * 12 * g.stride;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
         const float4 t = __ldg(in + k * g.stride + s);
@@ -333,6 +336,8 @@ __global__ void df2f_kernel(Geom g, const df2 *__restrict__ in, float4 *out)
 {
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.Vh) return;
+    in += blockIdx.y * 12 * g.stride;
+    out += blockIdx.y * 6 * g.stride;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
         const df2 a = ldg(in + (2 * k) * g.stride + s), b = ldg(in + (2 * k + 1) * g.stride + s);
@@ -341,7 +346,7 @@ __global__ void df2f_kernel(Geom g, const df2 *__restrict__ in, float4 *out)
     }
 }
 
-void convert(const Exec &e, int from, const void *in, int to, void *out)
+void convert(const Exec &e, int from, const void *in, int to, void *out, int nfields)
 {
     if (from == P16 || to == P16) {
         bf16_convert(e, from, in, to, out);
@@ -351,15 +356,15 @@ void convert(const Exec &e, int from, const void *in, int to, void *out)
         copy(e, from, in, out);
         return;
     }
-    const double bytes = (double)e.g.Vh * ((from == P32 ? 96 : 192) + (to == P32 ? 96 : 192));
+    const double bytes = (double)e.g.Vh * nfields * ((from == P32 ? 96 : 192) + (to == P32 ? 96 : 192));
     Launch L_(e, K_LAYOUT, bytes);
     const unsigned b = nblk(e.g.Vh, 256);
     if (from == P64 && to == P32) d2f_kernel<<<b, 256, 0, e.st>>>(e.g, (const double2 *)in, (float4 *)out);
     else if (from == P32 && to == P64) f2d_kernel<<<b, 256, 0, e.st>>>(e.g, (const float4 *)in, (double2 *)out);
     else if (from == P64 && to == PDF) d2df_kernel<<<b, 256, 0, e.st>>>(e.g, (const double2 *)in, (df2 *)out);
     else if (from == PDF && to == P64) df2d_kernel<<<b, 256, 0, e.st>>>(e.g, (const df2 *)in, (double2 *)out);
-    else if (from == P32 && to == PDF) f2df_kernel<<<b, 256, 0, e.st>>>(e.g, (const float4 *)in, (df2 *)out);
-    else df2f_kernel<<<b, 256, 0, e.st>>>(e.g, (const df2 *)in, (float4 *)out);
+    else if (from == P32 && to == PDF) f2df_kernel<<<dim3(b, nfields), 256, 0, e.st>>>(e.g, (const float4 *)in, (df2 *)out);
+    else df2f_kernel<<<dim3(b, nfields), 256, 0, e.st>>>(e.g, (const df2 *)in, (float4 *)out);
 }
 
 // gamma_5 = diag(1, 1, -1, -1): negate the components of spins 2 and 3

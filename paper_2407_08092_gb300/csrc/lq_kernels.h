@@ -126,8 +126,9 @@ void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo);
 void export_full(const Exec &e, int prec, const void *fe, const void *fo, void *nat);
 // the rows of one parity of a natural full field from an FP32 field (dslash.cu)
 void export_parity(const Exec &e, const void *f, int parity, void *nat);
-// precision conversion between internal fields
-void convert(const Exec &e, int from, const void *in, int to, void *out);
+// precision conversion between internal fields (nfields consecutive ones between
+// FP32 and df64)
+void convert(const Exec &e, int from, const void *in, int to, void *out, int nfields = 1);
 // out = g5 in (negates spins 2 and 3); in == out allowed
 void gamma5(const Exec &e, int prec, const void *in, void *out);
 
@@ -263,8 +264,9 @@ void hop_group(const Exec &e, int mode, const LatDesc *desc, const int4 *tiles, 
 // right-hand sides sharing links and clover
 double hop_bytes(int mode, int prec, int nrhs, double sites);
 double hop_flops(int mode, double site_rhs);
-// out = C in (site-diagonal apply of packed blocks of one parity)
-void clover_mul(const Exec &e, int prec, const void *clov, const void *in, void *out);
+// out = C in (site-diagonal apply of packed blocks of one parity) for nfields
+// consecutive fields
+void clover_mul(const Exec &e, int prec, const void *clov, const void *in, void *out, int nfields = 1);
 
 // ---- BLAS-1 and reductions (blas.cu) ----------------------------------------
 // All vectors are internal fields of one parity (or n_vec of them spaced by
