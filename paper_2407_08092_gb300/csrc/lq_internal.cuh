@@ -167,8 +167,8 @@ __device__ __forceinline__ df64 &operator+=(df64 &a, df64 b) { return a = a + b;
 // significand m: hi = m's top 24 bits rounded to nearest even, and the
 // remainder m - hi, an integer R with |R| <= 2^28 in units of 2^(e-52), gives
 // lo = RN(R) 2^(e-52) -- the same values as hi = (float)d, lo = (float)(d - hi).
-// Zero, subnormal, very small or very large magnitudes and non-finite values
-// take the FP64 route, kept out of line: inlined, the compiler evaluates it for
+// Subnormal, very small or very large magnitudes and non-finite values take the
+// FP64 route, kept out of line: inlined, the compiler evaluates it for
 // every value and selects (four FP64-pipe operations per double, which then
 // bound the link import).
 static __device__ __noinline__ df64 df_split_rare(double d) { return df64(d); }
@@ -178,7 +178,10 @@ __device__ __forceinline__ df64 df_split(double d)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(d);
     const int e = (int)((b >> 52) & 0x7FF) - 1023;
-    if (e < -74 || e > 126) return df_split_rare(d);
+    if (e < -74 || e > 126) {
+        if ((b << 1) == 0) return df64(__uint_as_float((unsigned)(b >> 32)), 0.0f);   // +-0: point sources, zero guesses
+        return df_split_rare(d);
+    }
     const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
     unsigned q = (unsigned)(m >> 29);             // 2^23 <= q < 2^24
     int R = (int)(m & 0x1FFFFFFFull);             // 0 <= R < 2^29
