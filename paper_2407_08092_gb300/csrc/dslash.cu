@@ -32,13 +32,9 @@ static_assert(LQ_HOP_THREADS == kHopBlock, "hopping block size");
 #define LQ_HOP_BOUNDS __launch_bounds__(LQ_HOP_THREADS)
 #endif
 
-#ifndef LQ_F64_THREADS
-#define LQ_F64_THREADS 32
-#endif
-
 // one hop: acc += (1 -+ g_mu) W psi(nb), W = U_mu(x) (SIGN -1) or U_mu(x-mu)^+ (SIGN +1);
 // `bsign` is the fermion boundary factor of this hop
-template <int MU, int SIGN, bool FIRST = false, typename R, typename SV, typename LV>
+template <int MU, int SIGN, typename R, typename SV, typename LV>
 __device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *psi, const LV *__restrict__ U,
                                         long long link_site, long long nb, long long stride, R bsign)
 {
@@ -46,7 +42,7 @@ __device__ __forceinline__ void hop_dir(cx<R> acc[12], const SV *psi, const LV *
     load_spinor_rw(psi, stride, nb, p);   // the kernel before wrote it: not through the read-only path (after_previous)
     cx<R> m[9];
     load_link(U, stride, MU, link_site, m);
-    hop_apply<MU, SIGN, FIRST>(acc, p, m, bsign);
+    hop_apply<MU, SIGN>(acc, p, m, bsign);
 }
 
 template <typename R>
@@ -98,15 +94,12 @@ __device__ __forceinline__ void store_nat(const NatOut &o, double2 *tile, const 
 template <typename R, int MODE, bool NAT = false, bool SCALED = false, typename SV, typename LV, typename CV>
 __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV *Uin, const CV *clov, R omega,
                                          const SV *in, const SV *in2, const SV *bv, SV *out, long long s,
-                                         const Coords &c, const CV *clov2 = nullptr, SV *out2 = nullptr,
-                                         const NatOut &nat = NatOut(), double2 *tile = nullptr, int nvalid = 0)
+                                         const Coords &c, const NatOut &nat = NatOut(), double2 *tile = nullptr, int nvalid = 0)
 {
     const long long st = g.stride;
     cx<R> acc[12];
-    constexpr bool SET = std::is_same<R, double>::value;   // FP32: the compiler's schedule is the better with a zeroed sum
-    if (!SET)
 #pragma unroll
-        for (int i = 0; i < 12; i++) acc[i] = {R(0), R(0)};
+    for (int i = 0; i < 12; i++) acc[i] = {R(0), R(0)};
     const R one = R(1);
 
     // x direction: the neighbour changes x, so its cb index is recomputed
@@ -115,7 +108,7 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
         const int xp = (c.x + 1 == g.L[0]) ? 0 : c.x + 1;
         const int xm = (c.x == 0) ? g.L[0] - 1 : c.x - 1;
         const long long nf = LQ_IDX(base + (xp >> 1), g.Vh, B_HOP_NB), nb = LQ_IDX(base + (xm >> 1), g.Vh, B_HOP_NB);
-        hop_dir<0, -1, SET>(acc, in, Uout, s, nf, st, one);
+        hop_dir<0, -1>(acc, in, Uout, s, nf, st, one);
         hop_dir<0, +1>(acc, in, Uin, nb, nb, st, one);
     }
     // y, z, t: x is unchanged, so the cb index moves by a fixed stride
@@ -148,11 +141,11 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
 #pragma unroll
         for (int i = 0; i < 12; i++) acc[i] = (SCALED ? R(-0.5) * omega : R(-0.5)) * acc[i];
         clover_apply<R>(clov, st, s, acc, v);
-    } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL || MODE == HOP_RES) {
+    } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL) {
         cx<R> x[12];
         load_spinor_rw(in2, st, s, x);
         clover_apply<R>(clov, st, s, x, v);
-        const R f = (MODE == HOP_FULL || MODE == HOP_RES) ? R(-0.5) : R(0.5);
+        const R f = MODE == HOP_FULL ? R(-0.5) : R(0.5);
 #pragma unroll
         for (int i = 0; i < 12; i++) v[i] = (SCALED ? omega * v[i] : v[i]) + f * acc[i];
         if (MODE == HOP_RICH) {
@@ -161,26 +154,13 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
 #pragma unroll
             for (int i = 0; i < 12; i++) v[i] = x[i] + omega * (bb[i] - v[i]);
         }
-        if (MODE == HOP_RES) {
-            cx<R> bb[12];
-            load_spinor(bv, st, s, bb);
-#pragma unroll
-            for (int i = 0; i < 12; i++) v[i] = bb[i] - v[i];
-        }
-    } else {   // HOP_PREP, HOP_RECON, HOP_RECON_RES
+    } else {   // HOP_PREP, HOP_RECON
         cx<R> y[12];
         load_spinor_rw(in2, st, s, y);
 #pragma unroll
         for (int i = 0; i < 12; i++) y[i] = y[i] + R(0.5) * acc[i];
-        if (MODE == HOP_RECON || MODE == HOP_RECON_RES) {
+        if (MODE == HOP_RECON) {
             clover_apply<R>(clov, st, s, y, v);
-            if (MODE == HOP_RECON_RES) {   // the parity's residual u - C x_o of the x_o just formed
-                cx<R> w[12];
-                clover_apply<R>(clov2, st, s, v, w);
-#pragma unroll
-                for (int i = 0; i < 12; i++) w[i] = y[i] - w[i];
-                store_spinor(out2, st, s, w);
-            }
         } else {
 #pragma unroll
             for (int i = 0; i < 12; i++) v[i] = y[i];
@@ -302,12 +282,9 @@ __device__ __forceinline__ void hop_site(const Geom &g, const HopArgs<R> &k)
     }
     const Coords c = cb_coords(g, s, k.pout);
     double2 *tile = NAT ? nat_tile + (threadIdx.x >> 5) * 32 * kNatRow : nullptr;
-    if constexpr (std::is_same<R, float>::value)   // links and clover read once: no L1 allocation
-        hop_body<R, MODE, NAT>(g, (const F4S *)k.Uout, (const F4S *)k.Uin, (const F4S *)k.clov, k.omega, k.in, k.in2,
-                               k.b, k.out, s, c, (const F4S *)nullptr, (float4 *)nullptr, k.nat, tile, nv);
-    else
-        hop_body<R, MODE, NAT>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, k.clov2, k.out2, k.nat,
-                               tile, nv);
+    // links and clover read once: no L1 allocation
+    hop_body<R, MODE, NAT>(g, (const F4S *)k.Uout, (const F4S *)k.Uin, (const F4S *)k.clov, k.omega, k.in, k.in2, k.b,
+                           k.out, s, c, k.nat, tile, nv);
 }
 template <typename R, int MODE, bool NAT>
 __global__ void LQ_HOP_BOUNDS hop_kernel(Geom g, HopArgs<R> k)
@@ -352,8 +329,8 @@ __device__ __forceinline__ void hop_site_bf(const Geom &g, const HopArgsBF &k)
         if (s >= g.Vh) return;
     }
     const Coords c = cb_coords(g, s, k.pout);
-    hop_body<float, MODE, NAT>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, (const F4S *)nullptr,
-                               (BfS4 *)nullptr, k.nat, NAT ? nat_tile + (threadIdx.x >> 5) * 32 * kNatRow : nullptr, nv);
+    hop_body<float, MODE, NAT>(g, k.Uout, k.Uin, k.clov, k.omega, k.in, k.in2, k.b, k.out, s, c, k.nat,
+                               NAT ? nat_tile + (threadIdx.x >> 5) * 32 * kNatRow : nullptr, nv);
 }
 template <int MODE>
 __global__ void LQ_HOP_BOUNDS hop_kernel_bf(Geom g, HopArgsBF k)
@@ -370,14 +347,6 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_bf_nat(Geom g, H
 
 // shared memory of a block's natural output
 constexpr size_t nat_smem(int threads) { return (size_t)threads * kNatRow * sizeof(double2); }
-static NatOut nat_of(const HopCall &c)
-{
-    NatOut o;
-    o.p = (double2 *)c.nat;
-    o.full = c.nat_full;
-    o.flip = c.nat_g5 ? 0x80000000u : 0u;
-    return o;
-}
 // the modes that end a call on natural fields
 constexpr bool nat_mode(int mode) { return mode == HOP_K2 || mode == HOP_FULL; }
 
@@ -394,14 +363,18 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     k.clov = (const F4S *)c.clov;
     k.omega = (float)c.omega;
     k.pout = c.pout;
-    k.nat = nat_of(c);
+    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
+    // Blocks brought in early are not spread as evenly over the SMs, which costs more
+    // than the gap between the launches while they are few: D_S 31.4 us overlapped and
+    // 29.0 not on 18x10x14x22, 37.2 and 36.7 on 16^3x32, but 54.9 and 58.7 on 20^3x32.
+    const bool after = c.after && blocks > 512;
     if constexpr (MODE == HOP_K2)
         if (c.nat) {
-            launch_after(e, c.after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
+            launch_after(e, after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
             return;
         }
-    launch_after(e, c.after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
+    launch_after(e, after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
 }
 
 // The batched hop over the right-hand sides of several lattices of different
@@ -948,9 +921,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS) export_parity_kernel(Geom g, c
 void export_parity(const Exec &e, const void *f, int parity, void *nat)
 {
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (96 + 192));
-    NatOut o;
-    o.p = (double2 *)nat;
-    o.full = 1;
+    const NatOut o = nat_out(nat, true, false);
     export_parity_kernel<<<(unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS), LQ_HOP_THREADS,
                            nat_smem(LQ_HOP_THREADS), e.st>>>(e.g, (const float4 *)f, parity, o);
 }
@@ -987,12 +958,9 @@ static void launch_hop(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)St<R>::SPINOR_VECS * e.g.stride;
-    // FP64 blocks are one warp: the FP64 pipe is the bound, so the sites have to
-    // spread evenly over the SMs (D_S on 16^4: 172 us with 64 threads, 155 with 32)
-    constexpr int threads = std::is_same<R, double>::value ? LQ_F64_THREADS : LQ_HOP_THREADS;
-    constexpr int sites = std::is_same<R, df64>::value ? kDfSites : threads;   // of a block
+    constexpr int threads = LQ_HOP_THREADS, sites = std::is_same<R, df64>::value ? kDfSites : threads;   // of a block
     const unsigned blocks = (unsigned)((e.g.Vh + sites - 1) / sites);
-    k.nat = nat_of(c);
+    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
     if constexpr (std::is_same<R, df64>::value)
     {
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);
@@ -1011,8 +979,8 @@ static void launch_hop(const Exec &e, const HopCall &c)
     }
     else
     {
-        // several right-hand sides of FP64 or FP32 fields: one launch each (the
-        // batched FP32 solve uses the work-table kernel instead)
+        // several right-hand sides of FP32 fields: one launch each (the batched
+        // solve uses the work-table kernel instead)
         for (int r = 0; r < c.nrhs; r++) {
             HopArgs<R> kr = k;
             const long long o = r * k.fs;
@@ -1020,7 +988,6 @@ static void launch_hop(const Exec &e, const HopCall &c)
             kr.in2 = k.in2 ? k.in2 + o : nullptr;
             kr.b = k.b ? k.b + o : nullptr;
             kr.out = k.out + o;
-            kr.out2 = k.out2 ? k.out2 + o : nullptr;
             const size_t sm = c.nat ? nat_smem(threads) : 0;
             auto launch = [&](auto nat) {
                 constexpr bool NAT = decltype(nat)::value;
@@ -1132,8 +1099,7 @@ void hop(const Exec &e, const HopCall &c)
 {
 #define LQ_CASE(M)                                                              \
     case M:                                                                     \
-        if (c.prec == P64) launch_hop<double, M>(e, c);                         \
-        else if (c.prec == P32) launch_hop<float, M>(e, c);                     \
+        if (c.prec == P32) launch_hop<float, M>(e, c);                          \
         else if (c.prec == P16) launch_hop_bf<M>(e, c);                         \
         else launch_hop<df64, M>(e, c);                                         \
         break;
@@ -1146,6 +1112,7 @@ void hop(const Exec &e, const HopCall &c)
                              96.0 * (c.in32 + c.out32);
     Launch L_(e, hop_class(c.mode, c.prec), (double)e.g.Vh * (site_bytes + nat_bytes), (double)e.g.Vh * c_hop_flops[c.mode] * c.nrhs);
     if (hop_split(e, c)) return;
+    if (c.prec == P64) return hop_f64(e, c);
     switch (c.mode) {
         LQ_CASE(HOP_K1)
         LQ_CASE(HOP_K2)
@@ -1154,12 +1121,10 @@ void hop(const Exec &e, const HopCall &c)
         LQ_CASE(HOP_PREP)
         LQ_CASE(HOP_RECON)
     case HOP_RES:   // FP64 and df64 only (the solve's full residual)
-        if (c.prec == P64) launch_hop<double, HOP_RES>(e, c);
-        else if (c.prec == PDF) launch_hop<df64, HOP_RES>(e, c);
+        if (c.prec == PDF) launch_hop<df64, HOP_RES>(e, c);
         break;
     case HOP_RECON_RES:
-        if (c.prec == P64) launch_hop<double, HOP_RECON_RES>(e, c);
-        else if (c.prec == PDF) launch_hop<df64, HOP_RECON_RES>(e, c);
+        if (c.prec == PDF) launch_hop<df64, HOP_RECON_RES>(e, c);
         break;
     }
 #undef LQ_CASE

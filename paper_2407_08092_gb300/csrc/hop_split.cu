@@ -331,9 +331,7 @@ static void launch_split(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)(spinor_bytes(e.g, c.prec) / sizeof(SV));
-    k.nat.p = (double2 *)c.nat;
-    k.nat.full = c.nat_full;
-    k.nat.flip = c.nat_g5 ? 0x80000000u : 0u;
+    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + kSplitSites - 1) / kSplitSites) * (unsigned)c.nrhs;
     launch_after(e, c.after, hop_split_kernel<R, MODE, SV, LV, CV>, blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.g, k);
 }

@@ -227,6 +227,7 @@ void hop(const Exec &e, const HopCall &c);
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
 // done, where the one-thread kernels are the faster ones
 bool hop_split(const Exec &e, const HopCall &c);
+void hop_f64(const Exec &e, const HopCall &c);   // FP64 (hop_f64.cu)
 bool hop_split_takes(const Geom &g, int prec, int nrhs);
 
 // One member lattice of a batched solve over lattices of different sizes: its

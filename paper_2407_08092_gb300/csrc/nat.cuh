@@ -15,6 +15,15 @@ struct NatOut {
     unsigned flip = 0;      // sign bit of spins 2 and 3 (gamma_5)
 };
 
+static inline NatOut nat_out(void *p, bool full, bool g5)
+{
+    NatOut o;
+    o.p = (double2 *)p;
+    o.full = full;
+    o.flip = g5 ? 0x80000000u : 0u;
+    return o;
+}
+
 __device__ __forceinline__ double flip_sign64(double d, unsigned bit)
 {
     return __hiloint2double(__double2hiint(d) ^ (int)bit, __double2loint(d));

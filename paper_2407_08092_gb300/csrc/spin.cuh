@@ -43,13 +43,14 @@ template <int MU, int SIGN, bool FIRST = false, typename R>
 __device__ __forceinline__ void reconstruct(cx<R> acc[12], const cx<R> u[6])
 {
     if constexpr (FIRST) {
-        static_assert(!FIRST || (MU == 0 && SIGN < 0), "the first direction of the sums is forward x");
+        static_assert(!FIRST || SIGN < 0, "the first direction of a sum is a forward one");
 #pragma unroll
         for (int a = 0; a < 3; a++) {
-            acc[a] = u[a];
-            acc[3 + a] = u[3 + a];
-            acc[6 + a] = tmi(u[3 + a]);
-            acc[9 + a] = tmi(u[a]);
+            const cx<R> u0 = u[a], u1 = u[3 + a];
+            acc[a] = u0;
+            acc[3 + a] = u1;
+            acc[6 + a] = MU == 0 ? tmi(u1) : MU == 1 ? -u1 : MU == 2 ? tmi(u0) : -u0;
+            acc[9 + a] = MU == 0 ? tmi(u0) : MU == 1 ? u0 : MU == 2 ? ti(u1) : -u1;
         }
     } else
 #pragma unroll
