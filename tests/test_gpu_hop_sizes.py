@@ -61,3 +61,27 @@ def test_smoother_and_solve(pair, prec):
     assert status == lqdd.LQ_OK
     true = np.linalg.norm(r - lat.dirac(pair.host(x))) / np.linalg.norm(r)
     assert true <= 1.001e-10 and abs(st.rel_resid_true - true) <= 1e-13
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3], ids=["f64", "f32", "df64", "bf16"])
+def test_point_source(pair, prec):
+    """Zeros of either sign take a route of their own into df64 and FP32."""
+    from paper_2407_08092_gb300 import lqdd
+    x = np.zeros((pair.Vh, 4, 3), dtype=np.complex128)
+    x[::3] = complex(-0.0, -0.0)
+    x[pair.Vh // 2, 1, 2] = 1.0
+    assert rel(pair.apply(lqdd.LQ_OP_SCHUR, prec, x), pair.lat.schur(x)) < TOL[prec]
+
+
+def test_batch_matches_oracle(pair):
+    """Preparation, residuals and reconstruction of several right-hand sides in one launch."""
+    from paper_2407_08092_gb300 import lqdd
+    n = 3
+    b = np.stack([synth.gaussian_spinor(pair.V, 7100 + r) for r in range(n)])
+    x = pair.torch.zeros((n, pair.V, 4, 3), dtype=pair.torch.complex128, device="cuda")
+    status, stats = lqdd.lq_solve_batch(pair.ctx, lqdd.make_batch_params(tol=1e-10, restart=16), n, pair.dev(b), x)
+    assert status == lqdd.LQ_OK
+    got = pair.host(x)
+    for r in range(n):
+        true = np.linalg.norm(b[r] - pair.lat.dirac(got[r])) / np.linalg.norm(b[r])
+        assert true <= 1.001e-10 and abs(stats[r].rel_resid_true - true) <= 1e-13
