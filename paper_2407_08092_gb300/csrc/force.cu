@@ -43,11 +43,13 @@
 
 namespace lq {
 
-// Resident blocks per SM asked of the two kernels: four (128 registers, some
-// spills outside the products) against three (168): 5.44 against 5.64 ms for
-// lq_force on 24^3 x 48, and 6.32 at two.
+// Resident blocks per SM asked of the two kernels.  The link kernel takes three (168
+// registers, 74 KB of staged factors each): lq_force on 24^3 x 48 takes 5.15 ms,
+// 5.20 at two and 5.42 with the factors read where they are used at four (128
+// registers).  The plaquette kernel: four (some spills outside the products), 0.2 ms
+// under three.
 #ifndef LQ_FLINK_MINB
-#define LQ_FLINK_MINB 4
+#define LQ_FLINK_MINB 3
 #endif
 #ifndef LQ_FLOOP_MINB
 #define LQ_FLOOP_MINB 4
@@ -173,7 +175,8 @@ __device__ __forceinline__ M3<df64> load_mat(const df2 *__restrict__ m, long lon
 // one row of a product added to a row of sums: s_j += sum_k r_k B_kj.  Each
 // product and each sum is renormalised: twelve products summed with their low
 // parts left to grow put the force 9.6e-15 from its 64-bit value, 6.2e-15 so
-// (5.2 against 5.6 ms on 24^3 x 48).
+// (a twentieth of the time; renormalising a link's sums after every second product
+// would save half of that, at 6.5e-15 and twice the largest error).
 __device__ __forceinline__ void row_fma(cx<df64> s[3], const cx<df64> r[3], const M3<df64> &B)
 {
 #pragma unroll
@@ -318,6 +321,47 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
     const df2 *Xx = parity ? Xo : Xe, *Yx = parity ? Yo : Ye;      // at x
     const df2 *Xn = parity ? Xe : Xo, *Yn = parity ? Ye : Yo;      // at x + mu
 
+    // The clover term's products h: plane (h / 4), plaquette at x (0) or x - nu (1),
+    // first or second product of the link's two,
+    //   U_mu = a: W2 E'^+, E Z^+    = c: V E', E^+ W    = d: E Z, W E'^+    = b: E^+ W2, V^+ E'
+    // (E: of the nu links; E' at z + mu).  Both factors are copied to shared memory
+    // one product ahead, the first during the hopping term; each thread reads only
+    // what it copied itself.
+    struct Product {
+        bool lower, down, second, efirst;   // lower: mu < nu; efirst: E is the left factor and sits at z
+    };
+    auto product = [&](int h) {
+        const int q = h >> 2, nu = q < mu ? q : q + 1;
+        Product r;
+        r.lower = mu < nu;
+        r.down = h & 2;
+        r.second = h & 1;
+        r.efirst = r.lower == r.second;
+        return r;
+    };
+    extern __shared__ float4 force_stage[];
+    float4 *stage = force_stage + threadIdx.x;
+    auto entry = [&](int h, int e) { return stage + ((h & 1) * 18 + e) * 128; };   // left factor 0..8, right 9..17
+    auto copy_product = [&](int h) {
+        const Product r = product(h);
+        const int q = h >> 2, nu = q < mu ? q : q + 1;
+        const int p = c_plane[r.lower ? mu * 4 + nu : nu * 4 + mu];
+        int z[4], zu[4];
+        step(g, c, nu, r.down ? -1 : 0, z);
+        step(g, z, mu, +1, zu);
+        const long long iz = S.site(g, z), iu = S.site(g, zu);
+        const int other = r.down ? (r.efirst ? (r.lower ? F_W : F_W2) : F_V) : (r.efirst ? F_Z : (r.lower ? F_W2 : F_W));
+        const df2 *E = S.at(p, r.lower ? F_EN : F_EM, r.efirst ? iz : iu), *O = S.at(p, other, iz);
+        const df2 *A = r.efirst ? E : O, *B = r.efirst ? O : E;
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            copy_async(entry(h, e), A + e * S.n);
+            copy_async(entry(h, 9 + e), B + e * S.n);
+        }
+        copy_commit();
+    };
+    copy_product(0);
+
     M3<df64> acc;
 #pragma unroll
     for (int k = 0; k < 9; k++) acc.a[k] = {df64(0.0f, 0.0f), df64(0.0f, 0.0f)};
@@ -367,33 +411,37 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
     // ---- clover term: the two plaquettes of each plane (mu, nu) that hold U_mu(x) ----
 #pragma unroll 1
     for (int h = 0; h < 12; h++) {
-        // plane (h / 4), plaquette at x (0) or x - nu (1), first or second product
-        const int q = h >> 2, nu = q < mu ? q : q + 1;
-        const bool down = h & 2, second = h & 1, lower = mu < nu;
-        const int p = c_plane[lower ? mu * 4 + nu : nu * 4 + mu];
-        int z[4], zu[4];
-        step(g, c, nu, down ? -1 : 0, z);
-        step(g, z, mu, +1, zu);
-        const long long iz = S.site(g, z), iu = S.site(g, zu);
-        // the operands of each product (E: of the nu links; E' at z + mu):
-        //   U_mu = a: W2 E'^+, E Z^+    = c: V E', E^+ W    = d: E Z, W E'^+    = b: E^+ W2, V^+ E'
-        const int e = lower ? F_EN : F_EM;
-        const bool efirst = lower == second;   // E is the left factor and sits at z
-        const int other = down ? (efirst ? (lower ? F_W : F_W2) : F_V) : (efirst ? F_Z : (lower ? F_W2 : F_W));
-        const df2 *E = S.at(p, e, efirst ? iz : iu), *O = S.at(p, other, iz);
-        const df2 *A = efirst ? E : O;
-        const bool dag = down && (efirst || !lower);
-        const M3<df64> B = load_mat(efirst ? O : E, S.n, !down && (efirst ? lower : true));
-        const unsigned sre = second ? 0x80000000u : 0u, sim = (second != dag) ? 0x80000000u : 0u;
+        if (h < 11) {
+            copy_product(h + 1);
+            copy_wait<1>();
+        } else {
+            copy_wait<0>();
+        }
+        const Product r = product(h);
+        const bool dag = r.down && (r.efirst || !r.lower), dagb = !r.down && (r.efirst ? r.lower : true);
+        const unsigned sre = r.second ? 0x80000000u : 0u, sim = (r.second != dag) ? 0x80000000u : 0u;
+        const unsigned sb = dagb ? 0x80000000u : 0u;
+        auto factor = [&](int at, bool t, int i, int k) {   // entry (i, k) of a factor as stored, or its transpose
+            const float4 v = *entry(h, at + (t ? k * 3 + i : i * 3 + k));
+            return cx<df64>{df64(v.x, v.z), df64(v.y, v.w)};
+        };
+        M3<df64> B;
 #pragma unroll
-        for (int i = 0; i < 3; i++) {   // the left factor one row at a time, with the product's sign
-            cx<df64> r[3];
+        for (int i = 0; i < 3; i++)
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                const cx<df64> t = df2_cx(ldg(A + (dag ? k * 3 + i : i * 3 + k) * S.n));
-                r[k] = {flip_sign(t.re, sre), flip_sign(t.im, sim)};
+                const cx<df64> t = factor(9, dagb, i, k);
+                B.a[i * 3 + k] = {t.re, flip_sign(t.im, sb)};
             }
-            row_fma(acc.a + 3 * i, r, B);
+#pragma unroll
+        for (int i = 0; i < 3; i++) {   // the left factor one row at a time, with the product's sign
+            cx<df64> row[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const cx<df64> t = factor(0, dag, i, k);
+                row[k] = {flip_sign(t.re, sre), flip_sign(t.im, sim)};
+            }
+            row_fma(acc.a + 3 * i, row, B);
         }
     }
 
@@ -462,7 +510,9 @@ void force_links(const Exec &e, const void *Udf[2], const void *X[2], const void
         // the hopping term's 2 x 4 x 9 outer-product entries
         Launch L_(e, K_FORCE, (double)ns * (2 * 192 + 36 * 144 + 4 * 144),
                   (double)ns * 4 * (12 * (198 + 18) + 2 * 4 * (9 * 8 + 12)));
-        force_link_kernel<<<dim3(blocks_of(ns, 128), 4), 128, 0, e.st>>>(
+        constexpr int sm = 2 * 18 * 128 * (int)sizeof(float4);
+        cudaFuncSetAttribute(force_link_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        force_link_kernel<<<dim3(blocks_of(ns, 128), 4), 128, sm, e.st>>>(
             g, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1], S, t0, ns, coef, (double2 *)G);
     }
 }
