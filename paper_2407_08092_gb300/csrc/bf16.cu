@@ -72,18 +72,6 @@ __global__ void bf16_to_df_kernel(Geom g, const BfS4 *__restrict__ in, df2 *out)
     store_spinor(out, g.stride, s, d);
 }
 
-// out = g5 in: spins 2, 3 (components 6..11) negated
-__global__ void bf16_gamma5_kernel(Geom g, const BfS4 *in, BfS4 *out)
-{
-    const long long s = blockIdx.x * 256LL + threadIdx.x;
-    if (s >= g.Vh) return;
-    cx<float> v[12];
-    load_spinor_rw(in, g.stride, s, v);
-#pragma unroll
-    for (int k = 6; k < 12; k++) v[k] = -v[k];
-    store_spinor(out, g.stride, s, v);
-}
-
 // y = a x + b y over nfields consecutive fields (complex a, b)
 __global__ void bf16_axpby_kernel(Geom g, int nfields, float ar, float ai, const BfS4 *x, float br, float bi,
                                   BfS4 *y)
@@ -131,12 +119,6 @@ void bf16_convert(const Exec &e, int from, const void *in, int to, void *out)
     } else {
         bf16_to_df_kernel<<<b, 256, 0, e.st>>>(e.g, (const BfS4 *)in, (df2 *)out);
     }
-}
-
-void bf16_gamma5(const Exec &e, const void *in, void *out)
-{
-    Launch L_(e, K_LAYOUT, (double)e.g.Vh * 2 * 48);
-    bf16_gamma5_kernel<<<nb256(e.g.Vh), 256, 0, e.st>>>(e.g, (const BfS4 *)in, (BfS4 *)out);
 }
 
 void bf16_axpby(const Exec &e, double ar, double ai, const void *x, double br, double bi, void *y, int nfields)

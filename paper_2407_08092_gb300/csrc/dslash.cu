@@ -1,7 +1,8 @@
 // The fused hopping kernels of the odd-even Wilson-clover operator.
 //
-// One thread per output site of one parity.  For each of the eight
-// directions the neighbour spinor is spin-projected onto a half spinor with
+// One thread per output site of one parity (FP32 and BF16 storage; the df64 form
+// below takes two, FP64 is hop_f64.cu and small lattices hop_split.cu).  For each
+// of the eight directions the neighbour spinor is spin-projected onto a half spinor with
 // (1 -+ g_mu), multiplied by the link (U_mu(x) forward, U_mu(x-mu)^+ backward)
 // and reconstructed into the 12-component accumulator; the epilogue then
 // applies the site-diagonal clover block (C or C^{-1}) and whatever BLAS-1
@@ -170,10 +171,6 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
     else store_spinor(out, st, s, v);
 }
 
-// One thread per output site.  The batched form (MULTI) loops over the
-// right-hand sides, so each site's links and clover block come from DRAM once
-// and from the caches for the other right-hand sides; it is a separate
-// instantiation so that the single right-hand-side kernel keeps its registers.
 // Two right-hand sides per thread (K1 and K2 of the batched hop): each link is
 // loaded once and transports both neighbour spinors.
 template <int MU, int SIGN>
@@ -305,7 +302,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_occ(Geom g, HopA
 }
 
 
-// BF16 spinors and links, FP32 clover and arithmetic (all modes)
+// BF16 spinors and links, FP32 clover and arithmetic (K1, K2, Richardson)
 struct HopArgsBF {
     const BfS4 *in, *in2, *b;
     BfS4 *out;
@@ -347,7 +344,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, 6) hop_kernel_bf_nat(Geom g, H
 
 // shared memory of a block's natural output
 constexpr size_t nat_smem(int threads) { return (size_t)threads * kNatRow * sizeof(double2); }
-// the modes that end a call on natural fields
+// the modes that end a call on natural fields (HOP_FULL always does)
 constexpr bool nat_mode(int mode) { return mode == HOP_K2 || mode == HOP_FULL; }
 
 template <int MODE>
@@ -369,12 +366,10 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     // than the gap between the launches while they are few: D_S 31.4 us overlapped and
     // 29.0 not on 18x10x14x22, 37.2 and 36.7 on 16^3x32, but 54.9 and 58.7 on 20^3x32.
     const bool after = c.after && blocks > 512;
-    if constexpr (MODE == HOP_K2)
-        if (c.nat) {
-            launch_after(e, after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
-            return;
-        }
-    launch_after(e, after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
+    if constexpr (MODE == HOP_K2)   // always natural
+        launch_after(e, after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
+    else if constexpr (MODE == HOP_K1 || MODE == HOP_RICH)
+        launch_after(e, after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
 }
 
 // The batched hop over the right-hand sides of several lattices of different
@@ -974,8 +969,8 @@ static void launch_hop(const Exec &e, const HopCall &c)
         if constexpr (MODE == HOP_RECON)
             if (c.in32) return launch(std::integral_constant<int, kNat | kIn32>());
         if constexpr (nat_mode(MODE))
-            if (c.nat) return launch(std::integral_constant<int, kNat>());
-        launch(std::integral_constant<int, 0>());
+            if (MODE == HOP_FULL || c.nat) return launch(std::integral_constant<int, kNat>());
+        if constexpr (MODE != HOP_FULL) launch(std::integral_constant<int, 0>());
     }
     else
     {
@@ -988,7 +983,7 @@ static void launch_hop(const Exec &e, const HopCall &c)
             kr.in2 = k.in2 ? k.in2 + o : nullptr;
             kr.b = k.b ? k.b + o : nullptr;
             kr.out = k.out + o;
-            const size_t sm = c.nat ? nat_smem(threads) : 0;
+            const size_t sm = c.nat || MODE == HOP_FULL ? nat_smem(threads) : 0;
             auto launch = [&](auto nat) {
                 constexpr bool NAT = decltype(nat)::value;
                 if constexpr (std::is_same<R, float>::value && (MODE == HOP_K2 || MODE == HOP_RICH))
@@ -996,7 +991,9 @@ static void launch_hop(const Exec &e, const HopCall &c)
                 else
                     launch_after(e, c.after, hop_kernel<R, MODE, NAT>, blocks, threads, sm, e.g, kr);
             };
-            if constexpr (nat_mode(MODE)) {
+            if constexpr (MODE == HOP_FULL) {
+                launch(std::true_type());
+            } else if constexpr (nat_mode(MODE)) {
                 if (c.nat) launch(std::true_type());
                 else launch(std::false_type());
             } else {
@@ -1103,8 +1100,8 @@ void hop(const Exec &e, const HopCall &c)
         else if (c.prec == P16) launch_hop_bf<M>(e, c);                         \
         else launch_hop<df64, M>(e, c);                                         \
         break;
-    // df64 keeps the right-hand sides of a site in one thread (links and clover
-    // counted once); FP64 and FP32 launch once per right-hand side
+    // df64 and FP64 take all right-hand sides in one launch (links and clover
+    // counted once for df64); FP32 launches once per right-hand side
     const double site_bytes = c.prec == PDF ? hop_site_bytes(c.mode, c.prec, c.nrhs)
                                             : c.nrhs * hop_site_bytes(c.mode, c.prec, 1);
     // natural rows are complex doubles whatever the precision

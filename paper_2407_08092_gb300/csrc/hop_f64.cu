@@ -171,12 +171,15 @@ static void launch_f64(const Exec &e, const HopCall &c)
     // most of one wave: D_S on 18x10x14x22 140 us overlapped and 131 not, on 16^4 161
     // and 158, but 86 and 90 on 16^2x12^2 and 241 and 244 on 16^3x24.
     const bool after = c.after && (blocks <= 768 || blocks > 1216);
-    if constexpr (MODE == HOP_K2 || MODE == HOP_FULL)
-        if (c.nat) {
-            launch_after(e, after, hop_f64_kernel<MODE, true>, blocks, 2 * kF64Sites, 0, e.g, k);
-            return;
-        }
-    launch_after(e, after, hop_f64_kernel<MODE, false>, blocks, 2 * kF64Sites, 0, e.g, k);
+    auto launch = [&](auto kernel) { launch_after(e, after, kernel, blocks, 2 * kF64Sites, 0, e.g, k); };
+    if constexpr (MODE == HOP_FULL) {   // always natural
+        launch(hop_f64_kernel<MODE, true>);
+    } else if constexpr (MODE == HOP_K2) {
+        if (c.nat) launch(hop_f64_kernel<MODE, true>);
+        else launch(hop_f64_kernel<MODE, false>);
+    } else {
+        launch(hop_f64_kernel<MODE, false>);
+    }
 }
 
 void hop_f64(const Exec &e, const HopCall &c)

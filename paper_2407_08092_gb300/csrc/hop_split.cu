@@ -92,7 +92,7 @@ __device__ __forceinline__ CloverRow<R> load_row(const CV *C, long long st, long
 }
 
 // y0 + (row of C) x, x[j * kSplitSites] the six components of the block; `y0`
-// enters as the one-thread kernels add it: before the row in df64, not at all in
+// enters as the larger lattices' kernels add it: before the row in df64, not at all in
 // the others, where the caller adds to the row's product
 template <typename R>
 __device__ __forceinline__ cx<R> row_apply(const CloverRow<R> &w, int r, const cx<R> *x, cx<R>)
@@ -155,7 +155,7 @@ struct HalfHop {
     static __device__ __forceinline__ cx<R> norm(cx<R> acc) { return acc; }
     static __device__ __forceinline__ cx<R> scale(cx<R> a, float f) { return R(f) * a; }
 };
-// df64: one body for the eight directions, as in the one-thread kernel
+// df64: one body for the eight directions, as in hop_df_kernel
 template <>
 struct HalfHop<df64, df2, df2> {
     static __device__ __forceinline__ void run(int d, const df2 *psi, const df2 *Uout, const df2 *Uin, long long st,

@@ -407,10 +407,6 @@ __global__ void gamma5_df_kernel(Geom g, const float4 *in, float4 *out)
 
 void gamma5(const Exec &e, int prec, const void *in, void *out)
 {
-    if (prec == P16) {
-        bf16_gamma5(e, in, out);
-        return;
-    }
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (in == out ? 1 : 2) * (prec == P32 ? 96 : 192));
     if (prec == PDF) {
         gamma5_df_kernel<<<nblk(e.g.Vh, 256), 256, 0, e.st>>>(e.g, (const float4 *)in, (float4 *)out);

@@ -115,7 +115,6 @@ void links_to_bf16(const Exec &e, const void *U32, void *U16);
 // BF16 fields (bf16.cu): conversions (one side BF16) and axpby; the generic
 // launchers below dispatch here for P16
 void bf16_convert(const Exec &e, int from, const void *in, int to, void *out);
-void bf16_gamma5(const Exec &e, const void *in, void *out);
 void bf16_axpby(const Exec &e, double ar, double ai, const void *x, double br, double bi, void *y, int nfields);
 // natural half spinor [Vh][12] c128 <-> internal field of one parity
 // (g5: with spins 2 and 3 negated)
@@ -129,7 +128,7 @@ void export_parity(const Exec &e, const void *f, int parity, void *nat);
 // precision conversion between internal fields (nfields consecutive ones between
 // FP32 and df64)
 void convert(const Exec &e, int from, const void *in, int to, void *out, int nfields = 1);
-// out = g5 in (negates spins 2 and 3); in == out allowed
+// out = g5 in (negates spins 2 and 3), FP64, FP32 or df64; in == out allowed
 void gamma5(const Exec &e, int prec, const void *in, void *out);
 
 // ---- clover (clover.cu) ----------------------------------------------------
@@ -213,8 +212,8 @@ struct HopCall {
     void *out2 = nullptr;          // HOP_RECON_RES: the output parity's residual
     double omega;          // HOP_RICH weight
     int nrhs = 1;          // right-hand sides: in, in2, b, out are nrhs consecutive fields
-    // natural output (HOP_K2 in any precision, HOP_FULL but in BF16, HOP_RECON with
-    // in32; one right-hand side): complex-double rows in the place of `out`, those of
+    // natural output (HOP_K2; always for HOP_FULL, for HOP_RECON with in32 and in
+    // BF16, which offers HOP_K1, HOP_K2 and HOP_RICH; one right-hand side): complex-double rows in the place of `out`, those of
     // a full lattice or of one parity, spins 2 and 3 negated on request
     void *nat = nullptr;
     bool nat_full = false, nat_g5 = false;
@@ -225,7 +224,7 @@ struct HopCall {
 };
 void hop(const Exec &e, const HopCall &c);
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
-// done, where the one-thread kernels are the faster ones
+// done, where the other kernels are the faster ones
 bool hop_split(const Exec &e, const HopCall &c);
 void hop_f64(const Exec &e, const HopCall &c);   // FP64 (hop_f64.cu)
 bool hop_split_takes(const Geom &g, int prec, int nrhs);
