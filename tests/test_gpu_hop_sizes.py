@@ -85,3 +85,48 @@ def test_batch_matches_oracle(pair):
     for r in range(n):
         true = np.linalg.norm(b[r] - pair.lat.dirac(got[r])) / np.linalg.norm(b[r])
         assert true <= 1.001e-10 and abs(stats[r].rel_resid_true - true) <= 1e-13
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3], ids=["f64", "f32", "df64", "bf16"])
+def test_apply_replayed_from_a_graph(pair, prec):
+    """The overlapped launches of one call, captured and replayed on another input."""
+    import torch
+    from paper_2407_08092_gb300 import lqdd
+    s = torch.cuda.Stream()
+    ctx = lqdd.lq_create(lqdd.make_lattice(pair.L, -1, 0.05, 1.0), s.cuda_stream)
+    try:
+        lqdd.lq_set_gauge(ctx, pair.dU)
+        x = pair.dev(synth.gaussian_spinor(pair.Vh, 81))
+        out = torch.empty_like(x)
+        torch.cuda.synchronize()
+        lqdd.lq_apply(ctx, lqdd.LQ_OP_SCHUR, prec, x, out)   # workspaces and links of this precision
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            lqdd.lq_apply(ctx, lqdd.LQ_OP_SCHUR, prec, x, out)
+        y = synth.gaussian_spinor(pair.Vh, 82)
+        x.copy_(pair.dev(y))
+        for _ in range(2):
+            g.replay()
+        torch.cuda.synchronize()
+        assert rel(out.cpu().numpy(), pair.lat.schur(y)) < TOL[prec]
+    finally:
+        lqdd.lq_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,m", [(2, 0), (1, 1)])
+@pytest.mark.parametrize("block", [(4, 4, 4, 4), (2, 2, 4, 2)])
+def test_sap_few_steps(n, m, block):
+    """The shortest chains of the block solve's loads ahead: no and one Minimal Residual step."""
+    from oracle import sap as osap
+    from paper_2407_08092_gb300 import lqdd
+    p = Pair((8, 8, 4, 8), eps=0.25, seed=1500, m0=0.05, csw=1.0, t_bc=-1)
+    try:
+        r = synth.gaussian_spinor(p.V, 93)
+        out = p.torch.empty_like(p.dev(r))
+        prm = lqdd.make_params(smoother=lqdd.LQ_SMOOTH_SAP, smooth_n=n, smooth_m=m, inner_prec=lqdd.LQ_F32,
+                               prec=lqdd.LQ_DF64, sap_block=block)
+        lqdd.lq_smooth(p.ctx, prm, p.dev(r), out)
+        assert rel(p.host(out), osap.sap(p.lat, r, n, m, block)) < 1e-5
+    finally:
+        p.close()
