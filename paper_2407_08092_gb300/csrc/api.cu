@@ -38,9 +38,11 @@ typedef std::complex<double> cd;
 static constexpr int MAX_RESTART = 256;
 static constexpr int RED_SLOTS = 2 * MAX_RESTART + 8;
 // Sites per parity up to which the FP32 GMRES queues the next step's operator
-// before it reads a step's scalars.  The GPU idles about 10 us a step while the
-// host reads them; the product queued ahead of a cycle's last step is wasted.
-static constexpr long long kAheadSites = 1LL << 18;
+// before it reads a step's scalars.  The GPU idles some microseconds a step while
+// the host reads them; the product queued ahead of the step that ends a solve is
+// wasted.  Mixed solve with and without: 8^4 1.36 / 1.59 ms, 16^3 x 32 3.12 / 3.36,
+// 24^3 x 48 10.18 / 10.43, 32^4 (2^19 sites) 15.89 / 16.07.
+static constexpr long long kAheadSites = 1LL << 19;
 
 struct lq_ctx {
     Geom g;

@@ -132,12 +132,12 @@ __global__ void __launch_bounds__(RT, 4) multi_dot_kernel(const typename Vec<R>:
                                                           double *out = nullptr, unsigned *ticket = nullptr)
 {
     __shared__ R sh[(RT / 32) * 2 * NJ];
-    if (FIN) after_previous();
+    after_previous();
     R acc[2 * NJ];
 #pragma unroll
     for (int i = 0; i < 2 * NJ; i++) acc[i] = R(0);
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
-        const auto wv = FIN ? w[i] : __ldg(w + i);   // FIN: written by the kernel before (after_previous)
+        const auto wv = w[i];   // written by the kernel before (after_previous)
 #pragma unroll
         for (int j = 0; j < NJ; j++) cdot_acc(__ldg(Vb + j * n + i), wv, acc[2 * j], acc[2 * j + 1]);
     }
@@ -151,9 +151,10 @@ __global__ void __launch_bounds__(RT, 4) multi_dot_kernel(const typename Vec<R>:
 // ---- y = y + sign * sum_j c_j v_j, optionally the partials of ||y_new||^2 ------------
 template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT, 4) multi_axpy_kernel(const typename Vec<R>::V *__restrict__ Vb, long long n,
-                                                           int nv, const double2 *__restrict__ c, R sign,
+                                                           int nv, const double2 *c, R sign,
                                                            typename Vec<R>::V *y, double *partial, int pitch, int slot)
 {
+    after_previous();
     typedef typename Vec<R>::V V;
     __shared__ R sh[RT / 32];
     // the coefficients, converted once per block (a double -> float conversion
@@ -233,13 +234,14 @@ __global__ void __launch_bounds__(RT, 4) multi_axpy_fin_kernel(const float4 *__r
 }
 
 template <typename R>
-__global__ void __launch_bounds__(RT) norm2_kernel(const typename Vec<R>::V *__restrict__ w, long long n,
+__global__ void __launch_bounds__(RT) norm2_kernel(const typename Vec<R>::V *w, long long n,
                                                    double *partial, int pitch, int slot)
 {
+    after_previous();
     __shared__ R sh[RT / 32];
     R nrm[1] = {R(0)};
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT)
-        nrm[0] = nrm_acc(__ldg(w + i), nrm[0]);
+        nrm[0] = nrm_acc(w[i], nrm[0]);
     block_sum<R, 1>(nrm, sh);
     if (threadIdx.x == 0) {
         partial[(long long)blockIdx.x * pitch + 2 * slot] = (double)nrm[0];
@@ -264,9 +266,10 @@ __global__ void __launch_bounds__(RT) nat_norm2_kernel(const double2 *__restrict
 
 // one block per value: out[v] = sum_b partial[b][v] in a fixed tree order,
 // times scale[v / 2] when a scale (one real per complex value) is given
-__global__ void __launch_bounds__(RT) reduce_finish_kernel(const double *__restrict__ partial, int blocks, int pitch,
-                                                           const double *__restrict__ scale, double *out)
+__global__ void __launch_bounds__(RT) reduce_finish_kernel(const double *partial, int blocks, int pitch,
+                                                           const double *scale, double *out)
 {
+    after_previous();
     __shared__ double sh[RT / 32];
     const int v = blockIdx.x;
     double acc[1] = {0.0};
@@ -280,6 +283,7 @@ template <typename R>
 __global__ void __launch_bounds__(RT) axpby_kernel(R ar, R ai, const typename Vec<R>::V *x, R br, R bi,
                                                    typename Vec<R>::V *y, long long n)
 {
+    after_previous();
     const long long i = blockIdx.x * (long long)RT + threadIdx.x;
     if (i >= n) return;
     typename Vec<R>::V o = {}, xv = x[i], yv = y[i];
@@ -319,15 +323,15 @@ __device__ __forceinline__ void block_sum_df(df64 v[N], df64 *sh /* [RT/32][N] *
 
 template <int NJ>
 __global__ void __launch_bounds__(RT) multi_dot_df_kernel(const df2 *__restrict__ Vb, long long n,
-                                                          const df2 *__restrict__ w, double *partial, int pitch,
-                                                          int slot0)
+                                                          const df2 *w, double *partial, int pitch, int slot0)
 {
+    after_previous();
     __shared__ df64 sh[(RT / 32) * 2 * NJ];
     df64 acc[2 * NJ];
 #pragma unroll
     for (int i = 0; i < 2 * NJ; i++) acc[i] = df64(0.0f, 0.0f);
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
-        const cx<df64> wv = df2_cx(ldg(w + i));
+        const cx<df64> wv = df2_cx(w[i]);
 #pragma unroll
         for (int j = 0; j < NJ; j++) {
             const cx<df64> vv = df2_cx(ldg(Vb + j * n + i));
@@ -343,9 +347,10 @@ __global__ void __launch_bounds__(RT) multi_dot_df_kernel(const df2 *__restrict_
 
 template <bool NORM>
 __global__ void __launch_bounds__(RT) multi_axpy_df_kernel(const df2 *__restrict__ Vb, long long n, int nv,
-                                                           const double2 *__restrict__ c, int sign, df2 *y,
+                                                           const double2 *c, int sign, df2 *y,
                                                            double *partial, int pitch, int slot)
 {
+    after_previous();
     __shared__ df64 cs[2 * 256];
     __shared__ df64 sh[RT / 32];
     for (int j = threadIdx.x; j < nv; j += RT) {
@@ -371,13 +376,14 @@ __global__ void __launch_bounds__(RT) multi_axpy_df_kernel(const df2 *__restrict
     }
 }
 
-__global__ void __launch_bounds__(RT) norm2_df_kernel(const df2 *__restrict__ w, long long n, double *partial,
+__global__ void __launch_bounds__(RT) norm2_df_kernel(const df2 *w, long long n, double *partial,
                                                       int pitch, int slot)
 {
+    after_previous();
     __shared__ df64 sh[RT / 32];
     df64 nrm[1] = {df64(0.0f, 0.0f)};
     for (long long i = blockIdx.x * (long long)RT + threadIdx.x; i < n; i += (long long)gridDim.x * RT) {
-        const cx<df64> v = df2_cx(ldg(w + i));
+        const cx<df64> v = df2_cx(w[i]);
         nrm[0] = fma(v.re, v.re, fma(v.im, v.im, nrm[0]));
     }
     block_sum_df<1>(nrm, sh);
@@ -390,6 +396,7 @@ __global__ void __launch_bounds__(RT) norm2_df_kernel(const df2 *__restrict__ w,
 __global__ void __launch_bounds__(RT) axpby_df_kernel(df64 ar, df64 ai, const df2 *x, df64 br, df64 bi, df2 *y,
                                                       long long n)
 {
+    after_previous();
     const long long i = blockIdx.x * (long long)RT + threadIdx.x;
     if (i >= n) return;
     const cx<df64> a = {ar, ai}, b = {br, bi};
@@ -441,10 +448,12 @@ struct SmallVals {
 };
 __global__ void put_values_kernel(SmallVals s, int n, double *d)
 {
+    after_previous();
     if ((int)threadIdx.x < n) d[threadIdx.x] = s.v[threadIdx.x];
 }
-__global__ void get_values_kernel(const double *__restrict__ d, int n, double *h)
+__global__ void get_values_kernel(const double *d, int n, double *h)
 {
+    after_previous();
     for (int i = threadIdx.x; i < n; i += blockDim.x) h[i] = d[i];
 }
 __global__ void get_ints_kernel(const int *__restrict__ d, int n, int *h)
@@ -459,14 +468,14 @@ void put_values(const Exec &e, const double *h, int n, double *d)
         SmallVals s;
         for (int i = 0; i < m; i++) s.v[i] = h[k + i];
         Launch L_(e, K_FINISH, 0.0);
-        put_values_kernel<<<1, kSmallVals, 0, e.st>>>(s, m, d + k);
+        launch_after(e, true, put_values_kernel, 1, kSmallVals, 0, s, m, d + k);
     }
 }
 void get_values(const Exec &e, const double *d, int n, double *h_mapped)
 {
     if (n <= 0) return;
     Launch L_(e, K_FINISH, 0.0);
-    get_values_kernel<<<1, 128, 0, e.st>>>(d, n, h_mapped);
+    launch_after(e, true, get_values_kernel, 1, 128, 0, d, n, h_mapped);
 }
 void get_ints(const Exec &e, const int *d, int n, int *h_mapped)
 {
@@ -484,13 +493,17 @@ void axpby(const Exec &e, int prec, double ar, double ai, const void *x, double 
     // nfields consecutive fields are one linear array
     Launch L_(e, axpy_class(prec), 3.0 * nfields * e.g.Vh * sp_bytes(prec), (double)nfields * e.g.Vh * 12 * 14);
     const long long n = nvec(e.g, prec) * nfields;
+    // overlapped where the launch is short: a long one leaves the hop behind it
+    // unevenly placed (Richardson(5) on 24^3 x 48 867 us so, 859 not)
+    const bool after = nblk(n) <= 2048;
     if (prec == PDF)
-        axpby_df_kernel<<<nblk(n), RT, 0, e.st>>>(df64(ar), df64(ai), (const df2 *)x, df64(br), df64(bi), (df2 *)y, n);
+        launch_after(e, after, axpby_df_kernel, nblk(n), RT, 0, df64(ar), df64(ai), (const df2 *)x, df64(br), df64(bi),
+                     (df2 *)y, n);
     else if (prec == P64)
-        axpby_kernel<double><<<nblk(n), RT, 0, e.st>>>(ar, ai, (const double2 *)x, br, bi, (double2 *)y, n);
+        launch_after(e, after, axpby_kernel<double>, nblk(n), RT, 0, ar, ai, (const double2 *)x, br, bi, (double2 *)y, n);
     else
-        axpby_kernel<float><<<nblk(n), RT, 0, e.st>>>((float)ar, (float)ai, (const float4 *)x, (float)br, (float)bi,
-                                                     (float4 *)y, n);
+        launch_after(e, after, axpby_kernel<float>, nblk(n), RT, 0, (float)ar, (float)ai, (const float4 *)x, (float)br,
+                     (float)bi, (float4 *)y, n);
 }
 
 void multi_axpy(const Exec &e, int prec, const void *V, int nv, const double *c_dev, int sign, void *y,
@@ -505,22 +518,22 @@ void multi_axpy(const Exec &e, int prec, const void *V, int nv, const double *c_
     const double2 *c = (const double2 *)c_dev;
     if (prec == PDF) {
         if (r)
-            multi_axpy_df_kernel<true><<<blocks, RT, 0, e.st>>>((const df2 *)V, n, nv, c, sign, (df2 *)y, part, pitch, slot);
+            launch_after(e, true, multi_axpy_df_kernel<true>, blocks, RT, 0, (const df2 *)V, n, nv, c, sign, (df2 *)y, part, pitch, slot);
         else
-            multi_axpy_df_kernel<false><<<blocks, RT, 0, e.st>>>((const df2 *)V, n, nv, c, sign, (df2 *)y, part, pitch, slot);
+            launch_after(e, true, multi_axpy_df_kernel<false>, blocks, RT, 0, (const df2 *)V, n, nv, c, sign, (df2 *)y, part, pitch, slot);
     } else if (prec == P64) {
         if (r)
-            multi_axpy_kernel<double, true><<<blocks, RT, 0, e.st>>>((const double2 *)V, n, nv, c, (double)sign,
+            launch_after(e, true, multi_axpy_kernel<double, true>, blocks, RT, 0, (const double2 *)V, n, nv, c, (double)sign,
                                                                      (double2 *)y, part, pitch, slot);
         else
-            multi_axpy_kernel<double, false><<<blocks, RT, 0, e.st>>>((const double2 *)V, n, nv, c, (double)sign,
+            launch_after(e, true, multi_axpy_kernel<double, false>, blocks, RT, 0, (const double2 *)V, n, nv, c, (double)sign,
                                                                       (double2 *)y, part, pitch, slot);
     } else {
         if (r)
-            multi_axpy_kernel<float, true><<<blocks, RT, 0, e.st>>>((const float4 *)V, n, nv, c, (float)sign,
+            launch_after(e, true, multi_axpy_kernel<float, true>, blocks, RT, 0, (const float4 *)V, n, nv, c, (float)sign,
                                                                     (float4 *)y, part, pitch, slot);
         else
-            multi_axpy_kernel<float, false><<<blocks, RT, 0, e.st>>>((const float4 *)V, n, nv, c, (float)sign,
+            launch_after(e, true, multi_axpy_kernel<float, false>, blocks, RT, 0, (const float4 *)V, n, nv, c, (float)sign,
                                                                      (float4 *)y, part, pitch, slot);
     }
 }
@@ -568,13 +581,14 @@ static void dot_launch(const Exec &e, int blocks, const void *V, long long n, co
                        int slot0)
 {
     typedef typename Vec<R>::V VV;
-    multi_dot_kernel<R, NJ><<<blocks, RT, 0, e.st>>>((const VV *)V, n, (const VV *)w, part, pitch, slot0);
+    launch_after(e, true, multi_dot_kernel<R, NJ, false>, blocks, RT, 0, (const VV *)V, n, (const VV *)w, part, pitch, slot0,
+                 (const double *)nullptr, (double *)nullptr, (unsigned *)nullptr);
 }
 template <int NJ>
 static void dot_launch_df(const Exec &e, int blocks, const void *V, long long n, const void *w, double *part,
                           int pitch, int slot0)
 {
-    multi_dot_df_kernel<NJ><<<blocks, RT, 0, e.st>>>((const df2 *)V, n, (const df2 *)w, part, pitch, slot0);
+    launch_after(e, true, multi_dot_df_kernel<NJ>, blocks, RT, 0, (const df2 *)V, n, (const df2 *)w, part, pitch, slot0);
 }
 
 template <int NJ>
@@ -615,11 +629,11 @@ void norm2(const Exec &e, int prec, const void *w, const RedScratch &r, int slot
     const int pitch = 2 * r.maxv;
     const long long n = nvec(e.g, prec);
     if (prec == PDF)
-        norm2_df_kernel<<<r.blocks, RT, 0, e.st>>>((const df2 *)w, n, r.partial, pitch, slot);
+        launch_after(e, true, norm2_df_kernel, r.blocks, RT, 0, (const df2 *)w, n, r.partial, pitch, slot);
     else if (prec == P64)
-        norm2_kernel<double><<<r.blocks, RT, 0, e.st>>>((const double2 *)w, n, r.partial, pitch, slot);
+        launch_after(e, true, norm2_kernel<double>, r.blocks, RT, 0, (const double2 *)w, n, r.partial, pitch, slot);
     else
-        norm2_kernel<float><<<r.blocks, RT, 0, e.st>>>((const float4 *)w, n, r.partial, pitch, slot);
+        launch_after(e, true, norm2_kernel<float>, r.blocks, RT, 0, (const float4 *)w, n, r.partial, pitch, slot);
 }
 
 void nat_norm2(const Exec &e, const void *v, long long n_sites, const RedScratch &r, int slot)
@@ -633,8 +647,8 @@ void reduce_finish(const Exec &e, const RedScratch &r, int first, int count, con
 {
     if (count <= 0) return;
     Launch L_(e, K_FINISH, (double)r.blocks * 2 * count * 8.0);
-    reduce_finish_kernel<<<2 * count, RT, 0, e.st>>>(r.partial + 2 * first, r.blocks, 2 * r.maxv, scale,
-                                                     r.out + 2 * first);
+    launch_after(e, true, reduce_finish_kernel, 2 * count, RT, 0, r.partial + 2 * first, r.blocks, 2 * r.maxv, scale,
+                 r.out + 2 * first);
 }
 
 }  // namespace lq
