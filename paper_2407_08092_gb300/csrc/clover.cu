@@ -84,24 +84,19 @@ __device__ __forceinline__ void shifted(const Geom &g, const int c[4], int mu, i
     else out[3] = v;
 }
 
-// sum_k conj(B_k) A_k over three entries of two rows (or columns) `step` apart
-__device__ __forceinline__ df64x2 conj_dot(const cx<df64> *B, const cx<df64> *A, int step)
-{
-    dlrow t = dlrow_prod(B[0], dl2(A[0]));
-    dlrow_fma(t, B[step], dl2(A[step]));
-    dlrow_fma(t, B[2 * step], dl2(A[2 * step]));
-    return dlrow_conj(t);
-}
+// The sums below take their terms in turn, k by k with the product of the real
+// part first, packed or not.  Their last bits decide how the FP32 copies of the
+// clover blocks round, so another order (the products of the real parts summed
+// apart from those of the imaginary parts, say) changes FP32 operator outputs in
+// one component of ten million.
 
-// Im sum_k conj(B_k) A_k, unnormalised: both products of a term in one packed sum
-__device__ __forceinline__ df64 im_conj_dot(const cx<df64> *B, const cx<df64> *A, int step)
+// sum_k conj(B_k) A_k over three entries of two rows (or columns) `step` apart
+__device__ __forceinline__ cx<df64> conj_dot(const cx<df64> *B, const cx<df64> *A, int step)
 {
-    df64x2 t = dl2_prod(dl2(B[0]), dl2_swap(dl2(A[0])));   // (B.re A.im, B.im A.re)
-    dl2_fma(t, dl2(B[step]), dl2_swap(dl2(A[step])));
-    dl2_fma(t, dl2(B[2 * step]), dl2_swap(dl2(A[2 * step])));
-    cx<df64> s = dl2_cx(t);
-    dl_add(s.re, dl_neg(s.im));
-    return s.re;
+    cx<df64> t = dl_cmul({B[0].re, dl_neg(B[0].im)}, A[0]);
+    dl_cfmac(t, B[step], A[step]);
+    dl_cfmac(t, B[2 * step], A[2 * step]);
+    return t;
 }
 
 // A B^+ (full product), each entry a lazily normalised compensated sum
@@ -112,7 +107,7 @@ __device__ __forceinline__ M3<df64> mat_mul_nd(const M3<df64> &A, const M3<df64>
     for (int a = 0; a < 3; a++)
 #pragma unroll
         for (int b = 0; b < 3; b++)   // sum_k A_ak conj(B_bk)
-            P.a[a * 3 + b] = dl2_cx(dl2_norm(conj_dot(B.a + b * 3, A.a + a * 3, 1)));
+            P.a[a * 3 + b] = dl_cnorm(conj_dot(B.a + b * 3, A.a + a * 3, 1));
     return P;
 }
 
@@ -120,16 +115,25 @@ __device__ __forceinline__ M3<df64> mat_mul_nd(const M3<df64> &A, const M3<df64>
 __device__ __forceinline__ void ah_of_mul_nd(const M3<df64> &A, const M3<df64> &B, df64 v[9])
 {
 #pragma unroll
-    for (int a = 0; a < 3; a++) v[a] = dl_scale2(dl_norm(im_conj_dot(B.a + a * 3, A.a + a * 3, 1)), 2.0f);
+    for (int a = 0; a < 3; a++) {   // Im sum_k A_ak conj(B_ak) = sum_k (A.im B.re - A.re B.im)
+        df64 s = dl_prod(A.a[a * 3].im, B.a[a * 3].re);
+        dl_fma(s, dl_neg(A.a[a * 3].re), B.a[a * 3].im);
+#pragma unroll
+        for (int k = 1; k < 3; k++) {
+            dl_fma(s, A.a[a * 3 + k].im, B.a[a * 3 + k].re);
+            dl_fma(s, dl_neg(A.a[a * 3 + k].re), B.a[a * 3 + k].im);
+        }
+        v[a] = dl_scale2(dl_norm(s), 2.0f);
+    }
     const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
 #pragma unroll
     for (int q = 0; q < 3; q++) {
         const int a = pa[q], b = pb[q];
         // X = sum_k A_ak conj(B_bk), Y = sum_k A_bk conj(B_ak); AH_ab = X - conj(Y)
-        df64x2 x = conj_dot(B.a + b * 3, A.a + a * 3, 1);
-        const cx<df64> y = dl2_cx(conj_dot(B.a + a * 3, A.a + b * 3, 1));
-        dl2_add(x, dl2({dl_neg(y.re), y.im}));
-        const cx<df64> n = dl2_cx(dl2_norm(x));
+        cx<df64> x = conj_dot(B.a + b * 3, A.a + a * 3, 1);
+        const cx<df64> y = conj_dot(B.a + a * 3, A.a + b * 3, 1);
+        dl_cadd(x, {dl_neg(y.re), y.im});
+        const cx<df64> n = dl_cnorm(x);
         v[3 + 2 * q] = n.re;
         v[4 + 2 * q] = n.im;
     }
@@ -140,11 +144,20 @@ __device__ __forceinline__ void ah_conj(const M3<df64> &H, const M3<df64> &W, df
 {
     const M3<df64> Y = mat_mul<df64>(H, W);
 #pragma unroll
-    for (int a = 0; a < 3; a++) v[a] = dl_norm(im_conj_dot(W.a + a, Y.a + a, 3));   // Im sum_k conj(W_ka) Y_ka
+    for (int a = 0; a < 3; a++) {   // Im sum_k conj(W_ka) Y_ka = sum_k (W.re Y.im - W.im Y.re)
+        df64 s = dl_prod(W.a[a].re, Y.a[a].im);
+        dl_fma(s, dl_neg(W.a[a].im), Y.a[a].re);
+#pragma unroll
+        for (int k = 1; k < 3; k++) {
+            dl_fma(s, W.a[k * 3 + a].re, Y.a[k * 3 + a].im);
+            dl_fma(s, dl_neg(W.a[k * 3 + a].im), Y.a[k * 3 + a].re);
+        }
+        v[a] = dl_norm(s);
+    }
     const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
 #pragma unroll
     for (int q = 0; q < 3; q++) {   // sum_k conj(W_ka) Y_kb
-        const cx<df64> n = dl2_cx(dl2_norm(conj_dot(W.a + pa[q], Y.a + pb[q], 3)));
+        const cx<df64> n = dl_cnorm(conj_dot(W.a + pa[q], Y.a + pb[q], 3));
         v[3 + 2 * q] = n.re;
         v[4 + 2 * q] = n.im;
     }

@@ -67,11 +67,10 @@ __device__ __forceinline__ M3<df64> mat_mul<df64>(const M3<df64> &A, const M3<df
     for (int a = 0; a < 3; a++)
 #pragma unroll
         for (int b = 0; b < 3; b++) {
-            dlrow acc = dlrow_prod(A.a[a * 3], dl2(B.a[b]));
-            dlrow_fma(acc, A.a[a * 3 + 1], dl2(B.a[3 + b]));
-            dlrow_fma(acc, A.a[a * 3 + 2], dl2(B.a[6 + b]));
-            dl2_add(acc.r, dlrow_rot(acc));
-            P.a[a * 3 + b] = dl2_cx(dl2_norm(acc.r));
+            cx<df64> acc = dl_cmul(A.a[a * 3], B.a[b]);
+            dl_cfma(acc, A.a[a * 3 + 1], B.a[3 + b]);
+            dl_cfma(acc, A.a[a * 3 + 2], B.a[6 + b]);
+            P.a[a * 3 + b] = dl_cnorm(acc);
         }
     return P;
 }
