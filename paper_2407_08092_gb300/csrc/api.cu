@@ -1353,6 +1353,9 @@ lq_status guarded(lq_ctx *c, F &&f)
         return LQ_OK;
     } catch (const Fail &f) {
         return f.s;
+    } catch (const Refused &r) {
+        c->err = r.why;
+        return LQ_ERR_ARG;
     } catch (const std::bad_alloc &) {
         c->err = "host allocation failed";
         return LQ_ERR_OOM;

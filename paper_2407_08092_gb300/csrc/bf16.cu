@@ -1,5 +1,5 @@
-// BF16 fields: conversion to and from the other internal precisions and the
-// natural layout, gamma5, axpby, and the BF16 copy of the 12-real links.
+// BF16 fields: conversion to and from the other internal precisions, axpby, and
+// the BF16 copy of the 12-real links.
 // Arithmetic is FP32; stores round to nearest BF16.  Only the sites below V/2
 // are written, so the zero padding of a field stays zero.
 #include <type_traits>

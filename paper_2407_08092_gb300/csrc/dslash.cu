@@ -142,7 +142,7 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
 #pragma unroll
         for (int i = 0; i < 12; i++) acc[i] = (SCALED ? R(-0.5) * omega : R(-0.5)) * acc[i];
         clover_apply<R>(clov, st, s, acc, v);
-    } else if (MODE == HOP_K2 || MODE == HOP_RICH || MODE == HOP_FULL) {
+    } else {   // HOP_K2, HOP_RICH, HOP_FULL
         cx<R> x[12];
         load_spinor_rw(in2, st, s, x);
         clover_apply<R>(clov, st, s, x, v);
@@ -154,17 +154,6 @@ __device__ __forceinline__ void hop_body(const Geom &g, const LV *Uout, const LV
             load_spinor(bv, st, s, bb);
 #pragma unroll
             for (int i = 0; i < 12; i++) v[i] = x[i] + omega * (bb[i] - v[i]);
-        }
-    } else {   // HOP_PREP, HOP_RECON
-        cx<R> y[12];
-        load_spinor_rw(in2, st, s, y);
-#pragma unroll
-        for (int i = 0; i < 12; i++) y[i] = y[i] + R(0.5) * acc[i];
-        if (MODE == HOP_RECON) {
-            clover_apply<R>(clov, st, s, y, v);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 12; i++) v[i] = y[i];
         }
     }
     if (NAT) store_nat(nat, tile, (const SV *)nullptr, s - min((int)(threadIdx.x & 31), nvalid - 1), nvalid, c.x & 1, v);
@@ -366,9 +355,9 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     // than the gap between the launches while they are few: D_S 31.4 us overlapped and
     // 29.0 not on 18x10x14x22, 37.2 and 36.7 on 16^3x32, but 54.9 and 58.7 on 20^3x32.
     const bool after = c.after && blocks > 512;
-    if constexpr (MODE == HOP_K2)   // always natural
+    if constexpr (MODE == HOP_K2)   // always natural (hop_refused)
         launch_after(e, after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);
-    else if constexpr (MODE == HOP_K1 || MODE == HOP_RICH)
+    else
         launch_after(e, after, hop_kernel_bf<MODE>, blocks, LQ_HOP_THREADS, 0, e.g, k);
 }
 
@@ -1092,14 +1081,19 @@ void hop_group(const Exec &e, int mode, const LatDesc *desc, const int4 *tiles, 
     else hop_group_kernel<HOP_K2, 1><<<grid, block, 0, e.st>>>(desc, tiles, ntiles, i1, i2, o, scale, sstride);
 }
 
+template <int MODE>
+static void launch_mode(const Exec &e, const HopCall &c)
+{
+    if (c.prec == PDF) return launch_hop<df64, MODE>(e, c);
+    if constexpr (hop_form(MODE, P32))
+        if (c.prec == P32) return launch_hop<float, MODE>(e, c);
+    if constexpr (hop_form(MODE, P16))
+        if (c.prec == P16) return launch_hop_bf<MODE>(e, c);
+}
+
 void hop(const Exec &e, const HopCall &c)
 {
-#define LQ_CASE(M)                                                              \
-    case M:                                                                     \
-        if (c.prec == P32) launch_hop<float, M>(e, c);                          \
-        else if (c.prec == P16) launch_hop_bf<M>(e, c);                         \
-        else launch_hop<df64, M>(e, c);                                         \
-        break;
+    if (const char *why = hop_refused(e.g, c)) throw Refused{why};
     // df64 and FP64 take all right-hand sides in one launch (links and clover
     // counted once for df64); FP32 launches once per right-hand side
     const double site_bytes = c.prec == PDF ? hop_site_bytes(c.mode, c.prec, c.nrhs)
@@ -1111,24 +1105,20 @@ void hop(const Exec &e, const HopCall &c)
     if (hop_split(e, c)) return;
     if (c.prec == P64) return hop_f64(e, c);
     switch (c.mode) {
-        LQ_CASE(HOP_K1)
-        LQ_CASE(HOP_K2)
-        LQ_CASE(HOP_RICH)
-        LQ_CASE(HOP_FULL)
-        LQ_CASE(HOP_PREP)
-        LQ_CASE(HOP_RECON)
-    case HOP_RES:   // FP64 and df64 only (the solve's full residual)
-        if (c.prec == PDF) launch_hop<df64, HOP_RES>(e, c);
-        break;
-    case HOP_RECON_RES:
-        if (c.prec == PDF) launch_hop<df64, HOP_RECON_RES>(e, c);
-        break;
+    case HOP_K1: launch_mode<HOP_K1>(e, c); break;
+    case HOP_K2: launch_mode<HOP_K2>(e, c); break;
+    case HOP_RICH: launch_mode<HOP_RICH>(e, c); break;
+    case HOP_FULL: launch_mode<HOP_FULL>(e, c); break;
+    case HOP_PREP: launch_mode<HOP_PREP>(e, c); break;
+    case HOP_RECON: launch_mode<HOP_RECON>(e, c); break;
+    case HOP_RES: launch_mode<HOP_RES>(e, c); break;
+    case HOP_RECON_RES: launch_mode<HOP_RECON_RES>(e, c); break;
     }
-#undef LQ_CASE
 }
 
 void clover_mul(const Exec &e, int prec, const void *clov, const void *in, void *out, int nfields)
 {
+    if (prec == P16) throw Refused{"no clover multiply of BF16 fields"};
     Launch L_(e, K_HOP_OTHER,
               (double)e.g.Vh * (prec != P32 ? nfields * 192.0 * 2 + 576.0 : nfields * 96.0 * 2 + 288.0),
               (double)e.g.Vh * nfields * 552);

@@ -346,33 +346,30 @@ bool hop_split_takes(const Geom &g, int prec, int nrhs)
     return g.Vh * nrhs <= most;
 }
 
+template <int M>
+static void split_mode(const Exec &e, const HopCall &c)
+{
+    if (c.prec == P64) return launch_split<double, M, double2, double2, double2>(e, c);
+    if (c.prec == PDF) return launch_split<df64, M, df2, df2, df2>(e, c);
+    if constexpr (hop_form(M, P32))
+        if (c.prec == P32) return launch_split<float, M, float4, float4, float4>(e, c);
+    if constexpr (hop_form(M, P16))
+        if (c.prec == P16) return launch_split<float, M, BfS4, BfL2, float4>(e, c);
+}
+
 bool hop_split(const Exec &e, const HopCall &c)
 {
     if (!hop_split_takes(e.g, c.prec, c.nrhs)) return false;
-#define LQ_CASE(M)                                                                              \
-    case M:                                                                                     \
-        if (c.prec == P64) launch_split<double, M, double2, double2, double2>(e, c);            \
-        else if (c.prec == P32) launch_split<float, M, float4, float4, float4>(e, c);           \
-        else if (c.prec == P16) launch_split<float, M, BfS4, BfL2, float4>(e, c);               \
-        else launch_split<df64, M, df2, df2, df2>(e, c);                                        \
-        break;
     switch (c.mode) {
-        LQ_CASE(HOP_K1)
-        LQ_CASE(HOP_K2)
-        LQ_CASE(HOP_RICH)
-        LQ_CASE(HOP_FULL)
-        LQ_CASE(HOP_PREP)
-        LQ_CASE(HOP_RECON)
-    case HOP_RES:
-        if (c.prec == P64) launch_split<double, HOP_RES, double2, double2, double2>(e, c);
-        else launch_split<df64, HOP_RES, df2, df2, df2>(e, c);
-        break;
-    case HOP_RECON_RES:
-        if (c.prec == P64) launch_split<double, HOP_RECON_RES, double2, double2, double2>(e, c);
-        else launch_split<df64, HOP_RECON_RES, df2, df2, df2>(e, c);
-        break;
+    case HOP_K1: split_mode<HOP_K1>(e, c); break;
+    case HOP_K2: split_mode<HOP_K2>(e, c); break;
+    case HOP_RICH: split_mode<HOP_RICH>(e, c); break;
+    case HOP_FULL: split_mode<HOP_FULL>(e, c); break;
+    case HOP_PREP: split_mode<HOP_PREP>(e, c); break;
+    case HOP_RECON: split_mode<HOP_RECON>(e, c); break;
+    case HOP_RES: split_mode<HOP_RES>(e, c); break;
+    case HOP_RECON_RES: split_mode<HOP_RECON_RES>(e, c); break;
     }
-#undef LQ_CASE
     return true;
 }
 

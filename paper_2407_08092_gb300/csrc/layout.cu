@@ -247,6 +247,11 @@ static void export_t(const Exec &e, const void *f0, const void *f1, void *nat)
     export_tile_kernel<PR, FULL><<<nblk(n, TS), TT, 0, e.st>>>(e.g, (const T *)f0, (const T *)f1, (double2 *)nat);
 }
 
+static void no_bf16(int prec)
+{
+    if (prec == P16) throw Refused{"no such layout pass for BF16 fields"};
+}
+
 void import_half(const Exec &e, int prec, const void *nat, void *f, bool g5)
 {
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + (prec == P32 ? 96 : prec == P16 ? 48 : 192)));
@@ -258,6 +263,7 @@ void import_half(const Exec &e, int prec, const void *nat, void *f, bool g5)
 
 void export_half(const Exec &e, int prec, const void *f, void *nat)
 {
+    no_bf16(prec);
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (192 + (prec == P32 ? 96 : 192)));
     if (prec == PDF) export_t<PDF, false>(e, f, nullptr, nat);
     else if (prec == P64) export_t<P64, false>(e, f, nullptr, nat);
@@ -266,6 +272,7 @@ void export_half(const Exec &e, int prec, const void *f, void *nat)
 
 void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo)
 {
+    no_bf16(prec);
     Launch L_(e, K_LAYOUT, (double)e.g.V * (192 + (prec == P32 ? 96 : 192)));
     if (prec == PDF) import_t<PDF, true>(e, nat, fe, fo);
     else if (prec == P64) import_t<P64, true>(e, nat, fe, fo);
@@ -274,6 +281,7 @@ void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo)
 
 void export_full(const Exec &e, int prec, const void *fe, const void *fo, void *nat)
 {
+    no_bf16(prec);
     Launch L_(e, K_LAYOUT, (double)e.g.V * (192 + (prec == P32 ? 96 : 192)));
     if (prec == PDF) export_t<PDF, true>(e, fe, fo, nat);
     else if (prec == P64) export_t<P64, true>(e, fe, fo, nat);
@@ -348,6 +356,8 @@ __global__ void df2f_kernel(Geom g, const df2 *__restrict__ in, float4 *out)
 
 void convert(const Exec &e, int from, const void *in, int to, void *out, int nfields)
 {
+    if (nfields != 1 && !((from == P32 && to == PDF) || (from == PDF && to == P32)))
+        throw Refused{"several fields are converted between FP32 and df64 alone"};
     if (from == P16 || to == P16) {
         bf16_convert(e, from, in, to, out);
         return;
@@ -407,6 +417,7 @@ __global__ void gamma5_df_kernel(Geom g, const float4 *in, float4 *out)
 
 void gamma5(const Exec &e, int prec, const void *in, void *out)
 {
+    no_bf16(prec);
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (in == out ? 1 : 2) * (prec == P32 ? 96 : 192));
     if (prec == PDF) {
         gamma5_df_kernel<<<nblk(e.g.Vh, 256), 256, 0, e.st>>>(e.g, (const float4 *)in, (float4 *)out);

@@ -98,6 +98,12 @@ inline void launch_after(const Exec &e, bool after, void (*kernel)(P...), dim3 g
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// Thrown by a launcher, before anything is launched, for a form that it does not
+// have; the C entry points answer it with LQ_ERR_ARG.
+struct Refused {
+    const char *why;
+};
+
 // Bytes of one internal per-parity spinor field in a precision.
 inline size_t spinor_bytes(const Geom &g, int prec)
 {
@@ -119,14 +125,15 @@ void bf16_axpby(const Exec &e, double ar, double ai, const void *x, double br, d
 // natural half spinor [Vh][12] c128 <-> internal field of one parity
 // (g5: with spins 2 and 3 negated)
 void import_half(const Exec &e, int prec, const void *nat, void *f, bool g5 = false);
+// (export_half, import_full and export_full: FP64, FP32 or df64)
 void export_half(const Exec &e, int prec, const void *f, void *nat);
 // natural full spinor [V][12] c128 <-> internal even and odd fields
 void import_full(const Exec &e, int prec, const void *nat, void *fe, void *fo);
 void export_full(const Exec &e, int prec, const void *fe, const void *fo, void *nat);
 // the rows of one parity of a natural full field from an FP32 field (dslash.cu)
 void export_parity(const Exec &e, const void *f, int parity, void *nat);
-// precision conversion between internal fields (nfields consecutive ones between
-// FP32 and df64)
+// precision conversion between internal fields (several consecutive ones only
+// between FP32 and df64)
 void convert(const Exec &e, int from, const void *in, int to, void *out, int nfields = 1);
 // out = g5 in (negates spins 2 and 3), FP64, FP32 or df64; in == out allowed
 void gamma5(const Exec &e, int prec, const void *in, void *out);
@@ -212,9 +219,9 @@ struct HopCall {
     void *out2 = nullptr;          // HOP_RECON_RES: the output parity's residual
     double omega;          // HOP_RICH weight
     int nrhs = 1;          // right-hand sides: in, in2, b, out are nrhs consecutive fields
-    // natural output (HOP_K2; always for HOP_FULL, for HOP_RECON with in32 and in
-    // BF16, which offers HOP_K1, HOP_K2 and HOP_RICH; one right-hand side): complex-double rows in the place of `out`, those of
-    // a full lattice or of one parity, spins 2 and 3 negated on request
+    // natural output (HOP_K2, HOP_FULL and HOP_RECON with in32; one right-hand side):
+    // complex-double rows in the place of `out`, those of a full lattice or of one
+    // parity, spins 2 and 3 negated on request
     void *nat = nullptr;
     bool nat_full = false, nat_g5 = false;
     // df64 beyond hop_split's sizes, one right-hand side: HOP_PREP writes an FP32
@@ -222,12 +229,35 @@ struct HopCall {
     bool in32 = false, out32 = false;
     bool after = true;     // launch_after: not behind a kernel that made links or clover blocks of this call
 };
-void hop(const Exec &e, const HopCall &c);
+// The modes that a precision has: FP32 and BF16 apply the operator and the Richardson
+// sweep, preparation, reconstruction and residuals run in FP64 or df64.
+constexpr bool hop_form(int mode, int prec)
+{
+    if (mode < HOP_K1 || mode > HOP_RECON_RES) return false;
+    if (prec == P64 || prec == PDF) return true;
+    if (prec == P32) return mode <= HOP_FULL;
+    return prec == P16 && mode <= HOP_RICH;
+}
+bool hop_split_takes(const Geom &g, int prec, int nrhs);
+// What is wrong with a call, or nullptr.  HOP_FULL and the BF16 HOP_K2 have natural
+// output alone.
+inline const char *hop_refused(const Geom &g, const HopCall &c)
+{
+    if (!hop_form(c.mode, c.prec)) return "no hop of this mode in this precision";
+    const bool df = c.prec == PDF && c.nrhs == 1 && !hop_split_takes(g, PDF, 1);
+    if (c.in32 && !(df && c.mode == HOP_RECON && c.nat)) return "FP32 input is for the df64 reconstruction of larger lattices";
+    if (c.out32 && !(df && c.mode == HOP_PREP)) return "FP32 output is for the df64 preparation of larger lattices";
+    if (c.nat && c.mode != HOP_K2 && c.mode != HOP_FULL && !c.in32) return "no natural output in this mode";
+    if (!c.nat && (c.mode == HOP_FULL || (c.mode == HOP_K2 && c.prec == P16))) return "natural output only in this mode";
+    if (!c.nat && !c.out) return "no output field";
+    if (c.nrhs < 1 || (c.nrhs != 1 && (c.nat || c.prec == P16))) return "one right-hand side only in this form";
+    return nullptr;
+}
+void hop(const Exec &e, const HopCall &c);   // throws Refused
 // the same by the kernels of small lattices (hop_split.cu); false, and nothing
 // done, where the other kernels are the faster ones
 bool hop_split(const Exec &e, const HopCall &c);
 void hop_f64(const Exec &e, const HopCall &c);   // FP64 (hop_f64.cu)
-bool hop_split_takes(const Geom &g, int prec, int nrhs);
 
 // One member lattice of a batched solve over lattices of different sizes: its
 // geometry, FP32 links and clover, and where its right-hand sides' fields sit
