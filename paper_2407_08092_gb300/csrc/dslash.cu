@@ -251,7 +251,7 @@ __device__ __forceinline__ long long warp_site(const Geom &g, int &nvalid)
 {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x, s0 = s - (threadIdx.x & 31);
     nvalid = (int)min(32LL, g.Vh - s0);
-    return min(s, g.Vh - 1);
+    return LQ_IDX(min(s, g.Vh - 1), g.Vh, B_HOP_SITE);
 }
 template <typename R, int MODE, bool NAT>
 __device__ __forceinline__ void hop_site(const Geom &g, const HopArgs<R> &k)
@@ -349,7 +349,7 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     k.clov = (const F4S *)c.clov;
     k.omega = (float)c.omega;
     k.pout = c.pout;
-    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
+    k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
     // Blocks brought in early are not spread as evenly over the SMs, which costs more
     // than the gap between the launches while they are few: D_S 31.4 us overlapped and
@@ -883,7 +883,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS, LQ_DF_MINB) hop_df_kernel(cons
     // blocks stay whole: threads beyond the last site shadow it
     long long s = sb * (long long)kDfSites + threadIdx.x % kDfSites;
     const int nv = (int)min(32LL, g.Vh - (s - (threadIdx.x & 31)));
-    s = min(s, g.Vh - 1);
+    s = LQ_IDX(min(s, g.Vh - 1), g.Vh, B_HOP_SITE);
     const Coords c = cb_coords(g, s, k.pout);
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs;
     hop_df_body<MODE, IO>(g, k, k.in + o, k.in2 ? k.in2 + o : nullptr, k.b ? k.b + o : nullptr, k.out + o,
@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(LQ_HOP_THREADS) export_parity_kernel(Geom g, c
 void export_parity(const Exec &e, const void *f, int parity, void *nat)
 {
     Launch L_(e, K_LAYOUT, (double)e.g.Vh * (96 + 192));
-    const NatOut o = nat_out(nat, true, false);
+    const NatOut o = nat_out(e.g, nat, true, false);
     export_parity_kernel<<<(unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS), LQ_HOP_THREADS,
                            nat_smem(LQ_HOP_THREADS), e.st>>>(e.g, (const float4 *)f, parity, o);
 }
@@ -944,7 +944,7 @@ static void launch_hop(const Exec &e, const HopCall &c)
     k.fs = (long long)St<R>::SPINOR_VECS * e.g.stride;
     constexpr int threads = LQ_HOP_THREADS, sites = std::is_same<R, df64>::value ? kDfSites : threads;   // of a block
     const unsigned blocks = (unsigned)((e.g.Vh + sites - 1) / sites);
-    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
+    k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     if constexpr (std::is_same<R, df64>::value)
     {
         constexpr int sm = kDfVecs * LQ_HOP_THREADS * (int)sizeof(float4);

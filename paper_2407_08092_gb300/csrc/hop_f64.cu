@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(2 * kF64Sites, 8) hop_f64_kernel(const __grid_
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs, st = g.stride;
     const long long s0 = sb * (long long)kF64Sites;
     const int nv = (int)min((long long)kF64Sites, g.Vh - s0);
-    const long long s = s0 + min(lane, nv - 1);   // lanes beyond the last site shadow it
+    const long long s = LQ_IDX(s0 + min(lane, nv - 1), g.Vh, B_HOP_SITE);   // lanes beyond the last site shadow it
     const bool on = lane < nv;
     const Coords c = cb_coords(g, s, k.pout);
 
@@ -165,7 +165,7 @@ static void launch_f64(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)St<double>::SPINOR_VECS * e.g.stride;
-    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
+    k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + kF64Sites - 1) / kF64Sites) * (unsigned)c.nrhs;
     // Blocks brought in early are not spread as evenly, which shows when they are
     // most of one wave: D_S on 18x10x14x22 140 us overlapped and 131 not, on 16^4 161

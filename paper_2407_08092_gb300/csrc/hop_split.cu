@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kSplitThreads, std::is_same<R, df64>::value ? 
     const long long o = (blockIdx.x - sb * k.nrhs) * k.fs, st = g.stride;
     const long long s0 = sb * (long long)kSplitSites + lane;
     const bool on = s0 < g.Vh;
-    const long long s = on ? s0 : g.Vh - 1;                // idle lanes shadow the last site, without its stores
+    const long long s = LQ_IDX(on ? s0 : g.Vh - 1, g.Vh, B_HOP_SITE);   // idle lanes shadow the last site, without its stores
     constexpr bool CLOVER = MODE != HOP_PREP, SITE = MODE != HOP_K1;
     constexpr bool RECON = MODE == HOP_RECON || MODE == HOP_RECON_RES;
     const int blk = w >= 6 ? 1 : 0, row = w - 6 * blk;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kSplitThreads, std::is_same<R, df64>::value ? 
         const long long q = sb * (long long)kSplitSites + r;
         if (q < g.Vh) {
             const long long row = k.nat.full ? 2 * q + (cb_coords(g, q, k.pout).x & 1) : q;
-            k.nat.p[row * 12 + c] = tile[r * 13 + c];
+            k.nat.p[LQ_IDX(row, k.nat.rows, B_NAT) * 12 + c] = tile[r * 13 + c];
         }
     } else if (on) {
         st_comp(k.out + o, st, s, w, v);
@@ -331,7 +331,7 @@ static void launch_split(const Exec &e, const HopCall &c)
     k.pout = c.pout;
     k.nrhs = c.nrhs;
     k.fs = (long long)(spinor_bytes(e.g, c.prec) / sizeof(SV));
-    k.nat = nat_out(c.nat, c.nat_full, c.nat_g5);
+    k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + kSplitSites - 1) / kSplitSites) * (unsigned)c.nrhs;
     launch_after(e, c.after, hop_split_kernel<R, MODE, SV, LV, CV>, blocks, kSplitThreads, 60 * kSplitSites * sizeof(cx<R>), e.g, k);
 }

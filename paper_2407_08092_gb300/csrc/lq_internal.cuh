@@ -53,7 +53,8 @@ enum BoundsSite : unsigned {
     B_SAP_LOCAL,      // block-local (shared-memory) index of the SAP kernel
     B_SAP_GLOBAL,     // lattice index of the SAP kernel
     B_LEX,            // lexicographic site of the clover and force kernels
-    B_LAYOUT          // natural / internal index of the layout kernels
+    B_LAYOUT,         // natural / internal index of the layout kernels
+    B_NAT             // row of a natural field that a hopping kernel writes
 };
 #ifdef LQ_BOUNDS
 static __device__ unsigned int lq_bounds_count_tu;

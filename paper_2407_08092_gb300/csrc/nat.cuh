@@ -13,13 +13,15 @@ struct NatOut {
     double2 *p = nullptr;   // natural field, 12 complex numbers a row
     int full = 0;           // rows are the lattice's sites (else the sites of one parity)
     unsigned flip = 0;      // sign bit of spins 2 and 3 (gamma_5)
+    long long rows = 0;     // rows of the field
 };
 
-static inline NatOut nat_out(void *p, bool full, bool g5)
+static inline NatOut nat_out(const Geom &g, void *p, bool full, bool g5)
 {
     NatOut o;
     o.p = (double2 *)p;
     o.full = full;
+    o.rows = full ? g.V : g.Vh;
     o.flip = g5 ? 0x80000000u : 0u;
     return o;
 }
@@ -59,7 +61,7 @@ __device__ __forceinline__ void nat_write6(const NatOut &o, const double2 *tile,
         const int e = i * 32 + lane, r = e / 6, k = e - 6 * r;
         const int b = __shfl_sync(0xffffffffu, xbit, r);
         const long long row = o.full ? 2 * (s0 + r) + b : s0 + r;
-        if (r < n) o.p[row * 12 + 6 * half + k] = tile[at(r, k)];
+        if (r < n) o.p[LQ_IDX(row, o.rows, B_NAT) * 12 + 6 * half + k] = tile[at(r, k)];
     }
 }
 
