@@ -44,6 +44,12 @@ static constexpr int RED_SLOTS = 2 * MAX_RESTART + 8;
 // 24^3 x 48 10.18 / 10.43, 32^4 (2^19 sites) 15.89 / 16.07.
 static constexpr long long kAheadSites = 1LL << 19;
 
+// Scratch of the force's plaquette matrices (5184 B a site): as many time slices as
+// fit, at least three.  lq_force on 24^3 x 48 takes 5.24 ms with 512 MiB, 5.00 with 1 GiB,
+// 4.93 with 2 GiB; on 48^3 x 96 81.2 ms with three slices (1.7 GB), 78.1 with 8 GiB.
+static constexpr size_t kForceScratch = (size_t)2 << 30;
+static const char *const kForceWs = "force:M";
+
 struct lq_ctx {
     Geom g;
     lq_lattice lat;
@@ -81,6 +87,8 @@ struct lq_ctx {
     int sapbm_b[4] = {0, 0, 0, 0};    // block extents of the block-major SAP copies (0: none for this gauge)
     int4 *sap_origin[2] = {nullptr, nullptr};
     int sap_count[2] = {0, 0};
+    int force_slots = -1;             // time slices of the force's scratch (-1: not chosen yet)
+    long long force_limit = -1, refuse = -1;   // force_scratch_limit
     Exec ex() { return Exec{g, st, &ctr, &prof}; }
 };
 
@@ -126,10 +134,40 @@ void ck(lq_ctx *c, cudaError_t e, const char *what)
 
 void ck_launch(lq_ctx *c, const char *what) { ck(c, cudaGetLastError(), what); }
 
+// the next smaller choice of the force's scratch, in time slices (0: none)
+int fewer_force_slots(const lq_ctx *c, int n) { return n > 6 ? n / 2 : n > 3 && c->g.L[3] > 3 ? 3 : 0; }
+
+// Gives back the force's scratch, whose next call takes less: true if there was one.
+bool release_force_scratch(lq_ctx *c)
+{
+    auto it = c->ws.find(kForceWs);
+    if (it == c->ws.end()) return false;
+    cudaFree(it->second.first);
+    for (auto &p : c->owned)
+        if (p == it->second.first) p = nullptr;
+    c->ws.erase(it);
+    c->force_slots = fewer_force_slots(c, c->force_slots);
+    return true;
+}
+
+// cudaMalloc, a second time without the force's scratch when memory is short
+cudaError_t device_malloc(lq_ctx *c, void **p, size_t bytes)
+{
+    auto get = [&] {
+        return c->refuse >= 0 && bytes > (size_t)c->refuse ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    };
+    cudaError_t r = get();
+    if (r == cudaErrorMemoryAllocation && release_force_scratch(c)) {
+        cudaGetLastError();
+        r = get();
+    }
+    return r;
+}
+
 void *dev_alloc(lq_ctx *c, size_t bytes)
 {
     void *p = nullptr;
-    ck(c, cudaMalloc(&p, bytes), "cudaMalloc");
+    ck(c, device_malloc(c, &p, bytes), "cudaMalloc");
     // zero-fill: the BLAS kernels sweep whole fields and rely on the padding
     // sites (cb >= V/2), which no kernel writes, staying zero
     ck(c, cudaMemsetAsync(p, 0, bytes, c->st), "cudaMemsetAsync");
@@ -941,7 +979,12 @@ void *galloc(lq_group *G, size_t bytes)
 {
     lq_ctx *c = gctx(G);
     void *p = nullptr;
-    ck(c, cudaMalloc(&p, bytes), "cudaMalloc");
+    cudaError_t r = device_malloc(c, &p, bytes);
+    for (size_t l = 0; r == cudaErrorMemoryAllocation && l < G->mem.size(); l++) {
+        cudaGetLastError();
+        r = device_malloc(G->mem[l], &p, bytes);
+    }
+    ck(c, r, "cudaMalloc");
     G->owned.push_back(p);
     ck(c, cudaMemsetAsync(p, 0, bytes, G->st), "cudaMemsetAsync");
     return p;
@@ -1376,6 +1419,19 @@ static std::vector<unsigned (*)(unsigned *)> &bounds_readers()
     return v;
 }
 void bounds_register(unsigned (*read_clear)(unsigned *first)) { bounds_readers().push_back(read_clear); }
+
+// For the tests of lq_force on small lattices: this context's scratch holds at most
+// `limit` bytes, and its allocations of more than `refuse` bytes fail as they do when
+// memory is short (-1: no limit, none fails).  Returns the slices chosen before.
+int force_scratch_limit(lq_ctx *c, long long limit, long long refuse)
+{
+    const int n = c->force_slots;
+    release_force_scratch(c);
+    c->force_slots = -1;
+    c->force_limit = limit;
+    c->refuse = refuse;
+    return n;
+}
 }  // namespace lq
 
 extern "C" {
@@ -2093,6 +2149,30 @@ lq_status lq_export_clover(lq_ctx *c, int which, void *out)
     });
 }
 
+// The scratch of the force's plaquette matrices: all time slices, as many as fit the
+// limit, or, when memory is short, fewer and in the end none.  What could be had is
+// kept, so that later calls neither allocate nor try again.
+static void *force_scratch(lq_ctx *c)
+{
+    const int Lt = c->g.L[3];
+    const size_t slice = force_scratch_bytes(c->g, 1);
+    if (c->force_slots < 0) {
+        const size_t limit = c->force_limit >= 0 ? (size_t)c->force_limit : std::max(kForceScratch, 3 * slice);
+        const int n = (int)std::min<size_t>(limit / slice, Lt);
+        c->force_slots = n == Lt || n >= 3 ? n : 0;
+    }
+    while (c->force_slots > 0) {
+        const size_t bytes = c->force_slots * slice;
+        try {
+            return ws(c, kForceWs, bytes);
+        } catch (const Fail &f) {
+            if (f.s != LQ_ERR_OOM) throw;
+            c->force_slots = fewer_force_slots(c, c->force_slots);
+        }
+    }
+    return nullptr;
+}
+
 // G = coef grad_U Re(Y^+ D X) for natural full spinors X, Y (df64 throughout)
 static void force_apply(lq_ctx *c, const void *X, const void *Y, double coef, void *G)
 {
@@ -2105,19 +2185,8 @@ static void force_apply(lq_ctx *c, const void *X, const void *Y, double coef, vo
     const void *U[2] = {c->Udf[0], c->Udf[1]};
     void *gam = ws(c, "clover:F", (size_t)6 * 9 * 8 * c->g.V);
     force_insertion(e, Xs, Ys, c->lat.csw, gam);
-    // scratch for as many time slices as fit 2 GiB, fewer when memory is short
-    int slices = c->g.L[3];
-    while (slices > 1 && force_scratch_bytes(c->g, slices) > ((size_t)2 << 30)) slices--;
-    void *scratch = nullptr;
-    while (!scratch) {
-        try {
-            scratch = ws(c, "force:M", force_scratch_bytes(c->g, slices));
-        } catch (const Fail &f) {
-            if (f.s != LQ_ERR_OOM || slices == 1) throw;
-            slices /= 2;
-        }
-    }
-    force_links(e, U, Xs, Ys, gam, scratch, slices, coef, G);
+    void *scratch = force_scratch(c);
+    force_links(e, U, Xs, Ys, gam, scratch, c->force_slots, coef, G);
     ck_launch(c, "force");
 }
 

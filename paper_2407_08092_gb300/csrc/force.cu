@@ -38,16 +38,18 @@
 // 96 per site, where the 24 leaves of each link, formed one by one, take 288.
 //
 // Arithmetic is df64 (FP64-accurate on the FP32 units) throughout.
+#include <type_traits>
+
 #include "leaves.cuh"
 #include "lq_kernels.h"
 
 namespace lq {
 
 // Resident blocks per SM asked of the two kernels.  The link kernel takes three (168
-// registers, 74 KB of staged factors each): lq_force on 24^3 x 48 takes 5.15 ms,
-// 5.20 at two and 5.42 with the factors read where they are used at four (128
-// registers).  The plaquette kernel: four (some spills outside the products), 0.2 ms
-// under three.
+// registers, 74 KB of staged factors each): lq_force on 24^3 x 48 takes 4.93 ms (5.15
+// with the matrices of each range made anew, 0.05 more at two blocks and 0.27 more with
+// the factors read where they are used at four, 128 registers).  The plaquette kernel:
+// four (some spills outside the products), 0.2 ms under three.
 #ifndef LQ_FLINK_MINB
 #define LQ_FLINK_MINB 3
 #endif
@@ -205,73 +207,76 @@ __device__ __forceinline__ cx<df64> antiherm_entry(const float2 *__restrict__ ba
     return {i < k ? re : dl_neg(re), im};
 }
 
-// The plaquette matrices of a range of time slices: [plane][matrix][9][sites] df2
-// with the sites of slice t (x fastest) at ((t - tb) mod Lt) * S3.
+// The plaquette matrices of some time slices, in a ring of `slots` slices:
+// [plane][matrix][9][slot][site of the slice, x fastest] df2.  A slice's slot stands in
+// the place of its time coordinate, with the extent `slots`; `head` is the slot of the
+// first slice of a launch.
 constexpr int F_W = 0, F_W2 = 1, F_Z = 2, F_V = 3, F_EM = 4, F_EN = 5, F_MATS = 6;
 struct LoopMats {
     df2 *m;
-    int tb;          // first stored slice
+    int head, slots;
     long long s3;    // sites of a slice
-    long long n;     // sites stored
+    long long n;     // sites of the ring
     __device__ __forceinline__ df2 *at(int p, int q, long long site) const
     {
         return m + ((long long)(p * F_MATS + q) * 9) * n + site;
     }
-    // the stored index of coordinates c
+    // the slot of the launch's slice tl
+    __device__ __forceinline__ int slot(int tl) const { return head + tl >= slots ? head + tl - slots : head + tl; }
+    // the stored index of coordinates c, c[3] the slot
     __device__ __forceinline__ long long site(const Geom &g, const int c[4]) const
     {
-        const int t = c[3] >= tb ? c[3] - tb : c[3] - tb + g.L[3];
-        return LQ_IDX((long long)t * s3 + c[0] + (long long)g.L[0] * (c[1] + (long long)g.L[1] * c[2]), n, B_LEX);
+        return LQ_IDX(c[3] * s3 + c[0] + (long long)g.L[0] * (c[1] + (long long)g.L[1] * c[2]), n, B_LEX);
     }
 };
 
-// coordinates c moved by +-1 along mu (mu uniform over a block)
-__device__ __forceinline__ void step(const Geom &g, const int c[4], int mu, int s, int o[4])
+// coordinates c moved by +-1 along mu (mu uniform over a block); Lt, the extent of c[3]
+__device__ __forceinline__ void step(const Geom &g, const int c[4], int mu, int s, int o[4], int Lt)
 {
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         int v = c[k];
         if (k == mu) {
             v += s;
-            v = v < 0 ? v + g.L[k] : (v >= g.L[k] ? v - g.L[k] : v);
+            const int L = k == 3 ? Lt : g.L[k];
+            v = v < 0 ? v + L : (v >= L ? v - L : v);
         }
         o[k] = v;
     }
 }
 
-// W, W2, Z, V, E_m and E_n of one plaquette per thread (plane = blockIdx.y).  The
-// eight products share one copy of the product code, their operands picked by
-// the step: links a, b, c, d (0..3) and Gam at z, z+m, z+n (4..6).
-__global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, const df2 *__restrict__ Ue,
-                                                         const df2 *__restrict__ Uo, const float2 *__restrict__ Gam,
-                                                         LoopMats S)
-{
-    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (id >= S.n) return;
-    const int p = blockIdx.y, m = c_pmu[p], n = c_pnu[p];
-    int z[4], zm[4], zn[4];
+// One plaquette of plane p at z: its links a, b, c, d (0..3) and Gam at z, z+m, z+n
+// (4..6), and the eight products that make its matrices, which share one copy of
+// the product code, their operands picked by the step.
+struct Plaquette {
+    const df2 *Uz, *Un;
+    const float2 *Gam;
+    const Geom &g;
+    long long lz, lm, ln;
+    int p, m, n;
+    __device__ __forceinline__ Plaquette(const Geom &geom, const df2 *Ue, const df2 *Uo, const float2 *gam, int plane,
+                                         const int z[4])
+        : Gam(gam), g(geom), p(plane), m(c_pmu[plane]), n(c_pnu[plane])
     {
-        const int tl = (int)(id / S.s3);
-        unsigned r = (unsigned)(id - tl * S.s3);
-        z[0] = (int)(r % (unsigned)g.L[0]);
-        r /= (unsigned)g.L[0];
-        z[1] = (int)(r % (unsigned)g.L[1]);
-        z[2] = (int)(r / (unsigned)g.L[1]);
-        z[3] = S.tb + tl >= g.L[3] ? S.tb + tl - g.L[3] : S.tb + tl;
+        int zm[4], zn[4];
+        step(g, z, m, +1, zm, g.L[3]);
+        step(g, z, n, +1, zn, g.L[3]);
+        lz = lex_of(g, z);
+        lm = lex_of(g, zm);
+        ln = lex_of(g, zn);
+        const bool odd = (z[0] + z[1] + z[2] + z[3]) & 1;
+        Uz = (odd ? Uo : Ue) + (lz >> 1);
+        Un = odd ? Ue : Uo;   // z + m and z + n have the other parity
     }
-    step(g, z, m, +1, zm);
-    step(g, z, n, +1, zn);
-    const long long lz = lex_of(g, z), lm = lex_of(g, zm), ln = lex_of(g, zn);
-    const bool odd = (z[0] + z[1] + z[2] + z[3]) & 1;
-    const df2 *Uz = (odd ? Uo : Ue) + (lz >> 1), *Un = odd ? Ue : Uo;   // z + m and z + n have the other parity
-    auto link = [&](int code) {   // U_m(z), U_n(z+m), U_m(z+n), U_n(z)
+    __device__ __forceinline__ const df2 *link(int code) const   // U_m(z), U_n(z+m), U_m(z+n), U_n(z)
+    {
         const df2 *u = code == 0 || code == 3 ? Uz : Un + ((code == 1 ? lm : ln) >> 1);
         return u + (long long)(code == 0 || code == 2 ? m : n) * 9 * g.stride;
-    };
-    M3<df64> acc;
-#pragma unroll 1
-    for (int j = 0; j < 8; j++) {
-        // a b | d c | b c^+ | d^+ a | Gam_z a, a Gam_{z+m} | Gam_z d, d Gam_{z+n}
+    }
+    // acc = or, for the second product of an E, += product j of
+    // a b | d c | b c^+ | d^+ a | Gam_z a, a Gam_{z+m} | Gam_z d, d Gam_{z+n}
+    __device__ __forceinline__ void product(int j, M3<df64> &acc) const
+    {
         const int lc = (0x34043130 >> (4 * j)) & 15, rc = (0x63500221 >> (4 * j)) & 15;
         const M3<df64> B = rc >= 4 ? load_antiherm(Gam, g.V, rc == 5 ? lm : ln, p) : load_mat(link(rc), g.stride, j == 2);
         if (j != 5 && j != 7)
@@ -293,8 +298,37 @@ __global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, 
             }
             row_fma(acc.a + 3 * i, r, B);
         }
+    }
+};
+
+// W, W2, Z, V, E_m and E_n of one plaquette per thread (plane = blockIdx.y), for
+// the n sites of the slices from t0 on (t0 may be Lt, the first slice again)
+__global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, const df2 *__restrict__ Ue,
+                                                         const df2 *__restrict__ Uo, const float2 *__restrict__ Gam,
+                                                         LoopMats S, int t0, long long n)
+{
+    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (id >= n) return;
+    const int p = blockIdx.y;
+    int z[4];
+    long long site;
+    {
+        const int tl = (int)(id / S.s3);
+        unsigned r = (unsigned)(id - tl * S.s3);
+        z[0] = (int)(r % (unsigned)g.L[0]);
+        r /= (unsigned)g.L[0];
+        z[1] = (int)(r % (unsigned)g.L[1]);
+        z[2] = (int)(r / (unsigned)g.L[1]);
+        z[3] = t0 + tl >= g.L[3] ? t0 + tl - g.L[3] : t0 + tl;
+        site = LQ_IDX(id + (long long)(S.slot(tl) - tl) * S.s3, S.n, B_LEX);
+    }
+    const Plaquette P(g, Ue, Uo, Gam, p, z);
+    M3<df64> acc;
+#pragma unroll 1
+    for (int j = 0; j < 8; j++) {
+        P.product(j, acc);
         if (j == 4 || j == 6) continue;
-        df2 *o = S.at(p, j < 4 ? j : j == 5 ? F_EM : F_EN, id);
+        df2 *o = S.at(p, j < 4 ? j : j == 5 ? F_EM : F_EN, site);
 #pragma unroll
         for (int k = 0; k < 9; k++) o[(long long)k * S.n] = cx_df2(acc.a[k]);
     }
@@ -302,8 +336,13 @@ __global__ void __launch_bounds__(128, LQ_FLOOP_MINB) force_loop_kernel(Geom g, 
 
 // G(x, mu) for one (site, direction) per thread, sites of the slices t0 ..
 // (mu = blockIdx.y): the hopping term's outer products, then per plane that
-// contains mu the link's two plaquettes, two products each.
-__global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, const df2 *__restrict__ Xe,
+// contains mu the link's two plaquettes, two products each.  FORM: without stored
+// matrices, each formed where it is used: 192 products a site in the place of 96, the
+// same values, 11.7 ms on 24^3 x 48 (4.93 with them).  It runs when no scratch can be had.
+template <bool FORM>
+__global__ void __launch_bounds__(128, FORM ? 2 : LQ_FLINK_MINB) force_link_kernel(Geom g, const df2 *__restrict__ Ue,
+                                                         const df2 *__restrict__ Uo, const float2 *__restrict__ Gam,
+                                                         const df2 *__restrict__ Xe,
                                                          const df2 *__restrict__ Xo, const df2 *__restrict__ Ye,
                                                          const df2 *__restrict__ Yo, LoopMats S, int t0, long long ns,
                                                          double coef, double2 *G)
@@ -316,7 +355,7 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
     lex_coords(g, lex, c);
     const int parity = (c[0] + c[1] + c[2] + c[3]) & 1;
     int cn[4];
-    step(g, c, mu, +1, cn);
+    step(g, c, mu, +1, cn, g.L[3]);
     const long long cb = lex >> 1, cbn = lex_of(g, cn) >> 1;
     const df2 *Xx = parity ? Xo : Xe, *Yx = parity ? Yo : Ye;      // at x
     const df2 *Xn = parity ? Xe : Xo, *Yn = parity ? Ye : Yo;      // at x + mu
@@ -342,13 +381,41 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
     extern __shared__ float4 force_stage[];
     float4 *stage = force_stage + threadIdx.x;
     auto entry = [&](int h, int e) { return stage + ((h & 1) * 18 + e) * 128; };   // left factor 0..8, right 9..17
+    // the factors of product h into their entries, the left one first
+    auto form_product = [&](int h) {
+        const Product r = product(h);
+        const int q = h >> 2, nu = q < mu ? q : q + 1;
+        const int p = c_plane[r.lower ? mu * 4 + nu : nu * 4 + mu];
+        int z[4], zu[4];
+        step(g, c, nu, r.down ? -1 : 0, z, g.L[3]);
+        step(g, z, mu, +1, zu, g.L[3]);
+        const int other = r.down ? (r.efirst ? (r.lower ? F_W : F_W2) : F_V) : (r.efirst ? F_Z : (r.lower ? F_W2 : F_W));
+#pragma unroll 1
+        for (int f = 0; f < 2; f++) {
+            const bool is_e = (f == 0) == r.efirst;
+            int y[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) y[k] = is_e && !r.efirst ? zu[k] : z[k];
+            const Plaquette P(g, Ue, Uo, Gam, p, y);
+            const int j0 = is_e ? (r.lower ? 6 : 4) : other, j1 = is_e ? j0 + 2 : j0 + 1;
+            M3<df64> t;
+#pragma unroll 1
+            for (int j = j0; j < j1; j++) P.product(j, t);
+#pragma unroll
+            for (int e = 0; e < 9; e++) {
+                const df2 v = cx_df2(t.a[e]);
+                *entry(h, 9 * f + e) = make_float4(v.rh, v.ih, v.rl, v.il);
+            }
+        }
+    };
+    const int cs[4] = {c[0], c[1], c[2], S.slot(c[3] - t0)};
     auto copy_product = [&](int h) {
         const Product r = product(h);
         const int q = h >> 2, nu = q < mu ? q : q + 1;
         const int p = c_plane[r.lower ? mu * 4 + nu : nu * 4 + mu];
         int z[4], zu[4];
-        step(g, c, nu, r.down ? -1 : 0, z);
-        step(g, z, mu, +1, zu);
+        step(g, cs, nu, r.down ? -1 : 0, z, S.slots);
+        step(g, z, mu, +1, zu, S.slots);
         const long long iz = S.site(g, z), iu = S.site(g, zu);
         const int other = r.down ? (r.efirst ? (r.lower ? F_W : F_W2) : F_V) : (r.efirst ? F_Z : (r.lower ? F_W2 : F_W));
         const df2 *E = S.at(p, r.lower ? F_EN : F_EM, r.efirst ? iz : iu), *O = S.at(p, other, iz);
@@ -360,7 +427,7 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
         }
         copy_commit();
     };
-    copy_product(0);
+    if (!FORM) copy_product(0);
 
     M3<df64> acc;
 #pragma unroll
@@ -411,7 +478,9 @@ __global__ void __launch_bounds__(128, LQ_FLINK_MINB) force_link_kernel(Geom g, 
     // ---- clover term: the two plaquettes of each plane (mu, nu) that hold U_mu(x) ----
 #pragma unroll 1
     for (int h = 0; h < 12; h++) {
-        if (h < 11) {
+        if (FORM) {
+            form_product(h);
+        } else if (h < 11) {
             copy_product(h + 1);
             copy_wait<1>();
         } else {
@@ -474,46 +543,63 @@ void force_insertion(const Exec &e, const void *X[2], const void *Y[2], double c
         (float2 *)Gam);
 }
 
-// The plaquette matrices take 5184 B a site, so the lattice goes through in
-// ranges of time slices whose matrices (with one more slice on either side) fit
-// the scratch: bytes of scratch for `slices` slices of output.
-size_t force_scratch_bytes(const Geom &g, int slices)
+// The plaquette matrices take 5184 B a site, so the lattice goes through in ranges
+// of time slices: the matrices of a range and of the slice on either side stand in
+// a ring of slices, in which the next range finds the two that it shares with this
+// one: 7.6 ns a site on 48^3 x 96 in ranges of one slice, 14.0 with the neighbours made
+// anew for each, 7.4 on 24^3 x 48 in ranges of 27.  Bytes of a ring of `slots` slices.
+size_t force_scratch_bytes(const Geom &g, int slots)
 {
-    const long long s3 = g.V / g.L[3];
-    const int stored = slices + 2 < g.L[3] ? slices + 2 : g.L[3];
-    return (size_t)stored * s3 * 6 * F_MATS * 9 * sizeof(df2);
+    return (size_t)slots * (g.V / g.L[3]) * 6 * F_MATS * 9 * sizeof(df2);
 }
 
+// slots: Lt (every slice at once), from 3 to Lt - 1 (ranges of slots - 2 slices), or
+// 0 (no scratch)
 void force_links(const Exec &e, const void *Udf[2], const void *X[2], const void *Y[2], const void *Gam, void *scratch,
-                 int slices, double coef, void *G)
+                 int slots, double coef, void *G)
 {
     const Geom &g = e.g;
+    const int Lt = g.L[3];
+    const df2 *Ue = (const df2 *)Udf[0], *Uo = (const df2 *)Udf[1];
     LoopMats S;
     S.m = (df2 *)scratch;
-    S.s3 = g.V / g.L[3];
-    const bool whole = slices + 2 >= g.L[3];
-    if (whole) slices = g.L[3];
-    for (int t0 = 0; t0 < g.L[3]; t0 += slices) {
-        const int nt = g.L[3] - t0 < slices ? g.L[3] - t0 : slices;
-        const int stored = whole ? g.L[3] : nt + 2;
-        S.tb = whole ? 0 : (t0 + g.L[3] - 1) % g.L[3];
-        S.n = stored * S.s3;
+    S.s3 = g.V / Lt;
+    S.slots = slots;
+    S.n = slots * S.s3;
+    S.head = 0;
+    const int range = slots == 0 || slots == Lt ? Lt : slots - 2;
+    auto links = [&](auto form, int t0, int nt) {
+        constexpr bool FORM = decltype(form)::value;
         const long long ns = nt * S.s3;
+        // X and Y, the matrices, the 4 gradients (c128); per link 12 products and
+        // the hopping term's 2 x 4 x 9 outer-product entries
+        Launch L_(e, K_FORCE, (double)ns * (2 * 192 + (FORM ? 4 * 144 + 6 * 72 : 36 * 144) + 4 * 144),
+                  (double)ns * 4 * ((FORM ? 48 : 12) * (198 + 18) + 2 * 4 * (9 * 8 + 12)));
+        constexpr int sm = 2 * 18 * 128 * (int)sizeof(float4);
+        cudaFuncSetAttribute(force_link_kernel<FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        force_link_kernel<FORM><<<dim3(blocks_of(ns, 128), 4), 128, sm, e.st>>>(
+            g, Ue, Uo, (const float2 *)Gam, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1],
+            S, t0, ns, coef, (double2 *)G);
+    };
+    if (slots == 0) return links(std::true_type(), 0, Lt);
+    for (int t0 = 0; t0 < Lt; t0 += range) {
+        const int nt = Lt - t0 < range ? Lt - t0 : range;
+        int from = 0, count = Lt;   // the slices to make
+        if (slots != Lt) {          // t0 - 1 .. t0 + nt, of which the first two are there from the second range on;
+                                    // slice t has the slot (t + 1) mod slots
+            from = t0 ? t0 + 1 : Lt - 1;
+            count = t0 ? nt : nt + 2;
+            S.head = t0 ? (t0 + 2) % slots : 0;
+        }
         {
             // unique bytes per site: 4 df64 links and six Gam in, 36 matrices out; per
             // plane eight 3x3 products of 198 flops
-            Launch L_(e, K_FORCE, (double)S.n * (4 * 144 + 6 * 72 + 36 * 144), (double)S.n * 6 * 8 * 198);
-            force_loop_kernel<<<dim3(blocks_of(S.n, 128), 6), 128, 0, e.st>>>(
-                g, (const df2 *)Udf[0], (const df2 *)Udf[1], (const float2 *)Gam, S);
+            const long long n = count * S.s3;
+            Launch L_(e, K_FORCE, (double)n * (4 * 144 + 6 * 72 + 36 * 144), (double)n * 6 * 8 * 198);
+            force_loop_kernel<<<dim3(blocks_of(n, 128), 6), 128, 0, e.st>>>(g, Ue, Uo, (const float2 *)Gam, S, from, n);
         }
-        // X and Y, the matrices, the 4 gradients (c128); per link 12 products and
-        // the hopping term's 2 x 4 x 9 outer-product entries
-        Launch L_(e, K_FORCE, (double)ns * (2 * 192 + 36 * 144 + 4 * 144),
-                  (double)ns * 4 * (12 * (198 + 18) + 2 * 4 * (9 * 8 + 12)));
-        constexpr int sm = 2 * 18 * 128 * (int)sizeof(float4);
-        cudaFuncSetAttribute(force_link_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        force_link_kernel<<<dim3(blocks_of(ns, 128), 4), 128, sm, e.st>>>(
-            g, (const df2 *)X[0], (const df2 *)X[1], (const df2 *)Y[0], (const df2 *)Y[1], S, t0, ns, coef, (double2 *)G);
+        if (slots != Lt) S.head = (t0 + 1) % slots;
+        links(std::false_type(), t0, nt);
     }
 }
 

@@ -183,10 +183,11 @@ void sap_block_major(const Exec &e, const int b[4], int parity, int rows, const 
 // X, Y: internal df64 full fields (even, odd).  Gam: device scratch of
 // 6 * 9 * V * 8 bytes.  G: natural c128 [V][4][3][3], G = coef grad_U Re(Y^+ D X).
 void force_insertion(const Exec &e, const void *X[2], const void *Y[2], double csw, void *Gam);
-// bytes of scratch that force_links takes for `slices` time slices at a time
-size_t force_scratch_bytes(const Geom &g, int slices);
+// bytes of a scratch of `slots` time slices for force_links, which takes all of the
+// lattice's, at least 3, or none
+size_t force_scratch_bytes(const Geom &g, int slots);
 void force_links(const Exec &e, const void *Udf[2], const void *X[2], const void *Y[2], const void *Gam, void *scratch,
-                 int slices, double coef, void *G);
+                 int slots, double coef, void *G);
 // out = g5 in on natural full spinors (in == out allowed)
 void gamma5_nat(const Exec &e, const void *in, void *out);
 
