@@ -40,8 +40,9 @@ static constexpr int RED_SLOTS = 2 * MAX_RESTART + 8;
 // Sites per parity up to which the FP32 GMRES queues the next step's operator
 // before it reads a step's scalars.  The GPU idles some microseconds a step while
 // the host reads them; the product queued ahead of the step that ends a solve is
-// wasted.  Mixed solve with and without: 8^4 1.36 / 1.59 ms, 16^3 x 32 3.12 / 3.36,
-// 24^3 x 48 10.18 / 10.43, 32^4 (2^19 sites) 15.89 / 16.07.
+// wasted.  Mixed solve with and without: 8^4 1.36 / 1.59 ms, 16^3 x 32 2.96 / 3.17,
+// 24^3 x 48 9.93 / 10.07, 32^4 (2^19 sites) 15.59 / 15.63, 32^3 x 48 22.54 / 22.45,
+// 32^3 x 64 29.53 / 29.31.
 static constexpr long long kAheadSites = 1LL << 19;
 
 // Scratch of the force's plaquette matrices (5184 B a site): as many time slices as

@@ -352,8 +352,9 @@ static void launch_hop_bf(const Exec &e, const HopCall &c)
     k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + LQ_HOP_THREADS - 1) / LQ_HOP_THREADS);
     // Blocks brought in early are not spread as evenly over the SMs, which costs more
-    // than the gap between the launches while they are few: D_S 31.4 us overlapped and
-    // 29.0 not on 18x10x14x22, 37.2 and 36.7 on 16^3x32, but 54.9 and 58.7 on 20^3x32.
+    // than the gap between the launches while they are few.  D_S in us, overlapped and
+    // not: 217 blocks 32.2 / 28.9, 288 33.0 / 30.7, 405 35.0 / 33.4, 512 37.2 / 37.1, 625
+    // 39.7 / 42.2, 1000 55.1 / 58.2, 2592 112.5 / 118.
     const bool after = c.after && blocks > 512;
     if constexpr (MODE == HOP_K2)   // always natural (hop_refused)
         launch_after(e, after, hop_kernel_bf_nat, blocks, LQ_HOP_THREADS, nat_smem(LQ_HOP_THREADS), e.g, k);

@@ -14,7 +14,7 @@
 
 namespace lq {
 
-constexpr int kF64Sites = 32;
+constexpr int kF64Sites = 32, kF64Blocks = 8;   // sites of a block, blocks of an SM
 
 struct F64Args {
     const double2 *in, *in2, *b;
@@ -41,7 +41,7 @@ __device__ __forceinline__ void hop_one(const Geom &g, const F64Args &k, const d
 }
 
 template <int MODE, bool NAT>
-__global__ void __launch_bounds__(2 * kF64Sites, 8) hop_f64_kernel(const __grid_constant__ Geom g,
+__global__ void __launch_bounds__(2 * kF64Sites, kF64Blocks) hop_f64_kernel(const __grid_constant__ Geom g,
                                                                const __grid_constant__ F64Args k)
 {
     __shared__ double2 handed[2][6][kF64Sites];
@@ -167,10 +167,12 @@ static void launch_f64(const Exec &e, const HopCall &c)
     k.fs = (long long)St<double>::SPINOR_VECS * e.g.stride;
     k.nat = nat_out(e.g, c.nat, c.nat_full, c.nat_g5);
     const unsigned blocks = (unsigned)((e.g.Vh + kF64Sites - 1) / kF64Sites) * (unsigned)c.nrhs;
-    // Blocks brought in early are not spread as evenly, which shows when they are
-    // most of one wave: D_S on 18x10x14x22 140 us overlapped and 131 not, on 16^4 161
-    // and 158, but 86 and 90 on 16^2x12^2 and 241 and 244 on 16^3x24.
-    const bool after = c.after && (blocks <= 768 || blocks > 1216);
+    // Blocks brought in early are not spread as evenly, which shows when they are most
+    // of one wave, but not nearly all of it.  D_S in us, overlapped and not: 576 blocks
+    // 86.4 / 90.5, 784 139.2 / 129.4, 867 139.7 / 131.0, 1024 160.4 / 158.0, 1152
+    // 167.1 / 170.4, 1280 203.7 / 209.3, 4000 548 / 553.
+    constexpr unsigned wave = kSMs * kF64Blocks;
+    const bool after = c.after && (blocks <= wave * 5 / 8 || blocks > wave * 7 / 8);
     auto launch = [&](auto kernel) { launch_after(e, after, kernel, blocks, 2 * kF64Sites, 0, e.g, k); };
     if constexpr (MODE == HOP_FULL) {   // always natural
         launch(hop_f64_kernel<MODE, true>);

@@ -9,14 +9,13 @@
 //      whose entries it loaded before step 1.
 // The operations are those of the larger lattices' kernels.
 //
-// lq_apply of D_S in us, twelve threads against one and before the launches
-// overlapped (launch_after: df64 at 2048 sites 18.8 -> 14.4), at 2048 sites a
-// parity: df64 18.8 / 39.3, FP32 18.6 / 20.7, FP64 37 / 88, BF16 18.8 / 20.8; at
-// 9216: 29 / 43,
-// 18.7 / 24.8, 63 / 88, 20.8 / 24.9; at 24576: 58 / 56, 31.0 / 29.0, 162 / 132,
-// 32 / 27.  The larger the lattice, the less it needs the extra threads, which
-// pass the eight half spinors through shared memory and idle while others work.
-// df64 takes one block an SM (168 registers; two: 27 us at 2048 sites, not 18.8).
+// lq_apply of D_S in us, twelve threads and the larger lattices' kernels (one thread
+// a site in FP32 and BF16, two in df64 and FP64), at 2048 sites a parity: df64
+// 14.5 / 22.6, FP32 12.3 / 18.4, FP64 34.8 / 47.2, BF16 12.4 / 24.7; at 24576: 53.4 / 40.5,
+// 26.7 / 28.9, 158 / 138, 28.8 / 28.8.  The larger the lattice, the less it needs the
+// extra threads, which pass the eight half spinors through shared memory and idle
+// while others work.
+// df64 takes one block an SM (168 registers; two: 8 us more at 2048 sites).
 #include <type_traits>
 
 #include "bf16.cuh"
@@ -338,11 +337,13 @@ static void launch_split(const Exec &e, const HopCall &c)
 
 bool hop_split_takes(const Geom &g, int prec, int nrhs)
 {
-    // sites up to which twelve threads are the faster (for df64 than two): df64
-    // 23.0 / 24.1 us at 9216, 31.4 / 31.1 at 13824, 39.2 / 35.1 at 16384; FP32
-    // 25.9 / 27.6 at 16384 and 31.0 / 29.0 at 24576; FP64 86 / 88 at 10368 and
-    // 114 / 92 at 16384; BF16 23.8 / 24.9 at 10368 and 26.9 / 24.9 at 13824
-    const long long most = prec == P16 ? 10368 : prec == P32 ? 16384 : 12288;
+    // Sites up to which twelve threads are the faster, in us with twelve and without:
+    // D_S of df64 22.7 / 24.4 at 9216, 30.9 / 30.9 at 12096, 39.1 / 35.0 at 16384; of FP32
+    // 20.6 / 27.0 at 18432, 26.7 / 28.9 at 24576, where Richardson(4) takes 118 / 111; of
+    // BF16 22.6 / 26.8 at 18432, 28.8 / 28.8 at 24576.  FP64: D_S 34.9 / 47.2 at 4096 and
+    // 84.0 / 69.8 at 12096, a GMRES solve 8.6 / 10.3 ms at 10368, 10.4 / 11.5 at 12096,
+    // 14.6 / 14.8 at 24576.
+    const long long most = prec == P32 || prec == P16 ? 20480 : 12288;
     return g.Vh * nrhs <= most;
 }
 

@@ -9,6 +9,8 @@
 
 namespace lq {
 
+constexpr int kSMs = 152;   // of a GB300
+
 // Internal precisions: native FP64, FP32, double-float (df64: FP64-accurate
 // arithmetic on the FP32 units, stored as float pairs in the FP64 layouts), and
 // BF16 storage of spinors and links with FP32 arithmetic and FP32 clover.
