@@ -389,7 +389,7 @@ lq_status lq_norm2_noalloc(const void *v, long long n_sites, double *out, void *
  * counts it, remembers the code of the first one (the enum BoundsSite of the
  * internal header: 1 hop site, 2 hop neighbour, 3 df64 hop neighbour, 4
  * batched-hop neighbour, 5 SAP block-local, 6 SAP lattice, 7 clover/force
- * lexicographic, 8 layout) and uses index 0 instead, so the access stays in
+ * lexicographic, 8 layout, 9 natural row of a hop) and uses index 0 instead, so the access stays in
  * bounds.  This call synchronises the current device, reads and clears those
  * flags and returns LQ_ERR_BOUNDS if any check failed since the last call,
  * else LQ_OK.  *checked = 1 in a checked build, 0 otherwise (where nothing is

@@ -7,7 +7,8 @@ through the C ABI (printing per-class device times), runs `--apps`
 mixed-precision solves (FGMRES(10) in df64 preconditioned by GMRES(8) in
 FP32), a batched solve of `--nrhs` point sources through a one-member group
 (printing the autotuner's choice), SAP(3, 4) smoother calls, the
-fermion-force kernel, or lq_set_gauge (the clover build), e.g.
+fermion-force kernels, Richardson(5) smoother calls in FP32 between df64 ends, or
+lq_set_gauge (the clover build), e.g.
 ``python -m paper_2407_08092_gb300.profile_case --lattice 24,24,24,48 --prec 1 --apps 3``.
 """
 import argparse
@@ -21,10 +22,10 @@ from paper_2407_08092_gb300 import lqdd, synth
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--lattice", default="24,24,24,48")
-    ap.add_argument("--prec", type=int, default=1, help="0 FP64, 1 FP32, 2 df64")
+    ap.add_argument("--prec", type=int, default=1, help="0 FP64, 1 FP32, 2 df64, 3 BF16")
     ap.add_argument("--apps", type=int, default=3)
     ap.add_argument("--op", type=int, default=lqdd.LQ_OP_SCHUR)
-    ap.add_argument("--mode", default="apply", choices=["apply", "solve", "batch", "force", "sap", "gauge"])
+    ap.add_argument("--mode", default="apply", choices=["apply", "solve", "batch", "force", "sap", "gauge", "richardson"])
     ap.add_argument("--nrhs", type=int, default=12)
     ap.add_argument("--shape", default=None,
                     help="batch mode: pin the batched hop's launch shape 'sites_per_tile,rhs_per_thread,grid_factor' "
@@ -88,6 +89,15 @@ def main():
                 print(f"{lqdd.lq_kernel_class_name(c):14s} {nl:5d} launches {1e3 * ms / nl:9.2f} us/launch "
                       f"{by / (ms * 1e6):8.1f} GB/s")
         lqdd.lq_profile(ctx, 0)
+        out = float(e.abs().sum())
+    elif a.mode == "richardson":
+        r = torch.from_numpy(synth.gaussian_spinor(V, 2003)).cuda()
+        e = torch.empty_like(r)
+        prm = lqdd.make_params(smoother=lqdd.LQ_SMOOTH_RICHARDSON, smooth_n=5, omega=0.8 / 5.2,
+                               inner_prec=lqdd.LQ_F32, prec=lqdd.LQ_DF64)
+        for _ in range(a.apps):
+            lqdd.lq_smooth(ctx, prm, r, e)
+        torch.cuda.synchronize()
         out = float(e.abs().sum())
     elif a.mode == "gauge":   # lq_set_gauge: layout, clover field, assembly and inverse
         U = torch.from_numpy(synth.gauge_links(L, 0.25, 1003)).cuda()
